@@ -277,7 +277,6 @@ __global__ void k_score(const float* opc, int m, const DevSac* sac, const float*
 // window (int), [23] unused.  With the 9-parameter model the vertex takes
 // [4..12].
 constexpr int kUnitRec = kUnitRecFloats;
-constexpr int kSortBins = 512;           // pulse-end time bins of the per-wave ordering
 
 // The search runs over N coordinates: N = 18, the OPC entries themselves, or
 // N = 9, the 9-parameter model (Sec. 2.2.2, Table 2).  A simplex has N + 1
@@ -322,12 +321,11 @@ __device__ __forceinline__ void u_to_p(const float* u, const float* pc, float ln
   }
 }
 
-// Saved simplex (serving): vertices, values, centroid, order, active, iterations.
+// Saved simplex (serving): vertices, values, order, active, iterations (the
+// centroid and the trial points follow from these).
 template <int N>
-__host__ __device__ constexpr int state_floats() { return verts<N>() * N + verts<N>() + N + verts<N>() + 2; }
+__host__ __device__ constexpr int state_floats() { return verts<N>() * N + 2 * verts<N>() + 2; }
 static_assert(state_floats<kNumParams>() == kSearchStateFloats, "saved simplex layout");
-constexpr int kHistPer = kSortBins / 32;              // bins per lane of the scanning warp
-constexpr int kHistLen = kSortBins + 32;                // bin b stored at b + b / kHistPer
 
 // One block runs G simplices in each of two groups (a unit of 2G simplices of
 // one saccade) with twelve warps, all of which evaluate: a group's wave (its
@@ -345,29 +343,20 @@ constexpr int kSearchWarps = 12;
 constexpr long long kMaxIdleCycles = 8000000000LL;
 template <int G, int N>
 __host__ __device__ constexpr int search_threads() { return 32 * kSearchWarps; }
-// candidates per lane when one warp orders a wave
-template <int G, int N>
-__host__ __device__ constexpr int wave_per_lane() { return (G * trials<N>() + 31) / 32; }
-
 // State of one group of G simplices over N coordinates.
 template <int G, int N>
-struct GroupSmem {
+struct alignas(16) GroupSmem {
   static constexpr int kNV = verts<N>();
   static constexpr int kNT = trials<N>();
+  static_assert(G <= 32, "the deciding warp takes one simplex per lane");
   float U[G][kNV][N];            // vertices, by slot
   float XT[G][4][N];             // reflection, expansion, outside/inside contraction
-  float XB[G][N];                // centroid of the best n vertices
   float F[G][kNV];               // vertex values, by slot
   float FT[G][kNT];              // trial values
-  int hist[kHistLen];            // counting sort of the pending wave by pulse-end time (padded)
-  unsigned short perm[G * kNT];  // candidate ids of the pending wave in key order
-  int kr[G * kNT];               // ordering scratch: key << 16 | rank within the key's bin, or -1
   unsigned char ord[G][kNV + 1]; // ord[r] = slot of rank r
+  unsigned char turn[G];         // turn[k] = k-th simplex of the pending wave
   int active[G];
   int iters[G];
-  int okf[G];   // decision scratch: value spread within tol_f
-  int okx[G];   // decision scratch: vertex spread within tol_x
-  int shr[G];   // decision scratch: the simplex shrinks this step
   int nsim;     // simplices of this group (0: empty group)
   int nvalid;   // candidates of the pending wave
   int kind;     // pending wave: 0 initial vertices, 1 trial points
@@ -376,7 +365,7 @@ struct GroupSmem {
   int evals;    // candidate evaluations of this group
   int pe;       // of those, candidates whose pulse ends inside the window
   int pub;      // published wave: sequence number << 16 | chunks (0 chunks: nothing to take)
-  int claim;    // sequence number << 16 | next chunk of 32 candidates (in key order) to claim
+  int claim;    // sequence number << 16 | next chunk of 32 candidates (in wave order) to claim
   int done;     // chunks of the published wave evaluated
 };
 
@@ -458,20 +447,6 @@ __device__ __forceinline__ float eval_u(const float (&u)[N], const float* pc, fl
   return objective<true, PACK>(p, sc, z, sum0, c0, qs, qstride, pe, mask);
 }
 
-// Sort key of a candidate: its pulse-end time, binned over the window (the
-// last bin holds pulses that outlast the window).  Lanes of a warp then run
-// nearly the same number of pulse-phase and step-phase samples.
-__device__ __forceinline__ int switch_key(float u_pw, float pc_pw, float lnlo, float lnhi, const SacConst& sc) {
-  const int ntot = sc.L - 1 - sc.onset;
-  if (ntot <= 0) return 0;
-  const float w = pc_pw * __expf(fminf(fmaxf(u_pw, lnlo), lnhi));
-  const float tau = fmaxf(w * sc.fs * 1e-3f, 0.0f);       // in samples after onset
-  const float x = tau * ((float)(kSortBins - 1) / (float)ntot);
-  return x >= (float)(kSortBins - 1) ? kSortBins - 1 : (int)x;
-}
-
-__device__ __forceinline__ int hist_slot(int b) { return b + b / kHistPer; }
-
 // Rows of trial point q of simplex gi, as u = a + (b - a) / 2 coordinate by
 // coordinate: a = b = the deciding warp's XT row for q < 4 (so u = a exactly),
 // the best vertex and vertex q - 3 for the shrink points.  One form for every
@@ -481,31 +456,6 @@ __device__ __forceinline__ void trial_rows(const GroupSmem<G, N>& g, int gi, int
   const unsigned char* o = g.ord[gi];
   a = q < 4 ? g.XT[gi][q] : g.U[gi][o[0]];
   b = q < 4 ? g.XT[gi][q] : g.U[gi][o[q - 3]];
-}
-
-// Centroid of the best n vertices and the vertex-spread half of the exit test
-// (Sec. 3.3: every vertex within tol_x of the best in max-norm), spread over
-// the deciding warp's lanes by (simplex, coordinate); `sel` picks the
-// simplices to process.  g.okx[gi] must be 1 on entry and is cleared by any
-// coordinate that fails.
-template <int G, int N, class Sel>
-__device__ __forceinline__ void centroids(GroupSmem<G, N>& g, int lane, float tolx, Sel sel) {
-  for (int p = lane; p < g.nsim * N; p += 32) {
-    const int gi = p / N, j = p - gi * N;
-    if (!sel(gi)) continue;
-    const unsigned char* o = g.ord[gi];
-    float x[verts<N>()];
-#pragma unroll
-    for (int r = 0; r < verts<N>(); ++r) x[r] = g.U[gi][o[r]][j];
-    float acc = 0.0f;
-    bool ok = true;
-#pragma unroll
-    for (int r = 0; r < N; ++r) acc += x[r];
-#pragma unroll
-    for (int r = 1; r < verts<N>(); ++r) ok = ok && (fabsf(x[r] - x[0]) <= tolx);
-    g.XB[gi][j] = acc / (float)N;
-    if (!ok) g.okx[gi] = 0;
-  }
 }
 
 // Stable ranking of 19 values by one thread: rank[r] = #{s : v_s < v_r or
@@ -535,41 +485,42 @@ __device__ __forceinline__ int value_spread_ok(const GroupSmem<G, N>& g, int gi,
   return ok ? 1 : 0;
 }
 
-// Ranking and first centroid of freshly evaluated initial simplices.
+// Ranking of freshly evaluated initial simplices, one lane per simplex.
+// Returns whether the lane's simplex is active; okf: its values agree within
+// tol_f.
 template <int G, int N>
-__device__ __forceinline__ void init_rank(GroupSmem<G, N>& g, int lane, float tolx, float tolf) {
-  for (int gi = lane; gi < g.nsim; gi += 32) {
+__device__ __forceinline__ bool init_rank(GroupSmem<G, N>& g, int lane, float tolf, bool& okf) {
+  const bool live = lane < g.nsim;
+  okf = false;
+  if (live) {
     int sl[verts<N>()];
     float fv[verts<N>()];
 #pragma unroll
     for (int r = 0; r < verts<N>(); ++r) {
       sl[r] = r;
-      fv[r] = g.F[gi][r];
+      fv[r] = g.F[lane][r];
     }
-    rank_simplex<G, N>(g, gi, sl, fv);
-    g.active[gi] = 1;
-    g.iters[gi] = 0;
-    g.okx[gi] = 1;
-    g.okf[gi] = value_spread_ok<G, N>(g, gi, tolf);
+    rank_simplex<G, N>(g, lane, sl, fv);
+    g.active[lane] = 1;
+    g.iters[lane] = 0;
+    okf = value_spread_ok<G, N>(g, lane, tolf) != 0;
   }
   __syncwarp();
-  centroids<G, N>(g, lane, tolx, [](int) { return true; });
-  __syncwarp();
-  for (int gi = lane; gi < g.nsim; gi += 32)
-    if (g.okx[gi] && g.okf[gi]) g.active[gi] = 0;
-  __syncwarp();
+  return live;
 }
 
 // Lagarias decision and re-sort of every active simplex of a group after a
-// trial wave.  One lane per simplex takes the decision (the slots and values
-// of its 19 vertices in registers, in rank order) and applies a replacement;
-// shrinks, centroids and the vertex-spread test are spread over all lanes.
+// trial wave, one lane per simplex (the slots and values of its vertices in
+// registers, in rank order); only a shrink's coordinates, which are rare, are
+// spread over all lanes.  Returns whether the lane's simplex is active; okf:
+// its values agree within tol_f.
 template <int G, int N>
-__device__ __forceinline__ void decide_group(GroupSmem<G, N>& g, int lane, float tolx, float tolf) {
-  for (int gi = lane; gi < g.nsim; gi += 32) {
-    g.shr[gi] = 0;
-    g.okx[gi] = 1;
-    if (!g.active[gi]) continue;
+__device__ __forceinline__ bool decide_group(GroupSmem<G, N>& g, int lane, float tolf, bool& okf) {
+  const int gi = lane;
+  const bool live = lane < g.nsim && g.active[lane] != 0;
+  bool shrink = false;
+  okf = false;
+  if (live) {
     unsigned char* o = g.ord[gi];
     int sl[verts<N>()];
     float fv[verts<N>()];
@@ -592,7 +543,8 @@ __device__ __forceinline__ void decide_group(GroupSmem<G, N>& g, int lane, float
       if (fci < fw) { kind = 3; fnew = fci; } else kind = -1;
     }
     g.iters[gi] += 1;
-    if (kind >= 0) {
+    shrink = kind < 0;
+    if (!shrink) {
       // replace the worst vertex; the new point goes after every vertex with
       // a value <= its own (ties stay in front of it)
       const int ws = sl[N];
@@ -616,156 +568,164 @@ __device__ __forceinline__ void decide_group(GroupSmem<G, N>& g, int lane, float
         }
 #pragma unroll
       for (int r = 0; r < verts<N>(); ++r) o[r] = (unsigned char)sl[r];
-      bool okf = true;
+      okf = true;
 #pragma unroll
       for (int r = 1; r < verts<N>(); ++r) okf = okf && (fabsf(fv[r] - fv[0]) <= tolf);
-      g.okf[gi] = okf ? 1 : 0;
     } else {
       // shrink toward the best vertex: the values now, the coordinates below
 #pragma unroll
       for (int r = 1; r < verts<N>(); ++r) g.F[gi][sl[r]] = g.FT[gi][4 + r - 1];
-      g.shr[gi] = 1;
+    }
+  }
+  // shrink coordinates: for each shrinking simplex, its N x N (vertex rank
+  // >= 1, coordinate) updates over the lanes (the best vertex's row is only read)
+  const unsigned smask = __ballot_sync(0xffffffffu, shrink);
+  if (smask) {
+    for (unsigned m = smask; m; m &= m - 1) {
+      const int gs = __ffs(m) - 1;
+      const unsigned char* o = g.ord[gs];
+      for (int e = lane; e < N * N; e += 32) {
+        const int r = e / N + 1, j = e - (r - 1) * N;
+        g.U[gs][o[r]][j] = shrink_coord(g.U[gs][o[0]][j], g.U[gs][o[r]][j]);
+      }
+    }
+    __syncwarp();
+    // stable re-sort of the shrunk simplices
+    if (shrink) {
+      int sl[verts<N>()];
+      float fv[verts<N>()];
+#pragma unroll
+      for (int r = 0; r < verts<N>(); ++r) {
+        sl[r] = g.ord[gi][r];
+        fv[r] = g.F[gi][sl[r]];
+      }
+      rank_simplex<G, N>(g, gi, sl, fv);
+      okf = value_spread_ok<G, N>(g, gi, tolf) != 0;
     }
   }
   __syncwarp();
-  // shrink coordinates: for each shrinking simplex, its 18 x 18 (vertex rank
-  // >= 1, coordinate) updates over the lanes (the best vertex's row is only read)
-  static_assert(G <= 32, "one ballot bit per simplex");
-  const unsigned smask = __ballot_sync(0xffffffffu, lane < g.nsim && g.shr[lane]);
-  for (unsigned m = smask; m; m &= m - 1) {
-    const int gi = __ffs(m) - 1;
-    const unsigned char* o = g.ord[gi];
+  return live;
+}
+
+// Order of a wave's simplices: turn[] lists the lanes with `live` set by
+// increasing pulse width `upw` (the ln-space coordinate, clamped to the box).
+// The candidates of one simplex differ little in pulse width, so 32
+// consecutive candidates of this order end their pulse at nearly the same
+// sample; with the 9-parameter model every candidate has the same width.
+// Ordering the simplices (one per lane, ranked by 32 shuffles) takes the
+// place of a 512-bin counting sort of all candidates, which cost the deciding
+// warp 18 k of a decision's 42 k cycles for the same order to within the
+// spread of one simplex.
+template <int G, int N>
+__device__ __forceinline__ void order_simplices(GroupSmem<G, N>& g, int lane, bool live, float upw, const SearchParams& P) {
+  const unsigned lives = __ballot_sync(0xffffffffu, live);
+  int rank = 0;
+  if constexpr (search_coord<N>(kPw) < 0) {
+    rank = __popc(lives & ((1u << lane) - 1u));
+  } else {
+    const int bits = __float_as_int(fminf(fmaxf(upw, P.lnlo), P.lnhi));
+    const int key = live ? (bits ^ ((bits >> 31) & 0x7fffffff)) : 0x7fffffff;   // ordered as the floats are
+#pragma unroll 8
+    for (int l = 0; l < 32; ++l) {
+      const int k = __shfl_sync(0xffffffffu, key, l);
+      rank += k < key || (k == key && l < lane) ? 1 : 0;
+    }
+  }
+  if (live) g.turn[rank] = (unsigned char)lane;
+}
+
+// A group's first wave, the initial vertices of its simplices (one warp).
+template <int G, int N>
+__device__ __forceinline__ void first_wave(GroupSmem<G, N>& g, const SearchParams& P, int lane) {
+  constexpr int jp = search_coord<N>(kPw) < 0 ? 0 : search_coord<N>(kPw);
+  const bool live = lane < g.nsim;
+  order_simplices<G, N>(g, lane, live, live ? g.U[lane][0][jp] : 0.0f, P);
+  if (lane == 0) g.kind = 0;
+  if (lane == 0) g.state = kPending;
+  if (lane == 0) g.nvalid = verts<N>() * g.nsim;
+  if (lane == 0) g.evals = verts<N>() * g.nsim;
+  __syncwarp();
+}
+
+// A group's next trial wave (one warp, one lane per simplex; `live`: the
+// lane's simplex is active, okf: its values agree within tol_f).  First the
+// other half of the exit test (Sec. 3.3: every vertex within tol_x of the
+// best in max-norm) for the simplices that pass the first, spread over all
+// lanes; a group with no active simplex left, or at its iteration cap, is
+// done.  Then each lane sums its simplex's best N vertices row by row (N
+// independent sums, two per packed instruction, 8-byte loads) and writes the
+// four trial points (reflection, expansion, both contractions); the N shrink
+// points are formed by the evaluating threads from the vertices.
+// One lane per simplex instead of one per (simplex, coordinate) reads each
+// row's slot once instead of N times and keeps the centroid in registers:
+// with the ordering by simplex a decision takes a quarter of the cycles.
+template <int G, int N>
+__device__ __forceinline__ void next_wave(GroupSmem<G, N>& g, const SearchParams& P, int lane, int t_run, bool live,
+                                          bool okf) {
+  constexpr int jp = search_coord<N>(kPw) < 0 ? 0 : search_coord<N>(kPw);
+  for (unsigned m = __ballot_sync(0xffffffffu, live && okf); m; m &= m - 1) {
+    const int gs = __ffs(m) - 1;
+    const unsigned char* o = g.ord[gs];
+    bool ok = true;
     for (int e = lane; e < N * N; e += 32) {
       const int r = e / N + 1, j = e - (r - 1) * N;
-      g.U[gi][o[r]][j] = shrink_coord(g.U[gi][o[0]][j], g.U[gi][o[r]][j]);
+      ok = ok && (fabsf(g.U[gs][o[r]][j] - g.U[gs][o[0]][j]) <= P.tolx);
+    }
+    if (__all_sync(0xffffffffu, ok) && lane == gs) {
+      live = false;
+      g.active[gs] = 0;
     }
   }
-  __syncwarp();
-  // stable re-sort of the shrunk simplices
-  for (int gi = lane; gi < g.nsim; gi += 32) {
-    if (!g.shr[gi]) continue;
-    int sl[verts<N>()];
-    float fv[verts<N>()];
+  const int nact = __popc(__ballot_sync(0xffffffffu, live));
+  if (g.it >= t_run || nact == 0) {
+    if (lane == 0) g.state = kDone;
+    if (lane == 0) g.nvalid = 0;
+    __syncwarp();
+    return;
+  }
+  float upw = 0.0f;
+  if (live) {
+    const unsigned char* o = g.ord[lane];
+    float acc[N];
+    if constexpr (N % 2 == 0) {
+      float2 a[N / 2];
 #pragma unroll
-    for (int r = 0; r < verts<N>(); ++r) {
-      sl[r] = g.ord[gi][r];
-      fv[r] = g.F[gi][sl[r]];
-    }
-    rank_simplex<G, N>(g, gi, sl, fv);
-    g.okf[gi] = value_spread_ok<G, N>(g, gi, tolf);
-  }
-  __syncwarp();
-  centroids<G, N>(g, lane, tolx, [&](int gi) { return g.active[gi] != 0; });
-  __syncwarp();
-  for (int gi = lane; gi < g.nsim; gi += 32)
-    if (g.active[gi] && g.okx[gi] && g.okf[gi]) g.active[gi] = 0;
-  __syncwarp();
-}
-
-// Set up a group's next wave (one warp): the initial vertices (kind 0) or the
-// 22 trial points of every active simplex; a group with nothing left to
-// evaluate, or at its iteration cap, is done.  The warp writes the four trial
-// points (reflection, expansion, both contractions) to XT; the 18 shrink
-// points are formed by the evaluating threads from the vertices.
-template <int G, int N>
-__device__ __forceinline__ void next_wave(GroupSmem<G, N>& g, int kind, int t_run, int lane) {
-  static_assert(G <= 32, "one lane per simplex counts the active ones");
-  int nact = 0;
-  if (kind == 1) {
-    nact = (int)__reduce_add_sync(0xffffffffu, lane < g.nsim ? (unsigned)g.active[lane] : 0u);
-    if (g.it >= t_run || nact == 0) {
-      if (lane == 0) g.state = kDone;
-      if (lane == 0) g.nvalid = 0;
-      __syncwarp();
-      return;
-    }
-  }
-  for (int i = lane; i < kHistLen; i += 32) g.hist[i] = 0;
-  if (kind == 1) {
-#pragma unroll 2
-    for (int e = lane; e < g.nsim * N; e += 32) {
-      const int gi = e / N, j = e - gi * N;
-      if (g.active[gi]) {
-        const float xb = g.XB[gi][j], w = g.U[gi][g.ord[gi][N]][j];
+      for (int j = 0; j < N / 2; ++j) a[j] = make_float2(0.0f, 0.0f);
+#pragma unroll 3
+      for (int r = 0; r < N; ++r) {
+        const float2* x = reinterpret_cast<const float2*>(g.U[lane][o[r]]);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) g.XT[gi][q][j] = trial_coord(q, xb, w);
+        for (int j = 0; j < N / 2; ++j) a[j] = __fadd2_rn(a[j], x[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < N / 2; ++j) {
+        acc[2 * j] = a[j].x;
+        acc[2 * j + 1] = a[j].y;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < N; ++j) acc[j] = 0.0f;
+#pragma unroll 3
+      for (int r = 0; r < N; ++r) {
+        const float* x = g.U[lane][o[r]];
+#pragma unroll
+        for (int j = 0; j < N; ++j) acc[j] += x[j];
       }
     }
+    const float* w = g.U[lane][o[N]];
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const float xb = acc[j] / (float)N;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) g.XT[lane][q][j] = trial_coord(q, xb, w[j]);
+      if (j == jp) upw = xb;
+    }
   }
-  if (lane == 0) g.kind = kind;
+  order_simplices<G, N>(g, lane, live, upw, P);
+  if (lane == 0) g.kind = 1;
   if (lane == 0) g.state = kPending;
-  if (lane == 0 && kind == 1) g.evals += trials<N>() * nact;
-  __syncwarp();
-}
-
-// Counting sort of a group's freshly set-up wave by pulse-end time, by the
-// warp that set it up: lane l keys candidates l, l + 32, ..., the histogram
-// (cleared by next_wave) is scanned by the same warp, and afterwards
-// g.perm[0 .. g.nvalid) lists the candidates in key order.
-template <int G, int N>
-__device__ __forceinline__ void order_wave(GroupSmem<G, N>& g, const SacStage& V, const SearchParams& P, int lane) {
-  constexpr int R = wave_per_lane<G, N>();
-  static_assert(G * trials<N>() <= 32 * R, "every candidate keyed");
-  static_assert(G * trials<N>() < (1 << 16), "bin rank in 16 bits");
-  constexpr int kPwCoord = search_coord<N>(kPw);   // -1: pulse width held at the centre
-  const int ncand = (g.kind == 0 ? verts<N>() : trials<N>()) * g.nsim;
-#pragma unroll 4
-  for (int r = 0; r < R; ++r) {
-    const int c = lane + 32 * r;
-    int key = -1;
-    if (c < ncand) {
-      if (g.kind == 0) {
-        const int gi = c / verts<N>(), v = c - gi * verts<N>();
-        key = switch_key(kPwCoord < 0 ? 0.0f : g.U[gi][v][kPwCoord < 0 ? 0 : kPwCoord], V.pc[kPw], P.lnlo,
-                         P.lnhi, V.sc);
-      } else {
-        const int gi = c / trials<N>(), q = c - gi * trials<N>();
-        if (g.active[gi]) {
-          const float* a;
-          const float* bb;
-          trial_rows(g, gi, q, a, bb);
-          const int jp = kPwCoord < 0 ? 0 : kPwCoord;
-          key = switch_key(kPwCoord < 0 ? 0.0f : shrink_coord(a[jp], bb[jp]), V.pc[kPw], P.lnlo, P.lnhi, V.sc);
-        }
-      }
-    }
-    if (c < G * trials<N>()) g.kr[c] = key >= 0 ? (key << 16) | atomicAdd(&g.hist[hist_slot(key)], 1) : -1;
-  }
-  __syncwarp();
-  {
-    // lane l owns bins [per l, per l + per), stored at hist_slot(per l + i) =
-    // (per + 1) l + i: one padding word per lane keeps the lanes on distinct
-    // banks; the counts are read once into registers
-    constexpr int per = kHistPer;
-    static_assert(per * 32 == kSortBins && (per + 1) * 31 + per <= kHistLen, "histogram layout");
-    int* h = g.hist + lane * (per + 1);
-    int v[per];
-    int sum = 0;
-#pragma unroll
-    for (int i = 0; i < per; ++i) {
-      v[i] = h[i];
-      sum += v[i];
-    }
-    int incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int x = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += x;
-    }
-    int run = incl - sum;
-#pragma unroll
-    for (int i = 0; i < per; ++i) {
-      h[i] = run;
-      run += v[i];
-    }
-    if (lane == 31) g.nvalid = incl;
-  }
-  __syncwarp();
-#pragma unroll 4
-  for (int c = lane; c < ncand; c += 32) {
-    const int kr = g.kr[c];
-    if (kr >= 0) g.perm[g.hist[hist_slot(kr >> 16)] + (kr & 0xffff)] = (unsigned short)c;
-  }
+  if (lane == 0) g.nvalid = trials<N>() * nact;
+  if (lane == 0) g.evals += trials<N>() * nact;
   __syncwarp();
 }
 
@@ -826,24 +786,22 @@ __device__ __forceinline__ int try_claim(GroupSmem<G, N>& g, int lane, int& nchu
 
 // The warp that completed a group's wave: Nelder-Mead decisions on the values
 // just computed (ranking of the initial simplices, or the Lagarias step of
-// every active simplex), then the group's next wave, its ordering and its
-// publication.
+// every active simplex), then the group's next wave and its publication.
 template <int G, int N>
-__device__ __forceinline__ void advance_group(GroupSmem<G, N>& g, const SacStage& V, const SearchParams& P, int lane,
-                                              int t_run) {
+__device__ __forceinline__ void advance_group(GroupSmem<G, N>& g, const SearchParams& P, int lane, int t_run) {
+  bool live, okf;
   if (g.kind == 0) {
-    init_rank<G, N>(g, lane, P.tolx, P.tolf);
+    live = init_rank<G, N>(g, lane, P.tolf, okf);
   } else {
-    decide_group<G, N>(g, lane, P.tolx, P.tolf);
+    live = decide_group<G, N>(g, lane, P.tolf, okf);
     if (lane == 0) g.it += 1;
     __syncwarp();
   }
-  next_wave<G, N>(g, 1, t_run, lane);
-  if (g.state == kPending) order_wave<G, N>(g, V, P, lane);
+  next_wave<G, N>(g, P, lane, t_run, live, okf);
   publish_wave<G, N>(g, lane);
 }
 
-// Evaluate the candidate at position pos (key order) of a group's pending
+// Evaluate the candidate at position pos (wave order) of a group's pending
 // wave; qs is the calling thread's propagator slot.  Returns 1 when that
 // candidate's pulse ends inside the window (its pulse-end sample was
 // integrated substep by substep), else 0 (also for pos past the wave).
@@ -856,7 +814,6 @@ __device__ __forceinline__ int eval_candidate(GroupSmem<G, N>& g, const SacStage
   int pe = 0;
   const SacConst& sc = S.sc;
   const float sum0 = S.st.sum0, c0 = S.st.c0;
-  const int c = g.perm[pos];
   static_assert(!LEAN || N == N, "register-lean walk: 18 coordinates only");
   // both kinds of wave through one walk: a vertex is the row pair (v, v), for
   // which a + (a - a) / 2 = a exactly
@@ -864,11 +821,11 @@ __device__ __forceinline__ int eval_candidate(GroupSmem<G, N>& g, const SacStage
   const float* bb;
   float* out;
   if (g.kind == 0) {
-    const int gi = c / verts<N>(), v = c - gi * verts<N>();
+    const int k = pos / verts<N>(), v = pos - k * verts<N>(), gi = g.turn[k];
     a = bb = g.U[gi][v];
     out = &g.F[gi][v];
   } else {
-    const int gi = c / trials<N>(), q = c - gi * trials<N>();
+    const int k = pos / trials<N>(), q = pos - k * trials<N>(), gi = g.turn[k];
     trial_rows(g, gi, q, a, bb);
     out = &g.FT[gi][q];
   }
@@ -978,8 +935,7 @@ __global__ void __launch_bounds__(search_threads<G, N>(), MINB) k_search(SearchP
         const float v = gstate[idx];
         if (r < verts<N>() * N) (&g.U[gi][0][0])[r] = v;
         else if (r < verts<N>() * N + verts<N>()) g.F[gi][r - verts<N>() * N] = v;
-        else if (r < verts<N>() * N + verts<N>() + N) g.XB[gi][r - verts<N>() * N - verts<N>()] = v;
-        else if (r < verts<N>() * N + 2 * verts<N>() + N) g.ord[gi][r - verts<N>() * N - verts<N>() - N] = (unsigned char)__float_as_int(v);
+        else if (r < verts<N>() * N + 2 * verts<N>()) g.ord[gi][r - verts<N>() * N - verts<N>()] = (unsigned char)__float_as_int(v);
         else if (r == state_floats<N>() - 2) g.active[gi] = __float_as_int(v);
         else if (r == state_floats<N>() - 1) g.iters[gi] = __float_as_int(v);
       }
@@ -1013,14 +969,12 @@ __global__ void __launch_bounds__(search_threads<G, N>(), MINB) k_search(SearchP
       }
     }
     __syncthreads();
-    // warp h < NG sets up, orders and publishes group h's first wave
+    // warp h < NG sets up and publishes group h's first wave
     if (warp < NG) {
       GroupSmem<G, N>& g = S.grp[warp];
       if (g.nsim > 0) {
-        if (it0 == 0 && lane == 0) g.evals = verts<N>() * g.nsim;
-        __syncwarp();
-        next_wave<G, N>(g, it0 > 0 ? 1 : 0, t_run, lane);
-        if (g.state == kPending) order_wave<G, N>(g, S.sv, P, lane);
+        if (it0 > 0) next_wave<G, N>(g, P, lane, t_run, lane < g.nsim && g.active[lane] != 0, false);
+        else first_wave<G, N>(g, P, lane);
         publish_wave<G, N>(g, lane);
       }
     }
@@ -1062,7 +1016,7 @@ __global__ void __launch_bounds__(search_threads<G, N>(), MINB) k_search(SearchP
         if (last) __threadfence_block();
         __syncwarp();
         if (last) {
-          advance_group<G, N>(g, S.sv, P, lane, t_run);
+          advance_group<G, N>(g, P, lane, t_run);
           pref = gsel + 1 < NG ? gsel + 1 : 0;
         } else {
           pref = gsel;
@@ -1103,8 +1057,7 @@ __global__ void __launch_bounds__(search_threads<G, N>(), MINB) k_search(SearchP
         float v;
         if (r < verts<N>() * N) v = (&g.U[gi][0][0])[r];
         else if (r < verts<N>() * N + verts<N>()) v = g.F[gi][r - verts<N>() * N];
-        else if (r < verts<N>() * N + verts<N>() + N) v = g.XB[gi][r - verts<N>() * N - verts<N>()];
-        else if (r < verts<N>() * N + 2 * verts<N>() + N) v = __int_as_float((int)g.ord[gi][r - verts<N>() * N - verts<N>() - N]);
+        else if (r < verts<N>() * N + 2 * verts<N>()) v = __int_as_float((int)g.ord[gi][r - verts<N>() * N - verts<N>()]);
         else if (r == state_floats<N>() - 2) v = __int_as_float(g.active[gi]);
         else if (r == state_floats<N>() - 1) v = __int_as_float(g.iters[gi]);
         else v = 0.0f;

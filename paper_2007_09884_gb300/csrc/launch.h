@@ -40,7 +40,7 @@ struct SearchParams {
   int round_iters;         // iterations per launch
 };
 
-constexpr int kSearchStateFloats = 19 * 18 + 19 + 18 + 19 + 2;   // per saved simplex
+constexpr int kSearchStateFloats = 19 * 18 + 19 + 19 + 2;   // per saved simplex
 
 cudaError_t launch_gather(const float* const* src, const DevSac* sacs, float* dst, int n, cudaStream_t st);
 cudaError_t launch_nominal(const DevSac* sacs, int n, int pulse_mode, const float* init_opc, float* pc,
