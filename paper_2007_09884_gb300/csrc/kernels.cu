@@ -1109,146 +1109,180 @@ __global__ void __launch_bounds__(search_threads<G, N>(), MINB) k_search(SearchP
 
 // ------------------------------------------------------------------ finalize
 // FP64 re-computation of the winner's error (the serial check next to the
-// parallel value, as Fig. 4's CPU_check column).  The same RK4 map is applied
-// in double precision as dense 6x6 step matrices: within one input phase one
-// RK4 step of e' = A e is e <- e + Q e with Q = hA(I + hA/2(I + hA/3(I + hA/4))),
+// parallel value, as Fig. 4's CPU_check column), one warp per saccade.  The
+// same RK4 map is applied in double precision: within one input phase one RK4
+// step of e' = A e is e <- e + Q e with Q = hA(I + hA/2(I + hA/3(I + hA/4))),
 // raised to one sample interval by squaring; the pulse-end substep is split
-// into two RK4 steps.  Independent of the FP32 search formulation (dense
-// matrices, double precision, its own equilibria).
-struct M6 {
-  double a[6][6];
+// into two RK4 steps.  Independent of the FP32 search formulation (double
+// precision, matrix powers instead of substeps, its own equilibria).
+//
+// The FP64 pipe bounds it (two lanes per SM and clock: a warp instruction
+// holds the SM's pipe for about 16 cycles however many lanes it uses), so
+// every lane carries work.  Matrices keep the plant's block form (a 4x4
+// mechanical block, a 4x2 coupling, a diagonal activation pair: 26 entries)
+// with one entry per lane, five FMAs a product; and a phase's samples go 32
+// at a time, lane l holding the state after sample l + 1: five predicated
+// steps by (I + P)^1, ^2, ^4, ^8, ^16 start the lanes, (I + P)^32 moves them.
+// One thread per saccade with dense 6x6 matrices in local memory took 365 us
+// for one saccade of 150 samples and 880 us for 2,000 uneven ones.
+
+// Products by entry: entry e of a 32-double matrix is m[e / 4][e % 4] for
+// e < 16, c[(e - 16) / 2][(e - 16) % 2] for e < 24, d[e - 24] for e < 26 and
+// 0 above.  Entry e of a b is the dot product of a[ia ..] and b[ib + sb ..]
+// over four terms plus a[ka] b[kb]; entries past 25 serve as zeros.
+struct Lane64 {
+  int e, ia, ib, sb, ka, kb;
+  double unit;   // entry e of the identity
+  __device__ explicit Lane64(int lane) : e(lane) {
+    ia = ib = ka = kb = 26;
+    sb = 0;
+    unit = 0.0;
+    if (e < 16) {
+      ia = e & ~3;
+      ib = e & 3;
+      sb = 4;
+      unit = (e >> 2) == (e & 3) ? 1.0 : 0.0;
+    } else if (e < 24) {
+      ia = 4 * ((e - 16) >> 1);
+      ib = 16 + (e & 1);
+      sb = 2;
+      ka = e;
+      kb = 24 + (e & 1);
+    } else if (e < 26) {
+      ka = kb = e;
+      unit = 1.0;
+    }
+  }
+  __device__ __forceinline__ double mul(const double* a, const double* b) const {
+    double t = a[ka] * b[kb];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) t = fma(a[ia + k], b[ib + sb * k], t);
+    return t;
+  }
+  // m[e] = v once every lane has read what it needs
+  __device__ __forceinline__ void put(double* m, double v) const {
+    __syncwarp();
+    m[e] = v;
+    __syncwarp();
+  }
 };
 
-__device__ void m6_zero(M6& m) {
-  for (int i = 0; i < 6; ++i)
-    for (int j = 0; j < 6; ++j) m.a[i][j] = 0.0;
+struct Warp64 {
+  double A[32], Q[32], W[32], B[32], P[6][32];
+  double par[kNumParams], rcp[12];
+  float opc[kNumParams];
+};
+
+// out = T4(h A) - I by Horner (w: scratch).
+__device__ void step_inc64(const Lane64& L, const double* A, double h, double* w, double* out) {
+  L.put(w, fma(0.25 * h, A[L.e], L.unit));
+  L.put(w, fma(h / 3.0, L.mul(A, w), L.unit));
+  L.put(w, fma(0.5 * h, L.mul(A, w), L.unit));
+  L.put(out, h * L.mul(A, w));
 }
 
-// r = a + b + a b (increment form of (I + a)(I + b)); r may alias neither
-__device__ void m6_mul_inc(const M6& a, const M6& b, M6& r) {
-  for (int i = 0; i < 6; ++i)
-    for (int j = 0; j < 6; ++j) {
-      double acc = a.a[i][j] + b.a[i][j];
-      for (int k = 0; k < 6; ++k) acc = fma(a.a[i][k], b.a[k][j], acc);
-      r.a[i][j] = acc;
-    }
+// r = a + b + a b (increment form of (I + a)(I + b)); r may be a or b.
+__device__ __forceinline__ void mul_inc64(const Lane64& L, const double* a, const double* b, double* r) {
+  L.put(r, a[L.e] + b[L.e] + L.mul(a, b));
 }
 
-// plant matrix of one phase (state theta, omega, x, y, Fa, Fn)
-__device__ void plant_matrix64(const double* p, double ita, double itn, M6& A) {
-  m6_zero(A);
-  const double kp = p[kNcAg] + p[kNcAnt];
-  const double iJ = 1.0 / p[kJ], iBa = 1.0 / p[kBAg], iBn = 1.0 / p[kBAnt];
-  A.a[0][1] = 1.0;
-  A.a[1][0] = -(p[kSeAg] + p[kSeAnt] + kp) * iJ;
-  A.a[1][1] = -p[kBp] * iJ;
-  A.a[1][2] = p[kSeAg] * iJ;
-  A.a[1][3] = -p[kSeAnt] * iJ;
-  A.a[2][0] = p[kSeAg] * iBa;
-  A.a[2][2] = -(p[kSeAg] + p[kLtAg]) * iBa;
-  A.a[2][4] = iBa;
-  A.a[3][0] = -p[kSeAnt] * iBn;
-  A.a[3][3] = -(p[kSeAnt] + p[kLtAnt]) * iBn;
-  A.a[3][5] = iBn;
-  A.a[4][4] = -ita;
-  A.a[5][5] = -itn;
-}
-
-// Q = T4(hA) - I by Horner
-__device__ void step_inc64(const M6& A, double h, M6& Q) {
-  M6 W, T;
-  for (int i = 0; i < 6; ++i)
-    for (int j = 0; j < 6; ++j) W.a[i][j] = (i == j ? 1.0 : 0.0) + 0.25 * h * A.a[i][j];
-  const double c[2] = {h / 3.0, 0.5 * h};
-  for (int lev = 0; lev < 2; ++lev) {
-    for (int i = 0; i < 6; ++i)
-      for (int j = 0; j < 6; ++j) {
-        double acc = 0.0;
-        for (int k = 0; k < 6; ++k) acc = fma(A.a[i][k], W.a[k][j], acc);
-        T.a[i][j] = (i == j ? 1.0 : 0.0) + c[lev] * acc;
-      }
-    W = T;
-  }
-  for (int i = 0; i < 6; ++i)
-    for (int j = 0; j < 6; ++j) {
-      double acc = 0.0;
-      for (int k = 0; k < 6; ++k) acc = fma(A.a[i][k], W.a[k][j], acc);
-      Q.a[i][j] = h * acc;
-    }
-}
-
-__device__ void pow_inc64(const M6& q, int n, M6& out) {
-  M6 base = q, tmp;
-  bool have = false;
-  while (true) {
-    if (n & 1) {
-      if (have) { m6_mul_inc(out, base, tmp); out = tmp; }
-      else { out = base; have = true; }
-    }
-    n >>= 1;
-    if (!n) break;
-    m6_mul_inc(base, base, tmp);
-    base = tmp;
+// out = (I + q)^n - I for n >= 0 (left to right; out is not q).
+__device__ void pow_inc64(const Lane64& L, const double* q, int n, double* out) {
+  L.put(out, n > 0 ? q[L.e] : 0.0);
+  for (int b = 30 - __clz(max(n, 1)); b >= 0; --b) {
+    mul_inc64(L, out, out, out);
+    if ((n >> b) & 1) mul_inc64(L, out, q, out);
   }
 }
 
-__device__ void apply_inc64(const M6& q, double* e) {
-  double n[6];
-  for (int i = 0; i < 6; ++i) {
-    double acc = e[i];
-    for (int k = 0; k < 6; ++k) acc = fma(q.a[i][k], e[k], acc);
-    n[i] = acc;
+// e <- (I + q) e on every lane's own vector.
+__device__ __forceinline__ void apply_inc64(const double* q, double (&e)[6]) {
+  double n[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    n[i] = fma(q[16 + 2 * i], e[4], e[i]);
+    n[i] = fma(q[17 + 2 * i], e[5], n[i]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) n[i] = fma(q[4 * i + k], e[k], n[i]);
   }
-  for (int i = 0; i < 6; ++i) e[i] = n[i];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) e[i] = n[i];
+  e[4] = fma(q[24], e[4], e[4]);
+  e[5] = fma(q[25], e[5], e[5]);
 }
 
-// one RK4 step of length hs on e' = A e (Horner form of T4(hs A) e)
-__device__ void rk4_vec64(const M6& A, double hs, double* e) {
-  double w[6], v[6];
-  for (int i = 0; i < 6; ++i) w[i] = e[i];
-  const double c[4] = {0.25 * hs, hs / 3.0, 0.5 * hs, hs};
-  for (int lev = 0; lev < 4; ++lev) {
-    for (int i = 0; i < 6; ++i) {
-      double acc = 0.0;
-      for (int k = 0; k < 6; ++k) acc = fma(A.a[i][k], w[k], acc);
-      v[i] = acc;
+__device__ __forceinline__ double warp_sum64(double v) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+struct Err64 {
+  double s2, s1;   // this lane's share of the squared and absolute errors
+  __device__ __forceinline__ void add(double r) {
+    s2 = fma(r, r, s2);
+    s1 += fabs(r);
+  }
+};
+
+// n samples of one phase from the state e (the same on every lane), the first
+// of them sample k0, around the equilibrium angle th; leaves the state after
+// the last one in e.  W.P[0] holds the one-sample propagator.
+__device__ void run_phase64(const Lane64& L, Warp64& W, double (&e)[6], int k0, int n, double th, double sg,
+                            const float* y, Err64& err) {
+  if (n <= 0) return;
+  for (int b = 1; b < 6; ++b) mul_inc64(L, W.P[b - 1], W.P[b - 1], W.P[b]);
+  apply_inc64(W.P[0], e);
+#pragma unroll 1
+  for (int b = 0; b < 5; ++b) {
+    double t[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) t[i] = e[i];
+    apply_inc64(W.P[b], t);
+    if ((L.e >> b) & 1)
+#pragma unroll
+      for (int i = 0; i < 6; ++i) e[i] = t[i];
+  }
+#pragma unroll 1
+  for (int i = L.e;; i += 32) {
+    if (i < n) err.add(sg * (th + e[0]) - (double)y[k0 + i]);
+    if (i - L.e + 32 >= n) break;   // warp-uniform
+    apply_inc64(W.P[5], e);
+  }
+#pragma unroll
+  for (int i = 0; i < 6; ++i) e[i] = __shfl_sync(0xffffffffu, e[i], (n - 1) & 31);
+}
+
+// Mean squared and mean absolute error of the OPC vector W.opc's trajectory
+// against the trace y, FP64, by one warp.
+__device__ void errors64(const Lane64& L, Warp64& W, const DevSac& d, const float* y, double* mse, double* mae) {
+  if (L.e < kNumParams) W.par[L.e] = (double)W.opc[L.e];
+  __syncwarp();
+  const double* p = W.par;
+  // the reciprocals, one lane each
+  enum { iJ, iBa, iBn, iSa, iSn, iSLa, iSLn, iTaA, iTaN, iTdA, iTdN };
+  {
+    const int idx[7] = {kJ, kBAg, kBAnt, kSeAg, kSeAnt, kSeAg, kSeAnt};
+    double den = 1.0, num = 1.0;
+    if (L.e < 7) {
+      den = p[idx[L.e]] + (L.e == iSLa ? p[kLtAg] : L.e == iSLn ? p[kLtAnt] : 0.0);
+    } else if (L.e < 11) {
+      den = p[kTacAg + L.e - 7];   // the four time constants, in OPC order
+      num = 1000.0;
     }
-    for (int i = 0; i < 6; ++i) w[i] = fma(c[lev], v[i], e[i]);
+    const double r = num / den;
+    if (L.e < 11) W.rcp[L.e] = r;
+    __syncwarp();
   }
-  for (int i = 0; i < 6; ++i) e[i] = w[i];
-}
-
-// equilibrium under constant active-state tensions (fa, fn), double
-__device__ void equilibrium64(const double* p, double fa, double fn, double* s) {
-  const double ag = p[kSeAg] / (p[kSeAg] + p[kLtAg]);
-  const double an = p[kSeAnt] / (p[kSeAnt] + p[kLtAnt]);
-  const double kp = p[kNcAg] + p[kNcAnt];
-  const double th = (ag * fa - an * fn) / (kp + ag * p[kLtAg] + an * p[kLtAnt]);
-  const double ta = ag * (fa - p[kLtAg] * th), tn = an * (fn + p[kLtAnt] * th);
-  s[0] = th; s[1] = 0.0;
-  s[2] = th + ta / p[kSeAg];
-  s[3] = tn / p[kSeAnt] - th;
-  s[4] = fa; s[5] = fn;
-}
-
-__device__ void step_levels64(const double* p, double th, double* fa, double* fn) {
-  const double ta = p[kNcFix] + p[kNcAg] * th, tn = p[kNcFix] - p[kNcAnt] * th;
-  *fa = ta * (1.0 + p[kLtAg] / p[kSeAg]) + p[kLtAg] * th;
-  *fn = tn * (1.0 + p[kLtAnt] / p[kSeAnt]) - p[kLtAnt] * th;
-}
-
-// Mean squared and mean absolute error of the winner's trajectory, FP64.
-__device__ void errors64(const float* pf, const DevSac& d, const float* y, double* mse, double* mae) {
-  double p[kNumParams];
-  for (int j = 0; j < kNumParams; ++j) p[j] = (double)pf[j];
+  const double* r = W.rcp;
   const double th0 = d.th0, thf = d.thf, sg = d.sign;
+  const double ag = p[kSeAg] * r[iSLa], an = p[kSeAnt] * r[iSLn], kp = p[kNcAg] + p[kNcAnt];
   // substeps refined for stiff candidates, the oracle's rule in double
-  const double tmin = fmin(fmin(p[kTacAg], p[kTacAnt]), fmin(p[kTdeAg], p[kTdeAnt]));
-  const double est = p[kBp] / p[kJ] + (p[kSeAg] + p[kLtAg]) / p[kBAg] + (p[kSeAnt] + p[kLtAnt]) / p[kBAnt] +
-                     1000.0 / tmin;
+  const double rate = fmax(fmax(r[iTaA], r[iTaN]), fmax(r[iTdA], r[iTdN]));
+  const double est = p[kBp] * r[iJ] + (p[kSeAg] + p[kLtAg]) * r[iBa] + (p[kSeAnt] + p[kLtAnt]) * r[iBn] + rate;
   int nsub = d.nsub;
   double h = 1.0 / ((double)d.fs * nsub);
-  for (int r = 0; r < kMaxRefine && !(h * est <= 2.5); ++r) {
+  for (int t = 0; t < kMaxRefine && !(h * est <= 2.5); ++t) {
     h *= 0.5;
     nsub *= 2;
   }
@@ -1257,110 +1291,155 @@ __device__ void errors64(const float* pf, const DevSac& d, const float* y, doubl
   if (tau > 1.0e9) tau = 1.0e9;
   const double fl = floor(tau);
   const double frac = tau - fl;
-  double fa0, fn0, faf, fnf;
-  step_levels64(p, th0, &fa0, &fn0);
-  step_levels64(p, thf, &faf, &fnf);
+  // equilibria, one lane each: rest at th0, the pulse held, rest at thf
   double s0[6], s1[6], s2[6];
-  equilibrium64(p, fa0, fn0, s0);          // rest at th0
-  equilibrium64(p, p[kNsacAg], p[kNsacAnt], s1);
-  equilibrium64(p, faf, fnf, s2);          // rest at thf
-  double s2e = 0.0, s1e = 0.0;
-  const int kend = d.onset < d.L - 1 ? d.onset : d.L - 1;
-  for (int k = 0; k <= kend; ++k) {       // at rest up to onset
-    const double e = sg * th0 - (double)y[k];
-    s2e += e * e;
-    s1e += fabs(e);
+  {
+    const double th = L.e == 0 ? th0 : thf;
+    const double ta = p[kNcFix] + p[kNcAg] * th, tn = p[kNcFix] - p[kNcAnt] * th;
+    double fa = ta * (1.0 + p[kLtAg] * r[iSa]) + p[kLtAg] * th;
+    double fn = tn * (1.0 + p[kLtAnt] * r[iSn]) - p[kLtAnt] * th;
+    if (L.e == 1) {
+      fa = p[kNsacAg];
+      fn = p[kNsacAnt];
+    }
+    const double q = (ag * fa - an * fn) / (kp + ag * p[kLtAg] + an * p[kLtAnt]);
+    const double xa = ag * (fa - p[kLtAg] * q), xn = an * (fn + p[kLtAnt] * q);
+    const double s[6] = {q, 0.0, q + xa * r[iSa], xn * r[iSn] - q, fa, fn};
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      s0[i] = __shfl_sync(0xffffffffu, s[i], 0);
+      s1[i] = __shfl_sync(0xffffffffu, s[i], 1);
+      s2[i] = __shfl_sync(0xffffffffu, s[i], 2);
+    }
   }
+  Err64 err{0.0, 0.0};
+  const int kend = d.onset < d.L - 1 ? d.onset : d.L - 1;
+  for (int k = L.e; k <= kend; k += 32) err.add(sg * th0 - (double)y[k]);   // at rest up to onset
   const int ntot = d.L - 1 - d.onset;
   if (ntot > 0) {
-    M6 A1, A2, Q1, Q2, P1, P2;
-    plant_matrix64(p, 1000.0 / p[kTacAg], 1000.0 / p[kTdeAnt], A1);
-    plant_matrix64(p, 1000.0 / p[kTdeAg], 1000.0 / p[kTacAnt], A2);
-    step_inc64(A1, h, Q1);
-    step_inc64(A2, h, Q2);
-    pow_inc64(Q1, nsub, P1);
-    pow_inc64(Q2, nsub, P2);
-    long long n1;
-    int jsw = 0;
+    // plant matrix of the pulse phase; the step phase differs in entries 24, 25
+    {
+      double a = 0.0;
+      switch (L.e) {
+        case 1: a = 1.0; break;
+        case 4: a = -(p[kSeAg] + p[kSeAnt] + kp) * r[iJ]; break;
+        case 5: a = -p[kBp] * r[iJ]; break;
+        case 6: a = p[kSeAg] * r[iJ]; break;
+        case 7: a = -p[kSeAnt] * r[iJ]; break;
+        case 8: a = p[kSeAg] * r[iBa]; break;
+        case 10: a = -(p[kSeAg] + p[kLtAg]) * r[iBa]; break;
+        case 12: a = -p[kSeAnt] * r[iBn]; break;
+        case 15: a = -(p[kSeAnt] + p[kLtAnt]) * r[iBn]; break;
+        case 20: a = r[iBa]; break;
+        case 23: a = r[iBn]; break;
+        case 24: a = -r[iTaA]; break;
+        case 25: a = -r[iTdN]; break;
+        default: break;
+      }
+      L.put(W.A, a);
+    }
+    int n1, jsw = 0;
     bool sw;
-    if (fl >= (double)ntot * nsub) { n1 = ntot; sw = false; }
-    else { const long long J = (long long)fl; n1 = J / nsub; jsw = (int)(J - n1 * nsub); sw = true; }
+    if (fl >= (double)ntot * nsub) {
+      n1 = ntot;
+      sw = false;
+    } else {
+      const int J = (int)fl;
+      n1 = J / nsub;
+      jsw = J - n1 * nsub;
+      sw = true;
+    }
     double e[6];
+#pragma unroll
     for (int i = 0; i < 6; ++i) e[i] = s0[i] - s1[i];
-    int k = d.onset + 1;
-    for (long long i = 0; i < n1; ++i, ++k) {
-      apply_inc64(P1, e);
-      const double r = sg * (s1[0] + e[0]) - (double)y[k];
-      s2e += r * r;
-      s1e += fabs(r);
+    step_inc64(L, W.A, h, W.W, W.Q);
+    if (n1 > 0) {
+      pow_inc64(L, W.Q, nsub, W.P[0]);
+      run_phase64(L, W, e, d.onset + 1, n1, s1[0], sg, y, err);
     }
     if (sw) {
-      for (int s = 0; s < jsw; ++s) apply_inc64(Q1, e);
-      rk4_vec64(A1, frac * h, e);
+      // the sample that holds the pulse end
+      pow_inc64(L, W.Q, jsw, W.B);
+      apply_inc64(W.B, e);
+      step_inc64(L, W.A, frac * h, W.W, W.B);
+      apply_inc64(W.B, e);
+#pragma unroll
       for (int i = 0; i < 6; ++i) e[i] += s1[i] - s2[i];
-      rk4_vec64(A2, h - frac * h, e);
-      for (int s = jsw + 1; s < nsub; ++s) apply_inc64(Q2, e);
-      double r = sg * (s2[0] + e[0]) - (double)y[k];
-      s2e += r * r;
-      s1e += fabs(r);
-      ++k;
-      for (; k < d.L; ++k) {
-        apply_inc64(P2, e);
-        r = sg * (s2[0] + e[0]) - (double)y[k];
-        s2e += r * r;
-        s1e += fabs(r);
+      L.put(W.A, L.e == 24 ? -r[iTdA] : L.e == 25 ? -r[iTaN] : W.A[L.e]);
+      step_inc64(L, W.A, h - frac * h, W.W, W.B);
+      apply_inc64(W.B, e);
+      step_inc64(L, W.A, h, W.W, W.Q);
+      pow_inc64(L, W.Q, nsub - 1 - jsw, W.B);
+      apply_inc64(W.B, e);
+      const int k = d.onset + 1 + n1;
+      if (L.e == 0) err.add(sg * (s2[0] + e[0]) - (double)y[k]);
+      if (k + 1 < d.L) {
+        pow_inc64(L, W.Q, nsub, W.P[0]);
+        run_phase64(L, W, e, k + 1, d.L - 1 - k, s2[0], sg, y, err);
       }
     }
   }
-  *mse = s2e / d.L;
-  *mae = s1e / d.L;
+  *mse = warp_sum64(err.s2) / d.L;
+  *mae = warp_sum64(err.s1) / d.L;
 }
 
+// Result of one saccade per warp (= block): the lowest value over its unit
+// records (ties to the lowest simplex), the winner's OPC vector and its FP64
+// errors.
 template <int N>
-__global__ void k_finalize(const DevSac* sacs, const float* traces, const float* pc, const int* ustart,
-                           int ngroups, const float* unit_best, float lnlo, float lnhi, int n,
-                           opmm_fit_result* out, const int* list) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(32) k_finalize(const DevSac* sacs, const float* traces, const float* pc,
+                                                 const int* ustart, int ngroups, const float* unit_best, float lnlo,
+                                                 float lnhi, int n, opmm_fit_result* out, const int* list) {
+  __shared__ Warp64 W;
+  const int i = blockIdx.x, lane = threadIdx.x;
   if (i >= n) return;
+  const Lane64 L(lane);
   const int b = list ? list[i] : i;
-  int w = -1, wsimp = 0x7fffffff, evals = 0, pe = 0;
+  int w = 0x7fffffff, wsimp = 0x7fffffff, evals = 0, pe = 0;
   float wf = INFINITY;
   const int u0 = ustart ? ustart[b] : b * ngroups;   // slot-major records when no start table
-  for (int u = u0; u < u0 + ngroups; ++u) {
+  for (int u = u0 + lane; u < u0 + ngroups; u += 32) {
     const float* rec = unit_best + (size_t)u * kUnitRec;
     const float f = rec[0];
     const int s = __float_as_int(rec[1]);
     evals += __float_as_int(rec[3]);
     pe += __float_as_int(rec[22]);
-    if (w < 0 || f < wf || (f == wf && s < wsimp)) { w = u; wf = f; wsimp = s; }
+    if (w == 0x7fffffff || f < wf || (f == wf && s < wsimp)) { w = u; wf = f; wsimp = s; }
   }
-  opmm_fit_result r;
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    const float f2 = __shfl_xor_sync(0xffffffffu, wf, o);
+    const int s2 = __shfl_xor_sync(0xffffffffu, wsimp, o), w2 = __shfl_xor_sync(0xffffffffu, w, o);
+    evals += __shfl_xor_sync(0xffffffffu, evals, o);
+    pe += __shfl_xor_sync(0xffffffffu, pe, o);
+    if (f2 < wf || (f2 == wf && (s2 < wsimp || (s2 == wsimp && w2 < w)))) { w = w2; wf = f2; wsimp = s2; }
+  }
   const DevSac d = sacs[b];
   const float* rec = unit_best + (size_t)w * kUnitRec;
-  {
-    float p[kNumParams];
-    u_to_p<N>(rec + 4, pc + (size_t)b * kNumParams, lnlo, lnhi, p);
-    for (int j = 0; j < kNumParams; ++j) r.opc[j] = p[j];
+  if (lane < kNumParams) {
+    // as u_to_p, one entry per lane
+    const int c = search_coord<N>(lane);
+    const float p0 = pc[(size_t)b * kNumParams + lane];
+    W.opc[lane] = c < 0 ? p0 : p0 * __expf(fminf(fmaxf(rec[4 + (c < 0 ? 0 : c)], lnlo), lnhi));
   }
-  r.f = wf;
-  r.iterations_run = __float_as_int(rec[2]);
-  r.winner = wsimp;
-  r.evaluations = evals;
-  r.pulse_end_evals = pe;
-  r.reserved = 0;
-  r.source = OPMM_SOURCE_PLAIN;
-  if (isfinite(wf)) {
-    double mse, mae;
-    errors64(r.opc, d, traces + d.off, &mse, &mae);
-    r.rms_deg = sqrt(mse);
+  __syncwarp();
+  double mse = INFINITY, mae = INFINITY;
+  const bool ok = isfinite(wf);
+  if (ok) errors64(L, W, d, traces + d.off, &mse, &mae);
+  opmm_fit_result& r = out[i];
+  if (lane < kNumParams) r.opc[lane] = W.opc[lane];
+  if (lane == 0) {
+    r.f = wf;
+    r.iterations_run = __float_as_int(rec[2]);
+    r.winner = wsimp;
+    r.evaluations = evals;
+    r.pulse_end_evals = pe;
+    r.reserved = 0;
+    r.source = OPMM_SOURCE_PLAIN;
+    r.rms_deg = ok ? sqrt(mse) : INFINITY;
     r.l1_deg = mae;
-    r.status = 0;
-  } else {
-    r.rms_deg = INFINITY;
-    r.l1_deg = INFINITY;
-    r.status = 1;
+    r.status = ok ? 0 : 1;
   }
-  out[i] = r;
 }
 
 // ------------------------------------------------------------------ refinement
@@ -1673,20 +1752,24 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(const DevSac* sacs, c
 }
 
 // FP64 re-computation of each refined vector's errors (as k_finalize does for
-// the search), one thread per saccade spread over the SMs.
-__global__ void k_refine_check(const DevSac* sacs, const float* traces, int n, opmm_fit_result* out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// the search), one warp per saccade.
+__global__ void __launch_bounds__(32) k_refine_check(const DevSac* sacs, const float* traces, int n,
+                                                     opmm_fit_result* out) {
+  __shared__ Warp64 W;
+  const int i = blockIdx.x, lane = threadIdx.x;
   if (i >= n) return;
   opmm_fit_result& r = out[i];
+  double mse = INFINITY, mae = INFINITY;
   if (r.status == 0) {
+    if (lane < kNumParams) W.opc[lane] = r.opc[lane];
+    __syncwarp();
     const DevSac d = sacs[i];
-    double mse, mae;
-    errors64(r.opc, d, traces + d.off, &mse, &mae);
-    r.rms_deg = sqrt(mse);
+    errors64(Lane64(lane), W, d, traces + d.off, &mse, &mae);
+    mse = sqrt(mse);
+  }
+  if (lane == 0) {
+    r.rms_deg = mse;
     r.l1_deg = mae;
-  } else {
-    r.rms_deg = INFINITY;
-    r.l1_deg = INFINITY;
   }
 }
 
@@ -1734,7 +1817,7 @@ cudaError_t launch_refine(int dim, const DevSac* sacs, const float* traces, cons
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_refine_check<<<(n + 3) / 4, 4, 0, st>>>(sacs, traces, n, out);
+  k_refine_check<<<n, 32, 0, st>>>(sacs, traces, n, out);
   return cudaGetLastError();
 }
 
@@ -1927,13 +2010,10 @@ cudaError_t launch_finalize(const DevSac* sacs, const float* traces, const float
                             int ngroups, const float* unit_best, float lnlo, float lnhi, int n,
                             opmm_fit_result* out, cudaStream_t st, const int* list, int dim) {
   if (n <= 0) return cudaSuccess;
-  // the FP64 recomputation is latency bound per thread and the FP64 pipe is
-  // narrow: spread the saccades over all SMs, a few threads per block
   if (dim == 9)
-    k_finalize<9><<<(n + 3) / 4, 4, 0, st>>>(sacs, traces, pc, ustart, ngroups, unit_best, lnlo, lnhi, n, out, list);
+    k_finalize<9><<<n, 32, 0, st>>>(sacs, traces, pc, ustart, ngroups, unit_best, lnlo, lnhi, n, out, list);
   else if (dim == kNumParams)
-    k_finalize<kNumParams><<<(n + 3) / 4, 4, 0, st>>>(sacs, traces, pc, ustart, ngroups, unit_best, lnlo, lnhi, n,
-                                                       out, list);
+    k_finalize<kNumParams><<<n, 32, 0, st>>>(sacs, traces, pc, ustart, ngroups, unit_best, lnlo, lnhi, n, out, list);
   else
     return cudaErrorInvalidValue;
   return cudaGetLastError();
