@@ -484,6 +484,12 @@ Status enqueue_fit(opmm_plan* p, cudaStream_t st) {
                      "D2H error word");
 }
 
+// One Nelder-Mead step of a search unit against its 32-candidate chunks, in
+// thousands of SM cycles (2 x 32 packed, 150 samples at 1 kHz; one simplex
+// 22.6, 8 33.7, 16 39.8, 32 53.1, 48 79.2, 64 simplices 101): a chunk's and a
+// decision's latency first, the SM's throughput from about 24 chunks on.
+static double unit_step(int chunks) { return std::max(21.0 + 1.5 * chunks, 5.0 + 2.18 * chunks); }
+
 // Candidate launch shapes: the search kernel's variants (simplices per block G,
 // threads = 22 G rounded to warps, register bound for MINB resident blocks) at
 // the occupancy the device allows for this trace capacity.  Returns (variant,
@@ -537,8 +543,20 @@ static Status autotune(opmm_plan* p) {
     return Status();
   }
   if (!p->autotune || cands.size() == 1) {
-    p->variant = cands[0].first;        // variant 0 (16 simplices per block) when launchable
-    p->blocks_per_sm = cands[0].second;
+    // untuned (one-shot) fits take the shape the tuner keeps choosing: the
+    // first of search_variant_default's preferences that this trace capacity
+    // leaves room for
+    auto first = cands[0];
+    for (int k = 0; search_variant_default(p->dim, k) >= 0; ++k) {
+      const int v = search_variant_default(p->dim, k);
+      auto c = std::find_if(cands.begin(), cands.end(), [&](const std::pair<int, int>& x) { return x.first == v; });
+      if (c != cands.end()) {
+        first = *c;
+        break;
+      }
+    }
+    p->variant = first.first;
+    p->blocks_per_sm = first.second;
     return Status();
   }
   cudaStream_t st = ctx->stream;
@@ -584,13 +602,47 @@ static Status autotune(opmm_plan* p) {
   return Status();
 }
 
+// Units per saccade: the number of units that n saccades' S simplices are
+// split into evenly, at most G simplices each, or 0 for full units of G and a
+// last one with the rest.  The split with the least turns of the blocks times
+// the step of one unit: a batch with many units per block keeps its units as
+// large as they come (a simplex costs 1.6 k cycles a step in a unit of 64 and
+// 2.5 k in one of 16), a few saccades are spread over every SM (one saccade
+// of 186 simplices: 93 units of two instead of 6 of 32).  A simplex evolves
+// the same in any unit, so the results do not depend on the split.
+static int split_units(int n, int S, int variant, int blocks) {
+  const int G = search_variant_g(variant), NG = search_variant_groups(variant);
+  const int nt = search_variant_dim(variant) + 4;
+  auto step = [&](int m) {   // one step of a unit of m simplices in NG even groups
+    int chunks = 0;
+    for (int h = 0; h < NG; ++h) chunks += (nt * ((m * (h + 1)) / NG - (m * h) / NG) + 31) / 32;
+    return unit_step(chunks);
+  };
+  auto turns = [&](int ng) { return std::max(1.0, (double)(((long long)n * ng + blocks - 1) / blocks)); };
+  const int least = (S + G - 1) / G;
+  double best = 1e300;
+  int pick = least;
+  for (int ng = least; ng <= S; ++ng) {
+    const double t = turns(ng) * step((S + ng - 1) / ng);
+    if (t < best * 0.999) {
+      best = t;
+      pick = ng;
+    }
+  }
+  // with many units per saccade an even split only rounds every group up to
+  // whole chunks, and full units lose only in their last one
+  return pick == least && (S % G == 0 || least > 8) ? 0 : pick;
+}
+
 // Unit list for G simplices per block: saccades in decreasing order of work
-// (samples after onset), each split into ceil(S / G) groups of simplices.
+// (samples after onset), each split into units by split_units (a probe: into
+// full units).
 // With probe_stride k > 1, the autotuner's sample: only the saccades at
 // positions k/2, k/2 + k, ... of that order (the unit starts are then not
 // meaningful; no result is read from a probe).
 Status build_units(opmm_plan* p, int G, int probe_stride) {
-  p->ngroups = (p->S + G - 1) / G;
+  const int even = probe_stride > 1 ? 0 : split_units(p->n, p->S, p->variant, p->ctx->num_sms * p->blocks_per_sm);
+  p->ngroups = even ? even : (p->S + G - 1) / G;
   const size_t nu = (size_t)p->n * (size_t)p->ngroups;
   if (nu > (size_t)0x7fffffff) return Status(OPMM_EINVAL, "too many work units");
   std::vector<int> order((size_t)p->n);
@@ -623,7 +675,7 @@ Status build_units(opmm_plan* p, int G, int probe_stride) {
   p->params.units = p->d_units.as<int2>();
   p->params.n_units = p->n_units;
   p->params.ngroups = p->ngroups;
-  p->params.balanced = 0;
+  p->params.balanced = even ? 1 : 0;
   p->params.unit_best = p->d_unit_best.as<float>();
   return s;
 }

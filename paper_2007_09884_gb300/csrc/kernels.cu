@@ -1919,14 +1919,27 @@ constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 static bool variant_ok(int v) { return v >= 0 && v < kNumVariants; }
 int search_variant_count() { return kNumVariants; }
 int search_variant_g(int v) { return variant_ok(v) ? kVariants[v].NG * kVariants[v].G : 0; }
+int search_variant_groups(int v) { return variant_ok(v) ? kVariants[v].NG : 0; }
 int search_variant_dim(int v) { return variant_ok(v) ? kVariants[v].N : 0; }
 int search_variant_minb(int v) { return variant_ok(v) ? kVariants[v].minb : 0; }
 int search_variant_lean(int v) { return variant_ok(v) ? kVariants[v].lean : 0; }
 int search_variant_pack(int v) { return variant_ok(v) ? kVariants[v].pack : 0; }
+// The packed walk at that unit size when there is one (the same results as the
+// scalar walk, a quarter faster), else the first variant.
 int search_variant_for(int unit, int dim) {
+  int first = -1;
   for (int v = 0; v < kNumVariants; ++v)
-    if (kVariants[v].NG * kVariants[v].G == unit && kVariants[v].N == dim) return v;
-  return -1;
+    if (kVariants[v].NG * kVariants[v].G == unit && kVariants[v].N == dim) {
+      if (kVariants[v].pack) return v;
+      if (first < 0) first = v;
+    }
+  return first;
+}
+// 2 x 32 packed (9 coordinates: 4 x 27 packed), then the smaller packed shape
+// for traces too long to leave it room.
+int search_variant_default(int dim, int k) {
+  static const int pref18[] = {9, 8, -1}, pref9[] = {12, -1};
+  return dim == 9 ? pref9[k] : pref18[k];
 }
 
 template <int G, int N, int NG, int MINB, bool LEAN, bool PACK>

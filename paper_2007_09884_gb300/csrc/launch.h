@@ -54,6 +54,8 @@ cudaError_t launch_score(const float* opc, int m, const DevSac* sac, int L, cons
 // dynamic shared memory per block.
 int search_variant_count();
 int search_variant_g(int v);
+int search_variant_groups(int v);
+int search_variant_default(int dim, int k);   // k-th preferred variant of an untuned search, or -1
 int search_variant_dim(int v);
 int search_variant_minb(int v);
 int search_variant_lean(int v);
