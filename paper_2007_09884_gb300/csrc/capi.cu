@@ -986,7 +986,7 @@ extern "C" int opmm_refine_batch(opmm_ctx* ctx, const opmm_saccade* sacs, int32_
   DevBuf& b_start = ctx->scratch[8];
   DevBuf& b_rows = ctx->scratch[9];
   DevBuf& b_out = ctx->scratch[10];
-  const size_t rows = (size_t)n * (2 * (size_t)p.dim + 2) * (size_t)p.lcap;
+  const size_t rows = (size_t)n * (2 * (size_t)p.dim + 2) * ((size_t)p.lcap + 1);
   TRY(b_start.ensure(sizeof(float) * OPMM_NPARAM * (size_t)n));
   TRY(b_rows.ensure(sizeof(float) * rows));
   TRY(b_out.ensure(sizeof(opmm_fit_result) * (size_t)n));

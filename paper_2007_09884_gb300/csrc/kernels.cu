@@ -1459,6 +1459,11 @@ __global__ void __launch_bounds__(32) k_finalize(const DevSac* sacs, const float
 // scratch area in global memory.
 constexpr int kRefineThreads = 64;
 
+// Floats between trajectory rows: an odd number, so that threads that write
+// one row each, sample by sample, and dot products that read the same sample
+// of many rows, stay on distinct shared-memory banks.
+__host__ __device__ constexpr int refine_pitch(int lcap) { return lcap + 1; }   // lcap is a multiple of 4
+
 struct RowSink {
   float* out;
   __device__ __forceinline__ void emit(int k, float dth) { out[k] = dth; }
@@ -1473,7 +1478,7 @@ __device__ bool refine_row(const float (&p)[kNumParams], const SacConst& sc, flo
   const int kend = min(sc.onset, sc.L - 1);
   for (int k = 0; k <= kend; ++k) row[k] = sc.th0 - sc.thf;
   RowSink s{row};
-  return walk(p, sc, s, qs, kRefineThreads, true, pe) >= 0;
+  return walk<RowSink, false, true>(p, sc, s, qs, kRefineThreads, true, pe) >= 0;
 }
 
 template <int N>
@@ -1534,8 +1539,9 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(const DevSac* sacs, c
   float* qslot = z + lcap;                                  // kQSlotFloats x kRefineThreads
   const int b = blockIdx.x, tid = threadIdx.x;
   const DevSac d = sacs[b];
+  const int pitch = refine_pitch(lcap);
   float* rows = rows_in_smem ? qslot + kQSlotFloats * kRefineThreads
-                             : scratch + (size_t)b * (2 * N + 2) * (size_t)lcap;
+                             : scratch + (size_t)b * (2 * N + 2) * (size_t)pitch;
   if (tid == 0) {
     mbar_init(&S.bar, 1);
     fence_mbar_init();
@@ -1567,7 +1573,7 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(const DevSac* sacs, c
   }
   __syncthreads();
   const SacConst sc = S.sc;
-  float* rcur[2] = {rows + (size_t)(2 * N) * lcap, rows + (size_t)(2 * N + 1) * lcap};
+  float* rcur[2] = {rows + (size_t)(2 * N) * pitch, rows + (size_t)(2 * N + 1) * pitch};
   if (tid == 0) {
     float p[kNumParams];
     u_to_p<N>(S.u, S.pc, lnlo, lnhi, p);
@@ -1595,51 +1601,69 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(const DevSac* sacs, c
         float p[kNumParams];
         u_to_p<N>(ut, S.pc, lnlo, lnhi, p);
         int pe = 0;
-        S.bad[tid] = refine_row(p, sc, rows + (size_t)tid * lcap, &pe, qslot + tid) ? 0 : 1;
+        S.bad[tid] = refine_row(p, sc, rows + (size_t)tid * pitch, &pe, qslot + tid) ? 0 : 1;
         if (pe) atomicAdd(&S.pe, 1);
       }
       __syncthreads();
-      // A (lower triangle) and g: one task per entry, FP64
-      constexpr int kTasks = N * (N + 1) / 2 + N;
       // J columns in place of the plus rows (FP32); the products below sum
       // with compensation in FP32 (the GPU's FP64 rate is a small fraction of
       // its FP32 rate) and enter the FP64 solve
       const float inv2d = 1.0f / (2.0f * delta);
-      for (int e = tid; e < N * sc.L; e += kRefineThreads) {
-        const int j = e / sc.L, k = e - j * sc.L;
-        float* jp = rows + (size_t)(2 * j) * lcap;
-        jp[k] = (jp[k] - rows[(size_t)(2 * j + 1) * lcap + k]) * inv2d;
+      for (int k = tid; k < sc.L; k += kRefineThreads) {
+#pragma unroll 6
+        for (int j = 0; j < N; ++j) {
+          float* jp = rows + (size_t)(2 * j) * pitch + k;
+          *jp = (*jp - jp[pitch]) * inv2d;
+        }
       }
       __syncthreads();
-      for (int t = tid; t < kTasks; t += kRefineThreads) {
-        int a, bb;
-        const bool is_g = t >= N * (N + 1) / 2;
-        if (is_g) {
-          a = t - N * (N + 1) / 2;
-          bb = -1;
+      // A (lower triangle) and g: one compensated dot product per entry.  A
+      // thread runs its kTasksPer entries side by side: each sum is a chain of
+      // four dependent additions per sample, so one alone leaves the SM idle.
+      constexpr int kTasks = N * (N + 1) / 2 + N;
+      constexpr int kTasksPer = (kTasks + kRefineThreads - 1) / kRefineThreads;
+      const float* ja[kTasksPer];
+      const float* jb[kTasksPer];
+      int ea[kTasksPer], eb[kTasksPer];   // entry (a, b); b = -1: g[a]; a = -1: none
+      float sum[kTasksPer], c[kTasksPer];
+#pragma unroll
+      for (int q = 0; q < kTasksPer; ++q) {
+        const int t = tid + q * kRefineThreads;
+        int a = -1, bb = -1;
+        if (t >= N * (N + 1) / 2) {
+          a = t < kTasks ? t - N * (N + 1) / 2 : -1;
         } else {
           a = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
           while ((a + 1) * (a + 2) / 2 <= t) ++a;
           while (a * (a + 1) / 2 > t) --a;
           bb = t - a * (a + 1) / 2;
         }
+        ea[q] = a;
+        eb[q] = bb;
+        ja[q] = rows + (size_t)(a < 0 ? 0 : 2 * a) * pitch;
+        jb[q] = bb < 0 ? r0 : rows + (size_t)(2 * bb) * pitch;
+        sum[q] = c[q] = 0.0f;
+      }
+#pragma unroll 2
+      for (int k = 0; k < sc.L; ++k) {
+        const float zk = z[k];
+#pragma unroll
+        for (int q = 0; q < kTasksPer; ++q) {
+          const float bk = jb[q][k];
+          const float y = fmaf(ja[q][k], eb[q] < 0 ? bk - zk : bk, -c[q]);
+          const float tt = sum[q] + y;
+          c[q] = (tt - sum[q]) - y;
+          sum[q] = tt;
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kTasksPer; ++q) {
+        const int a = ea[q], bb = eb[q];
+        if (a < 0) continue;
         const bool za = S.bad[2 * a] || S.bad[2 * a + 1];
         const bool zb = bb >= 0 && (S.bad[2 * bb] || S.bad[2 * bb + 1]);
-        double acc = 0.0;
-        if (!za && !zb) {
-          const float* ja = rows + (size_t)(2 * a) * lcap;
-          const float* jb = is_g ? r0 : rows + (size_t)(2 * bb) * lcap;
-          float sum = 0.0f, c = 0.0f;
-          for (int k = 0; k < sc.L; ++k) {
-            const float other = is_g ? jb[k] - z[k] : jb[k];
-            const float y = fmaf(ja[k], other, -c);
-            const float tt = sum + y;
-            c = (tt - sum) - y;
-            sum = tt;
-          }
-          acc = (double)sum - (double)c;
-        }
-        if (is_g) S.g[a] = acc;
+        const double acc = za || zb ? 0.0 : (double)sum[q] - (double)c[q];
+        if (bb < 0) S.g[a] = acc;
         else S.A[a * N + bb] = S.A[bb * N + a] = acc;
       }
       __syncthreads();
@@ -1649,15 +1673,17 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(const DevSac* sacs, c
       }
     }
     // damped normal equations in FP64 by warp 0: the Cholesky factor column by
-    // column (every lane forms the diagonal, the rows below go over the lanes,
-    // multiplied by the diagonal's reciprocal), then lane 0 substitutes and
-    // simulates the trial point
+    // column, each column's products leaving the trailing matrix at once,
+    // spread over the lanes (every entry subtracts them in column order, as a
+    // row-by-row factorisation does, without its chain of up to N dependent
+    // FP64 operations per column); forward substitution one row per lane; then
+    // lane 0 substitutes back and simulates the trial point
     if (tid < 32) {
       double amax = 0.0;
       for (int j = 0; j < N; ++j) amax = S.A[j * N + j] > amax ? S.A[j * N + j] : amax;
       int go = amax > 0.0 ? 1 : 0;
       double* M = S.M;
-      double* du = S.du;
+      double fwd = 0.0;   // lane i: row i of the forward substitution
       if (go) {
         for (int e = tid; e < N * N; e += 32) M[e] = S.A[e];
         __syncwarp();
@@ -1667,8 +1693,7 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(const DevSac* sacs, c
         }
         __syncwarp();
         for (int j = 0; j < N; ++j) {
-          double sjj = M[j * N + j];
-          for (int k = 0; k < j; ++k) sjj -= M[j * N + k] * M[j * N + k];
+          const double sjj = M[j * N + j];
           if (!(sjj > 0.0)) {
             go = 0;
             break;
@@ -1679,22 +1704,32 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(const DevSac* sacs, c
             M[j * N + j] = ljj;
             S.inv[j] = il;
           }
-          for (int i = j + 1 + tid; i < N; i += 32) {
-            double t = M[i * N + j];
-            for (int k = 0; k < j; ++k) t -= M[i * N + k] * M[j * N + k];
-            M[i * N + j] = t * il;
+          if (j + 1 + tid < N) M[(j + 1 + tid) * N + j] *= il;
+          __syncwarp();
+          for (int i0 = j + 1; i0 < N; i0 += 2) {
+            const int i = i0 + (tid >> 4);
+            if (i < N)
+              for (int k = j + 1 + (tid & 15); k <= i; k += 16) M[i * N + k] -= M[i * N + j] * M[k * N + j];
           }
           __syncwarp();
         }
       }
-      if (go && tid == 0) {
-        for (int i = 0; i < N; ++i) {
-          double t = -S.g[i];
-          for (int k = 0; k < i; ++k) t -= M[i * N + k] * du[k];
-          du[i] = t * S.inv[i];
+      if (go) {
+        double t = tid < N ? -S.g[tid] : 0.0;
+        for (int k = 0; k < N; ++k) {
+          const double dk = __shfl_sync(0xffffffffu, t * S.inv[tid < N ? tid : 0], k);
+          if (tid == k) fwd = dk;
+          if (tid > k && tid < N) t -= M[tid * N + k] * dk;
         }
+        if (tid < N) S.du[tid] = fwd;
+        __syncwarp();
+      }
+      if (go && tid == 0) {
+        double du[N];
+#pragma unroll
         for (int i = N - 1; i >= 0; --i) {
-          double t = du[i];
+          double t = S.du[i];
+#pragma unroll
           for (int k = i + 1; k < N; ++k) t -= M[k * N + i] * du[k];
           du[i] = t * S.inv[i];
         }
@@ -1798,7 +1833,7 @@ cudaError_t launch_refine(int dim, const DevSac* sacs, const float* traces, cons
   if (n <= 0) return cudaSuccess;
   // the trajectory rows go to shared memory when they fit in 96 KB (windows up
   // to about 600 samples with 18 coordinates), leaving room for two blocks
-  const size_t rows_bytes = (2 * (size_t)dim + 2) * (size_t)lcap * sizeof(float);
+  const size_t rows_bytes = (2 * (size_t)dim + 2) * (size_t)refine_pitch(lcap) * sizeof(float);
   const int in_smem = rows_bytes <= (size_t)96 * 1024 ? 1 : 0;
   const size_t smem = 2 * (size_t)lcap * sizeof(float) + (size_t)kQSlotFloats * kRefineThreads * sizeof(float) +
                       (in_smem ? rows_bytes : 0);

@@ -72,7 +72,7 @@ cudaError_t launch_finalize(const DevSac* sacs, const float* traces, const float
                             opmm_fit_result* out, cudaStream_t st, const int* list = nullptr, int dim = 18);
 
 // Levenberg-Marquardt refinement of n saccades (dim 18 or 9); scratch holds
-// n * (2 dim + 2) * lcap floats.
+// n * (2 dim + 2) * (lcap + 1) floats.
 cudaError_t launch_refine(int dim, const DevSac* sacs, const float* traces, const float* pcs, const float* start,
                           int n, int K, float lnlo, float lnhi, float delta, float lambda0, int lcap, float* scratch,
                           opmm_fit_result* out, unsigned* err, cudaStream_t st);
