@@ -490,12 +490,47 @@ Status enqueue_fit(opmm_plan* p, cudaStream_t st) {
 // decision's latency first, the SM's throughput from about 24 chunks on.
 static double unit_step(int chunks) { return std::max(21.0 + 1.5 * chunks, 5.0 + 2.18 * chunks); }
 
+// Units per saccade: the number of units that n saccades' S simplices are
+// split into evenly, at most G simplices each, or 0 for full units of G and a
+// last one with the rest.  The split with the least turns of the blocks times
+// the step of one unit: a batch with many units per block keeps its units as
+// large as they come (a simplex costs 1.6 k cycles a step in a unit of 64 and
+// 2.5 k in one of 16), a few saccades are spread over every SM (one saccade
+// of 186 simplices: 93 units of two instead of 6 of 32).  A simplex evolves
+// the same in any unit, so the results do not depend on the split.
+static int split_units(int n, int S, int variant, int blocks) {
+  const int G = search_variant_g(variant), NG = search_variant_groups(variant);
+  const int nt = search_variant_dim(variant) + 4;
+  auto step = [&](int m) {   // one step of a unit of m simplices in NG even groups
+    int chunks = 0;
+    for (int h = 0; h < NG; ++h) chunks += (nt * ((m * (h + 1)) / NG - (m * h) / NG) + 31) / 32;
+    return unit_step(chunks);
+  };
+  auto turns = [&](int ng) { return std::max(1.0, (double)(((long long)n * ng + blocks - 1) / blocks)); };
+  const int least = (S + G - 1) / G;
+  double best = 1e300;
+  int pick = least;
+  for (int ng = least; ng <= S; ++ng) {
+    const double t = turns(ng) * step((S + ng - 1) / ng);
+    if (t < best * 0.999) {
+      best = t;
+      pick = ng;
+    }
+  }
+  // with many units per saccade an even split only rounds every group up to
+  // whole chunks, and full units lose only in their last one
+  return pick == least && (S % G == 0 || least > 8) ? 0 : pick;
+}
+
 // Candidate launch shapes: the search kernel's variants (simplices per block G,
 // threads = 22 G rounded to warps, register bound for MINB resident blocks) at
-// the occupancy the device allows for this trace capacity.  Returns (variant,
-// blocks per SM) pairs.
-static std::vector<std::pair<int, int>> shape_candidates(int lcap, int dim) {
-  std::vector<std::pair<int, int>> out;
+// the occupancy the device allows for this trace capacity, without the shapes
+// of more than 32 simplices where the split of these n saccades leaves every
+// unit at 32 or less (a smaller shape runs those units just as fast: 53.1
+// against 53.2 k cycles a step at 32 simplices).  Returns (variant, blocks per
+// SM) pairs.
+static std::vector<std::pair<int, int>> shape_candidates(int lcap, int dim, int n, int S, int num_sms) {
+  std::vector<std::pair<int, int>> out, small;
   for (int v = 0; v < search_variant_count(); ++v) {
     if (search_variant_dim(v) != dim) continue;
     int bps = 0;
@@ -503,9 +538,12 @@ static std::vector<std::pair<int, int>> shape_candidates(int lcap, int dim) {
       cudaGetLastError();
       continue;
     }
-    if (bps >= 1) out.push_back({v, bps});
+    if (bps < 1) continue;
+    out.push_back({v, bps});
+    const int G = search_variant_g(v), ng = split_units(n, S, v, num_sms * bps);
+    if (G <= 32 || ng == 0 || (S + ng - 1) / ng > 32) small.push_back({v, bps});
   }
-  return out;
+  return small.empty() ? out : small;
 }
 
 // Project-written autotuner: time each candidate shape on a sample of this
@@ -525,15 +563,17 @@ static Status autotune(opmm_plan* p) {
   const auto key = std::make_tuple(p->lcap, p->S, p->n >= 64 ? 64 : p->n,
                                    std::min(p->opts.iterations, 32) * 64 + (p->dim << 1));
   auto it = ctx->tune_cache.find(key);
-  auto cands = shape_candidates(p->lcap, p->dim);
+  auto cands = shape_candidates(p->lcap, p->dim, p->n, p->S, ctx->num_sms);
   if (cands.empty()) return Status(OPMM_ECUDA, "no launchable search shape (shared memory)");
   if (ctx->forced_variant >= 0) {
-    for (auto& cd : cands)
-      if (cd.first == ctx->forced_variant) {
-        p->variant = cd.first;
-        p->blocks_per_sm = cd.second;
-        return Status();
-      }
+    int bps = 0;
+    if (search_variant_dim(ctx->forced_variant) == p->dim &&
+        search_occupancy_v(ctx->forced_variant, p->lcap, &bps) == cudaSuccess && bps >= 1) {
+      p->variant = ctx->forced_variant;
+      p->blocks_per_sm = bps;
+      return Status();
+    }
+    cudaGetLastError();
     return Status(OPMM_EINVAL, "forced search variant cannot be launched with this batch or model");
   }
   if (it != ctx->tune_cache.end()) {
@@ -571,8 +611,8 @@ static Status autotune(opmm_plan* p) {
   const long long want = std::max(1LL, (kProbeSimplices + p->S - 1) / std::max(1, p->S));
   const int stride = (int)std::max(1LL, (long long)p->n / want);
   for (auto& c : cands) {
-    // the unit list depends on G: rebuild it (the probe's sample) for the probe
-    s = build_units(p, search_variant_g(c.first), stride);
+    // the unit list depends on the shape: rebuild it (the probe's sample) for the probe
+    s = build_units(p, c.first, c.second, stride);
     if (!s.ok()) break;
     SearchParams P = p->params;
     P.T = std::min(p->opts.iterations, kProbeIters);
@@ -602,46 +642,15 @@ static Status autotune(opmm_plan* p) {
   return Status();
 }
 
-// Units per saccade: the number of units that n saccades' S simplices are
-// split into evenly, at most G simplices each, or 0 for full units of G and a
-// last one with the rest.  The split with the least turns of the blocks times
-// the step of one unit: a batch with many units per block keeps its units as
-// large as they come (a simplex costs 1.6 k cycles a step in a unit of 64 and
-// 2.5 k in one of 16), a few saccades are spread over every SM (one saccade
-// of 186 simplices: 93 units of two instead of 6 of 32).  A simplex evolves
-// the same in any unit, so the results do not depend on the split.
-static int split_units(int n, int S, int variant, int blocks) {
-  const int G = search_variant_g(variant), NG = search_variant_groups(variant);
-  const int nt = search_variant_dim(variant) + 4;
-  auto step = [&](int m) {   // one step of a unit of m simplices in NG even groups
-    int chunks = 0;
-    for (int h = 0; h < NG; ++h) chunks += (nt * ((m * (h + 1)) / NG - (m * h) / NG) + 31) / 32;
-    return unit_step(chunks);
-  };
-  auto turns = [&](int ng) { return std::max(1.0, (double)(((long long)n * ng + blocks - 1) / blocks)); };
-  const int least = (S + G - 1) / G;
-  double best = 1e300;
-  int pick = least;
-  for (int ng = least; ng <= S; ++ng) {
-    const double t = turns(ng) * step((S + ng - 1) / ng);
-    if (t < best * 0.999) {
-      best = t;
-      pick = ng;
-    }
-  }
-  // with many units per saccade an even split only rounds every group up to
-  // whole chunks, and full units lose only in their last one
-  return pick == least && (S % G == 0 || least > 8) ? 0 : pick;
-}
-
-// Unit list for G simplices per block: saccades in decreasing order of work
-// (samples after onset), each split into units by split_units (a probe: into
-// full units).
+// Unit list for a search variant: saccades in decreasing order of work
+// (samples after onset), each split into units by split_units (a sampled
+// probe: into full units).
 // With probe_stride k > 1, the autotuner's sample: only the saccades at
 // positions k/2, k/2 + k, ... of that order (the unit starts are then not
 // meaningful; no result is read from a probe).
-Status build_units(opmm_plan* p, int G, int probe_stride) {
-  const int even = probe_stride > 1 ? 0 : split_units(p->n, p->S, p->variant, p->ctx->num_sms * p->blocks_per_sm);
+Status build_units(opmm_plan* p, int variant, int blocks_per_sm, int probe_stride) {
+  const int G = search_variant_g(variant);
+  const int even = probe_stride > 1 ? 0 : split_units(p->n, p->S, variant, p->ctx->num_sms * blocks_per_sm);
   p->ngroups = even ? even : (p->S + G - 1) / G;
   const size_t nu = (size_t)p->n * (size_t)p->ngroups;
   if (nu > (size_t)0x7fffffff) return Status(OPMM_EINVAL, "too many work units");
@@ -794,7 +803,7 @@ Status plan_build(opmm_ctx* ctx, const opmm_saccade* sacs, int32_t n, const opmm
   s = autotune(p);
   if (!s.ok()) return s;
   p->G = search_variant_g(p->variant);
-  s = build_units(p, p->G);
+  s = build_units(p, p->variant, p->blocks_per_sm);
   if (!s.ok()) return s;
   p->threads = search_variant_threads(p->variant);
   s = cuda_status(cudaEventCreate(&p->ev_search[0]), "event");

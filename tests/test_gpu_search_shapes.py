@@ -55,6 +55,20 @@ def test_results_do_not_depend_on_the_split(ctx, items, model, simplices, n):
             G.opmm_set_search_variant(ctx, -1)
 
 
+# small batches whose probes run every saccade, on each shape's own units
+@pytest.mark.parametrize("model,simplices", [(18, 1), (18, 17), (18, 33), (18, 70), (18, 300), (9, 40), (9, 300)])
+def test_tuned_plan_equals_the_one_shot_fit(ctx, items, model, simplices):
+    batch = to_batch(items)
+    kw = dict(candidates=simplices * (model + 4), iterations=5, seed=3, model=model, init_opc=centres(items))
+    plan = G.opmm_plan_create(ctx, batch, **kw)
+    try:
+        got = plan.execute()
+        if all(t["walk"] != "lean" or t["variant"] != plan.info()["variant"] for t in plan.tuning()):
+            _same(got, G.opmm_fit_batch(ctx, batch, **kw))
+    finally:
+        plan.destroy()
+
+
 # windows that end at the onset, that hold 1, 31, 32, 33, 64 and 65 samples after it, pulses shorter than a sample,
 # ending on a block's edge and outlasting the window, and a vector whose substeps are refined
 @pytest.mark.parametrize("fs,after,width", [(1000.0, 0, 20.0), (1000.0, 1, 20.0), (1000.0, 1, 0.3), (1000.0, 31, 16.05),
