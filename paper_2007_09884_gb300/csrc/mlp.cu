@@ -5,22 +5,22 @@
 // 5th-generation tensor cores:
 //
 //   k_gemm_tn   D = A . B^T for up to four same-shape problems per launch
-//               (each optionally split into K slices), BF16 operands, FP32
-//               accumulate: a producer warp streams 128 x 64 tiles of A and
-//               BN x 64 tiles of B into a shared-memory ring with TMA
+//               (each optionally split into K slices), BF16 operands stored
+//               along K or across it, FP32 accumulate: a producer warp
+//               streams 128 x 64 tiles of A and BN x 64 tiles of B into a
+//               shared-memory ring with TMA
 //               (cp.async.bulk.tensor, 128-byte swizzle), one thread of the
 //               MMA warp issues tcgen05.mma (M = 128, N = BN, K = 16) into a
 //               TMEM accumulator and frees each stage with tcgen05.commit,
 //               and 8 or 16 epilogue warps read the accumulator with
-//               tcgen05.ld, apply the epilogue (bias + GELU with Z and H^T;
-//               GELU' with the rounded error, its transpose and bias-gradient
-//               column sums; plain FP32) and stage the tile for bulk tensor
-//               stores.
+//               tcgen05.ld, apply the epilogue (bias + GELU with Z; GELU'
+//               with the rounded error and bias-gradient column sums; plain
+//               FP32) and stage the tile for bulk tensor stores.
 //
 // Around it: the training head (output layer, loss, the layer-3 error, the
 // output layer's gradient partials), the gradient assembly fused with AdamW,
-// the transposes of the BF16 weights, the inference head, the on-device
-// training data generator and the featurizer.
+// the inference head, the on-device training data generator and the
+// featurizer.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -133,10 +133,24 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
   return d;
 }
 
+// The same for a tile stored across K (MN-major, one row of 64 BF16 per K
+// index): boxes of [64 K rows][64 columns], 8-row groups 1024 B apart (stride
+// byte offset), the next 64 columns one box further (leading byte offset).
+__device__ __forceinline__ uint64_t sw128_desc_mn(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
+  d |= (uint64_t)((uint32_t)kMnBoxBytes >> 4) << 16;
+  d |= (uint64_t)(1024u >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
+  return d;
+}
+
 // Instruction descriptor of tcgen05.mma.kind::f16: FP32 accumulator, BF16 A
-// and B, both K-major, N >> 3 and M >> 4.
-__host__ __device__ constexpr uint32_t f16_idesc(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+// and B, each K-major or (amn, bmn) MN-major, N >> 3 and M >> 4.
+__host__ __device__ constexpr uint32_t f16_idesc(int M, int N, bool amn, bool bmn) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((amn ? 1u : 0u) << 15) | ((bmn ? 1u : 0u) << 16) |
+         ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 // The Gaussian CDF Phi(z) = (1 + erf(z / sqrt 2)) / 2 with erf from
@@ -169,19 +183,18 @@ __device__ __forceinline__ float gelu_grad(float z) {
 
 // ------------------------------------------------------------------ GEMM
 // Tensor maps of a grouped launch: A and B of each problem, and its outputs
-// (FP32 in 32-column boxes, BF16 row-major and transposed in 64-column
-// boxes, all 128 rows high with the 128-byte swizzle).
+// (FP32 in 32-column boxes, BF16 in 64-column boxes, 128 rows high with the
+// 128-byte swizzle).
 struct GemmMaps {
   CUtensorMap a[kMaxGroup];
   CUtensorMap b[kMaxGroup];
   CUtensorMap of[kMaxGroup];
   CUtensorMap ob[kMaxGroup];
-  CUtensorMap ot[kMaxGroup];
 };
 
 // The launch's shape and the problems' outputs, as the kernel sees them.
 struct GemmArgs {
-  int M, N, nkb, ksplit, ldo, ldt;     // nkb: 64-wide K blocks per slice
+  int M, N, nkb, ksplit, ldo;          // nkb: 64-wide K blocks per slice
   long long zstride;
   unsigned* err;
   GemmProblem p[kMaxGroup];
@@ -207,19 +220,23 @@ __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"
 // CTAs per SM).  Staging, as the 128-byte swizzle of the tensor maps lays a
 // box out (row q of a box at 128 q bytes, its 16-byte chunk c at position
 // c ^ (q & 7)): Sf, BN / 32 FP32 boxes of [128 rows][32 columns] at 0; Sbf,
-// two BF16 boxes of [128 rows][64 columns] at 64 KB; St, the transpose, two
-// BF16 boxes of [128 columns][64 rows] at 96 KB.  The swizzle also puts the
+// two BF16 boxes of [128 rows][64 columns] at 64 KB.  The swizzle also puts the
 // 32 rows of a warp that write one logical chunk on distinct banks.  Every
 // wait is bounded; a wait that expires raises the error word and the tile's
 // output is not written.
-template <int STAGES, int EPI, int BN>
+// AMN, BMN: the operand is stored across K ([K][M] or [K][N] row-major) and
+// its tile arrives in boxes of 64 columns, which the MMA reads as MN-major.
+// So the weight gradients dZ^T . H read the row-major errors and activations,
+// and the error GEMMs the row-major weights: no pass of a training step
+// writes a transpose.
+template <int STAGES, int EPI, int BN, bool AMN, bool BMN>
 __global__ void __launch_bounds__(gemm_threads(STAGES), STAGES <= 3 ? 2 : 1)
     k_gemm_tn(const __grid_constant__ GemmMaps maps, const __grid_constant__ GemmArgs g) {
   constexpr int EW = gemm_epi_warps(STAGES), ET = EW * 32, NC = BN * 4 / EW;
   constexpr int kTmaWarp = EW, kMmaWarp = EW + 1;
   constexpr int kStageBytes = stage_bytes(BN);
   static_assert(EPI == kEpiF32 || BN == 128, "the BF16 epilogues take 128-wide tiles");
-  static_assert(STAGES * kStageBytes >= (EPI == kEpiF32 ? kBM * BN * 4 : 131072),
+  static_assert(STAGES * kStageBytes >= (EPI == kEpiF32 ? kBM * BN * 4 : 98304),
                 "the epilogue stages its tile in the ring");
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -264,14 +281,26 @@ __global__ void __launch_bounds__(gemm_threads(STAGES), STAGES <= 3 ? 2 : 1)
         }
         unsigned char* st = sm + s * kStageBytes;
         mbar_arrive_expect_tx(&full[s], kStageBytes);
-        tma_load_2d(st, ma, (kb0 + kb) * kBK, tm * kBM, &full[s]);
-        tma_load_2d(st + kTileABytes, mb, (kb0 + kb) * kBK, tn * BN, &full[s]);
+        const int k = (kb0 + kb) * kBK;
+        if constexpr (AMN) {
+#pragma unroll
+          for (int bx = 0; bx < kBM / 64; ++bx) tma_load_2d(st + bx * kMnBoxBytes, ma, tm * kBM + 64 * bx, k, &full[s]);
+        } else {
+          tma_load_2d(st, ma, k, tm * kBM, &full[s]);
+        }
+        if constexpr (BMN) {
+#pragma unroll
+          for (int bx = 0; bx < BN / 64; ++bx)
+            tma_load_2d(st + kTileABytes + bx * kMnBoxBytes, mb, tn * BN + 64 * bx, k, &full[s]);
+        } else {
+          tma_load_2d(st + kTileABytes, mb, k, tn * BN, &full[s]);
+        }
       }
     }
   } else if (warp == kMmaWarp) {
     if (lane == 0) {
       // MMA issuer
-      constexpr uint32_t idesc = f16_idesc(kBM, BN);
+      constexpr uint32_t idesc = f16_idesc(kBM, BN, AMN, BMN);
       for (int kb = 0; kb < nk; ++kb) {
         const int s = kb % STAGES;
         const uint32_t use = (uint32_t)(kb / STAGES);
@@ -285,7 +314,8 @@ __global__ void __launch_bounds__(gemm_threads(STAGES), STAGES <= 3 ? 2 : 1)
         const uint32_t b0 = a0 + kTileABytes;
 #pragma unroll
         for (int k = 0; k < kBK / 16; ++k)
-          tc_mma(tmem, sw128_desc(a0 + k * 32), sw128_desc(b0 + k * 32), idesc, (kb | k) != 0 ? 1u : 0u);
+          tc_mma(tmem, AMN ? sw128_desc_mn(a0 + k * 2048) : sw128_desc(a0 + k * 32),
+                 BMN ? sw128_desc_mn(b0 + k * 2048) : sw128_desc(b0 + k * 32), idesc, (kb | k) != 0 ? 1u : 0u);
         tc_commit(&empty[s]);
       }
       tc_commit(done);
@@ -328,9 +358,7 @@ __global__ void __launch_bounds__(gemm_threads(STAGES), STAGES <= 3 ? 2 : 1)
     const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16);
     unsigned char* Sf = sm;                      // BN / 32 boxes [128][32] FP32
     unsigned char* Sbf = sm + 65536;             // 2 boxes [128][64] BF16
-    unsigned char* St = sm + 98304;              // 2 boxes [128 columns][64 rows] BF16
     const bool want_f32 = EPI == kEpiF32 || (EPI == kEpiBiasGelu && P.out_f32 != nullptr);
-    const bool want_t = EPI != kEpiF32 && P.out_t != nullptr;
     const int sw = r & 7;
     if (go) {
       float v[NC];
@@ -368,17 +396,6 @@ __global__ void __launch_bounds__(gemm_threads(STAGES), STAGES <= 3 ? 2 : 1)
             *reinterpret_cast<uint4*>(Sbf + (cc >> 6) * 16384 + r * 128 + ((((cc & 63) >> 3) ^ sw) << 4)) =
                 *reinterpret_cast<const uint4*>(&h[4 * j]);
           }
-          if (want_t) {
-            // element (row r, column cc): box r / 64, box row cc, chunk (r % 64) / 8
-            unsigned char* tb = St + (r >> 6) * 16384 + (r & 7) * 2;
-            const int rc = (r & 63) >> 3;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const int c0 = col0 + 2 * i, c1 = c0 + 1;
-              *reinterpret_cast<__nv_bfloat16*>(tb + c0 * 128 + ((rc ^ (c0 & 7)) << 4)) = h[i].x;
-              *reinterpret_cast<__nv_bfloat16*>(tb + c1 * 128 + ((rc ^ (c1 & 7)) << 4)) = h[i].y;
-            }
-          }
         }
       }
     }
@@ -396,8 +413,6 @@ __global__ void __launch_bounds__(gemm_threads(STAGES), STAGES <= 3 ? 2 : 1)
         }
         if constexpr (EPI != kEpiF32) {
           for (int bx = 0; bx < 2; ++bx) tma_store_2d(&maps.ob[prob], x0 + 64 * bx, y0, Sbf + bx * 16384);
-          if (want_t)
-            for (int bx = 0; bx < 2; ++bx) tma_store_2d(&maps.ot[prob], y0 + 64 * bx, x0, St + bx * 16384);
         }
         bulk_commit();
       }
@@ -407,6 +422,7 @@ __global__ void __launch_bounds__(gemm_threads(STAGES), STAGES <= 3 ? 2 : 1)
           const unsigned char* cbp = Sbf + (tid >> 6) * 16384 + (tid & 7) * 2;
           const int ch = (tid & 63) >> 3;
           float s = 0.0f;
+#pragma unroll 16
           for (int rr = 0; rr < 128; ++rr)
             s += __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(cbp + rr * 128 + ((ch ^ (rr & 7)) << 4)));
           P.colpart[(size_t)tm * g.N + x0 + tid] = s;
@@ -423,22 +439,6 @@ __global__ void __launch_bounds__(gemm_threads(STAGES), STAGES <= 3 ? 2 : 1)
 }
 
 // ------------------------------------------------------------------ elementwise / reductions
-// Transposes of the hidden weight matrices: wt_l = wb_l^T for the four
-// 512 x 512 BF16 matrices (blockIdx.z = layer), through a 32 x 32 tile.
-// When step_idx is given (the step index of a replayed training sequence),
-// one thread advances it: this kernel follows the step's AdamW, the last
-// reader of the index.
-__global__ void k_transpose_layers(const __nv_bfloat16* wb, __nv_bfloat16* wt, int* step_idx) {
-  if (step_idx && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0 && threadIdx.y == 0)
-    *step_idx += 1;
-  __shared__ __nv_bfloat16 t[32][34];
-  const size_t lo = (size_t)blockIdx.z * kHidden * kHidden;
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) t[i][threadIdx.x] = wb[lo + (size_t)(r0 + i) * kHidden + c0 + threadIdx.x];
-  __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) wt[lo + (size_t)(c0 + i) * kHidden + r0 + threadIdx.x] = t[threadIdx.x][i];
-}
-
 // Output layer and loss: Y[m][o] = H[m] . W5[o] + b5[o] (o < 18, CUDA cores);
 // loss contribution and dY = 2 (Y - T) / (M * 18).  One warp per row.
 __global__ void k_head_fwd_loss(const __nv_bfloat16* H, const __nv_bfloat16* W5, const float* b5, const float* T, int M,
@@ -478,8 +478,7 @@ __global__ void k_head_fwd_loss(const __nv_bfloat16* H, const __nv_bfloat16* W5,
 // and dY = 2 (y - t) / (M 18); then per column k (one thread each): the
 // block's partial sums of dW5[o][k] = sum_m dY[m][o] H3[m][k] (and of db5 =
 // sum_m dY), dH3 = dY . W5 and the rounded layer-3 error dZ3 = BF16(dH3 *
-// GELU'(Z3)), written row-major and transposed (through shared memory, in
-// whole rows) with its column sums over the block's rows.  W5 (as FP32) and
+// GELU'(Z3)) with its column sums over the block's rows.  W5 (as FP32) and
 // the block's H3 rows are staged in shared memory; each thread's 32 Z3
 // values are loaded at the start, so their latency overlaps the forward
 // part.  Every sum runs in a fixed order.
@@ -495,8 +494,11 @@ constexpr size_t kHeadSmem = (size_t)kOut * kHidden * 4 + (size_t)kHeadRows * kH
 __global__ void __launch_bounds__(kHeadThreads) k_head_train(const __nv_bfloat16* H, const __nv_bfloat16* W5,
                                                              const float* b5, const float* T, const float* Z, int M,
                                                              float* Y, float* dY, float* row_loss, __nv_bfloat16* dZ,
-                                                             __nv_bfloat16* dZt, float* colpart, float* dWpart,
-                                                             float* dbpart) {
+                                                             float* colpart, float* dWpart, float* dbpart,
+                                                             int* step_idx) {
+  // the step index of a replayed training sequence advances here: the last
+  // step's AdamW, its only reader, is over, and this step's is to come
+  if (step_idx && blockIdx.x == 0 && threadIdx.x == 0) *step_idx += 1;
   extern __shared__ __align__(16) unsigned char hsm[];
   float* sw = reinterpret_cast<float*>(hsm);                                    // [18][512]
   __nv_bfloat16* sh = reinterpret_cast<__nv_bfloat16*>(sw + kOut * kHidden);   // [32][512]
@@ -628,19 +630,11 @@ __global__ void __launch_bounds__(kHeadThreads) k_head_train(const __nv_bfloat16
     dbpart[(size_t)blockIdx.x * kOut + tid] = s;
   }
   __syncthreads();
-  // dZ3 row-major (pairs of columns per thread), its transpose (8 rows of one
-  // column per 16-byte store) and the column sums
+  // dZ3 row-major (pairs of columns per thread) and the column sums
   for (int q = tid; q < kHeadRows * kHidden / 2; q += kHeadThreads) {
     const int i = q / (kHidden / 2), c2 = q - i * (kHidden / 2);
     *reinterpret_cast<__nv_bfloat162*>(dZ + (size_t)(r0 + i) * kHidden + 2 * c2) =
         *reinterpret_cast<const __nv_bfloat162*>(sdz + i * kSdzPitch + 2 * c2);
-  }
-  for (int q = tid; q < kHidden * (kHeadRows / 8); q += kHeadThreads) {
-    const int k = q / (kHeadRows / 8), part = q - k * (kHeadRows / 8);
-    __align__(16) __nv_bfloat16 v[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = sdz[(part * 8 + e) * kSdzPitch + k];
-    *reinterpret_cast<uint4*>(dZt + (size_t)k * M + r0 + part * 8) = *reinterpret_cast<const uint4*>(v);
   }
   {
     const int k = tid;
@@ -677,8 +671,7 @@ __device__ __forceinline__ void adamw_update(long long i, float gi, float* w, fl
 }
 
 // AdamW on the flat FP32 parameter vector with a given gradient; refreshes
-// the row-major BF16 working copies (their transposes follow from
-// k_transpose_layers).
+// the BF16 working copies.
 __global__ void k_adamw(float* w, const float* g, float* m1, float* m2, int n, float lr, float b1, float b2, float eps,
                         float wd, float bc1, float bc2, const AdamLayout L, __nv_bfloat16* wb) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -686,7 +679,7 @@ __global__ void k_adamw(float* w, const float* g, float* m1, float* m2, int n, f
   adamw_update(i, g[i], w, m1, m2, lr, b1, b2, eps, wd, bc1, bc2, L, wb);
 }
 
-// Refresh the row-major BF16 working copies from the FP32 master parameters.
+// Refresh the BF16 working copies from the FP32 master parameters.
 __global__ void k_pack_params(const float* w, int n, const AdamLayout L, __nv_bfloat16* wb) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -807,16 +800,13 @@ __global__ void __launch_bounds__(256) k_grad_finish(const __grid_constant__ Fin
 // Featurizer: resample the trace on a 1 ms grid from onset (256 points, linear
 // interpolation, held after the window end) in the positive frame, position
 // normalised by the amplitude (start fixation = 0, end fixation = 1) and
-// velocity as 10 x the per-millisecond difference.  Output BF16 [n][512]
-// and, optionally, its transpose [512][ldt].  A block of 4 warps takes 32
-// saccades (a warp per saccade at a time) and stages their features in shared
-// memory, then writes whole rows of X and, for each feature, the 32
-// saccades' values as 64 contiguous bytes of Xt.
+// velocity as 10 x the per-millisecond difference.  Output BF16 [n][512].
+// A block of 4 warps takes 32 saccades (a warp per saccade at a time) and
+// stages their features in shared memory, then writes whole rows of X.
 constexpr int kFeatRows = 32;
 constexpr int kSxPitch = kIn + 2;          // BF16 elements: rows one bank apart
 
-__global__ void __launch_bounds__(128) k_featurize(const DevSac* sacs, const float* traces, int n, __nv_bfloat16* X,
-                                                   __nv_bfloat16* Xt, int ldt) {
+__global__ void __launch_bounds__(128) k_featurize(const DevSac* sacs, const float* traces, int n, __nv_bfloat16* X) {
   __shared__ __align__(16) __nv_bfloat16 sx[kFeatRows * kSxPitch];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b0 = blockIdx.x * kFeatRows;
@@ -860,19 +850,6 @@ __global__ void __launch_bounds__(128) k_featurize(const DevSac* sacs, const flo
     const int i = q / (kIn / 2), c2 = q - i * (kIn / 2);
     *reinterpret_cast<__nv_bfloat162*>(X + (size_t)(b0 + i) * kIn + 2 * c2) =
         *reinterpret_cast<const __nv_bfloat162*>(sx + i * kSxPitch + 2 * c2);
-  }
-  if (Xt) {
-    for (int q = tid; q < kIn * (kFeatRows / 8); q += 128) {
-      const int k = q / (kFeatRows / 8), part = q - k * (kFeatRows / 8);
-      if (part * 8 + 8 <= nr) {
-        __align__(16) __nv_bfloat16 v[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = sx[(part * 8 + e) * kSxPitch + k];
-        *reinterpret_cast<uint4*>(Xt + (size_t)k * ldt + b0 + part * 8) = *reinterpret_cast<const uint4*>(v);
-      } else {
-        for (int e = 0; part * 8 + e < nr; ++e) Xt[(size_t)k * ldt + b0 + part * 8 + e] = sx[(part * 8 + e) * kSxPitch + k];
-      }
-    }
   }
 }
 
@@ -1007,8 +984,8 @@ static bool make_map_2d(CUtensorMap* map, const void* base, CUtensorMapDataType 
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// 2-D tensor map of a row-major BF16 matrix [rows][cols], box 64 x box_rows
-// (128-byte rows, 128-byte swizzle).
+// 2-D tensor map of a row-major BF16 matrix [rows][cols], box 64 columns x
+// box_rows (128-byte rows, 128-byte swizzle).
 static bool make_map(CUtensorMap* map, const void* base, int rows, int cols, int box_rows) {
   auto fn = encode_fn();
   if (!fn) return false;
@@ -1021,16 +998,16 @@ static bool make_map(CUtensorMap* map, const void* base, int rows, int cols, int
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int S, int E, int BN>
+template <int S, int E, int BN, bool AMN, bool BMN>
 static cudaError_t gemm_attr() {
-  return cudaFuncSetAttribute(k_gemm_tn<S, E, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(S, BN));
+  return cudaFuncSetAttribute(k_gemm_tn<S, E, BN, AMN, BMN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(S, BN));
 }
 
 cudaError_t gemm_prepare() {
-  cudaError_t e = gemm_attr<3, kEpiF32, 128>();
-  if (e == cudaSuccess) e = gemm_attr<6, kEpiBiasGelu, 128>();
-  if (e == cudaSuccess) e = gemm_attr<6, kEpiGeluBwd, 128>();
-  if (e == cudaSuccess) e = gemm_attr<4, kEpiF32, 256>();
+  cudaError_t e = gemm_attr<3, kEpiF32, 128, false, false>();
+  if (e == cudaSuccess) e = gemm_attr<6, kEpiBiasGelu, 128, false, false>();
+  if (e == cudaSuccess) e = gemm_attr<6, kEpiGeluBwd, 128, false, true>();
+  if (e == cudaSuccess) e = gemm_attr<4, kEpiF32, 256, true, true>();
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_head_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeadSmem);
   return e;
 }
@@ -1038,14 +1015,14 @@ cudaError_t gemm_prepare() {
 cudaError_t gemm(const GemmLaunch& L, cudaStream_t st) {
   if (L.np < 1 || L.np > kMaxGroup || L.ksplit < 1 || L.M <= 0 || L.N <= 0 || L.K <= 0) return cudaErrorInvalidValue;
   if (L.M % kBM || L.N % L.bn || L.K % (L.ksplit * kBK)) return cudaErrorInvalidValue;
-  // launchable (stages, epilogue, width): the epilogue's staging must fit the ring
-  const int kind = (L.stages == 3 && L.epi == kEpiF32 && L.bn == 128)        ? 0
-                   : (L.stages == 6 && L.epi == kEpiBiasGelu && L.bn == 128) ? 1
-                   : (L.stages == 6 && L.epi == kEpiGeluBwd && L.bn == 128)  ? 2
-                   : (L.stages == 4 && L.epi == kEpiF32 && L.bn == 256)      ? 3
-                                                                              : -1;
+  // launchable (stages, epilogue, width, operands): the epilogue's staging must fit the ring
+  const int kind = (L.stages == 3 && L.epi == kEpiF32 && L.bn == 128 && !L.amn && !L.bmn)        ? 0
+                   : (L.stages == 6 && L.epi == kEpiBiasGelu && L.bn == 128 && !L.amn && !L.bmn) ? 1
+                   : (L.stages == 6 && L.epi == kEpiGeluBwd && L.bn == 128 && !L.amn && L.bmn)   ? 2
+                   : (L.stages == 4 && L.epi == kEpiF32 && L.bn == 256 && L.amn && L.bmn)        ? 3
+                                                                                                  : -1;
   if (kind < 0) return cudaErrorInvalidValue;
-  if (L.ldo % 8 || (L.epi != kEpiF32 && L.ldt % 8)) return cudaErrorInvalidValue;
+  if (L.ldo % 8) return cudaErrorInvalidValue;
   if (L.ksplit > 1 && (L.epi != kEpiF32 || L.zstride != (long long)L.M * L.ldo)) return cudaErrorInvalidValue;
   GemmMaps maps;
   memset(&maps, 0, sizeof maps);
@@ -1057,19 +1034,17 @@ cudaError_t gemm(const GemmLaunch& L, cudaStream_t st) {
     const bool f32 = L.epi == kEpiF32 || (L.epi == kEpiBiasGelu && p.out_f32);
     if (f32 && (!p.out_f32 || mis(p.out_f32))) return cudaErrorInvalidValue;
     if (L.epi != kEpiF32 && (!p.out_bf16 || mis(p.out_bf16))) return cudaErrorInvalidValue;
-    if (p.out_t && mis(p.out_t)) return cudaErrorInvalidValue;
     if (L.epi == kEpiBiasGelu && !p.bias) return cudaErrorInvalidValue;
     if (L.epi == kEpiGeluBwd && (!p.zin || !p.colpart || mis(p.zin))) return cudaErrorInvalidValue;
-    if (!make_map(&maps.a[i], p.A, L.M, L.K, kBM) || !make_map(&maps.b[i], p.B, L.N, L.K, L.bn)) return cudaErrorInvalidValue;
-    // outputs: FP32 (K slices stacked by rows), BF16 row-major, BF16 transposed
+    if (!(L.amn ? make_map(&maps.a[i], p.A, L.K, L.M, kBK) : make_map(&maps.a[i], p.A, L.M, L.K, kBM)) ||
+        !(L.bmn ? make_map(&maps.b[i], p.B, L.K, L.N, kBK) : make_map(&maps.b[i], p.B, L.N, L.K, L.bn)))
+      return cudaErrorInvalidValue;
+    // outputs: FP32 (K slices stacked by rows), BF16
     if (f32 && !make_map_2d(&maps.of[i], p.out_f32, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, L.M * L.ksplit, L.N,
                             (size_t)L.ldo * 4, 32, kBM))
       return cudaErrorInvalidValue;
     if (L.epi != kEpiF32 && !make_map_2d(&maps.ob[i], p.out_bf16, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, L.M, L.N,
                                          (size_t)L.ldo * 2, 64, kBM))
-      return cudaErrorInvalidValue;
-    if (p.out_t && !make_map_2d(&maps.ot[i], p.out_t, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, L.N, L.M, (size_t)L.ldt * 2, 64,
-                                kBM))
       return cudaErrorInvalidValue;
     g.p[i] = p;
   }
@@ -1078,14 +1053,17 @@ cudaError_t gemm(const GemmLaunch& L, cudaStream_t st) {
   g.nkb = L.K / L.ksplit / kBK;
   g.ksplit = L.ksplit;
   g.ldo = L.ldo;
-  g.ldt = L.ldt;
   g.zstride = L.zstride;
   g.err = L.err;
   dim3 grid(L.N / L.bn, L.M / kBM, L.np * L.ksplit);
-  if (kind == 0) k_gemm_tn<3, kEpiF32, 128><<<grid, gemm_threads(3), gemm_smem(3, 128), st>>>(maps, g);
-  else if (kind == 1) k_gemm_tn<6, kEpiBiasGelu, 128><<<grid, gemm_threads(6), gemm_smem(6, 128), st>>>(maps, g);
-  else if (kind == 2) k_gemm_tn<6, kEpiGeluBwd, 128><<<grid, gemm_threads(6), gemm_smem(6, 128), st>>>(maps, g);
-  else k_gemm_tn<4, kEpiF32, 256><<<grid, gemm_threads(4), gemm_smem(4, 256), st>>>(maps, g);
+  if (kind == 0)
+    k_gemm_tn<3, kEpiF32, 128, false, false><<<grid, gemm_threads(3), gemm_smem(3, 128), st>>>(maps, g);
+  else if (kind == 1)
+    k_gemm_tn<6, kEpiBiasGelu, 128, false, false><<<grid, gemm_threads(6), gemm_smem(6, 128), st>>>(maps, g);
+  else if (kind == 2)
+    k_gemm_tn<6, kEpiGeluBwd, 128, false, true><<<grid, gemm_threads(6), gemm_smem(6, 128), st>>>(maps, g);
+  else
+    k_gemm_tn<4, kEpiF32, 256, true, true><<<grid, gemm_threads(4), gemm_smem(4, 256), st>>>(maps, g);
   return cudaGetLastError();
 }
 
@@ -1096,11 +1074,11 @@ cudaError_t head_fwd_loss(const __nv_bfloat16* H, const __nv_bfloat16* W5, const
 }
 
 cudaError_t head_train(const __nv_bfloat16* H, const __nv_bfloat16* W5, const float* b5, const float* T, const float* Z,
-                       int M, float* Y, float* dY, float* row_loss, __nv_bfloat16* dZ, __nv_bfloat16* dZt, float* colpart,
-                       float* dWpart, float* dbpart, cudaStream_t st) {
+                       int M, float* Y, float* dY, float* row_loss, __nv_bfloat16* dZ, float* colpart, float* dWpart,
+                       float* dbpart, int* step_idx, cudaStream_t st) {
   if (M % kHeadRows) return cudaErrorInvalidValue;
-  k_head_train<<<M / kHeadRows, kHeadThreads, kHeadSmem, st>>>(H, W5, b5, T, Z, M, Y, dY, row_loss, dZ, dZt, colpart, dWpart,
-                                                     dbpart);
+  k_head_train<<<M / kHeadRows, kHeadThreads, kHeadSmem, st>>>(H, W5, b5, T, Z, M, Y, dY, row_loss, dZ, colpart, dWpart,
+                                                               dbpart, step_idx);
   return cudaGetLastError();
 }
 
@@ -1108,9 +1086,7 @@ cudaError_t grad_finish(const FinishArgs& a, cudaStream_t st) {
   static_assert(kFinishW % 1024 == 0 && (long long)kFinishW + kFinishR == kNumParams, "every entry once");
   static_assert(kFinishBiasGroups * 32 + kFinishHeadWGroups * 32 + kOut == kFinishR, "every reduced entry once");
   k_grad_finish<<<kFinishWBlocks + kFinishRBlocks + 1, 256, 0, st>>>(a);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && a.adam) e = transpose_layers(a.wb, a.wt, st, a.t_idx);
-  return e;
+  return cudaGetLastError();
 }
 
 cudaError_t adam_corrections(float b1, float b2, int step, float* bc1, float* bc2) {
@@ -1122,31 +1098,21 @@ cudaError_t adam_corrections(float b1, float b2, int step, float* bc1, float* bc
   return cudaSuccess;
 }
 
-cudaError_t transpose_layers(const __nv_bfloat16* wb, __nv_bfloat16* wt, cudaStream_t st, int* step_idx) {
-  k_transpose_layers<<<dim3(kHidden / 32, kHidden / 32, kLayers), dim3(32, 8), 0, st>>>(wb, wt, step_idx);
-  return cudaGetLastError();
-}
-
 cudaError_t adamw(float* w, const float* g, float* m1, float* m2, int n, float lr, float b1, float b2, float eps,
-                  float wd, int step, const AdamLayout& L, __nv_bfloat16* wb, __nv_bfloat16* wt, cudaStream_t st) {
+                  float wd, int step, const AdamLayout& L, __nv_bfloat16* wb, cudaStream_t st) {
   float bc1, bc2;
   adam_corrections(b1, b2, step, &bc1, &bc2);
   k_adamw<<<(n + 255) / 256, 256, 0, st>>>(w, g, m1, m2, n, lr, b1, b2, eps, wd, bc1, bc2, L, wb);
-  cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? transpose_layers(wb, wt, st) : e;
+  return cudaGetLastError();
 }
 
-cudaError_t pack_params(const float* w, int n, const AdamLayout& L, __nv_bfloat16* wb, __nv_bfloat16* wt,
-                        cudaStream_t st) {
+cudaError_t pack_params(const float* w, int n, const AdamLayout& L, __nv_bfloat16* wb, cudaStream_t st) {
   k_pack_params<<<(n + 255) / 256, 256, 0, st>>>(w, n, L, wb);
-  cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? transpose_layers(wb, wt, st) : e;
+  return cudaGetLastError();
 }
 
-cudaError_t featurize(const DevSac* sacs, const float* traces, int n, __nv_bfloat16* X, __nv_bfloat16* Xt, int ldt,
-                      cudaStream_t st) {
-  if (Xt && ldt % 8) return cudaErrorInvalidValue;
-  k_featurize<<<(n + kFeatRows - 1) / kFeatRows, 128, 0, st>>>(sacs, traces, n, X, Xt, ldt);
+cudaError_t featurize(const DevSac* sacs, const float* traces, int n, __nv_bfloat16* X, cudaStream_t st) {
+  k_featurize<<<(n + kFeatRows - 1) / kFeatRows, 128, 0, st>>>(sacs, traces, n, X);
   return cudaGetLastError();
 }
 

@@ -31,20 +31,16 @@ constexpr int kTrainLcap = 400;         // longest training window
 constexpr int kWgradSplit = 4;          // largest number of K slices of the weight-gradient GEMM
 struct MlpBuffers {
   int M = 0;
-  DevBuf X, Xt, H[kLayers], Ht[kLayers], Z[kLayers], Y, dY, rowloss, dZ[kLayers], dZt[kLayers], colpart[kLayers],
-      wpart, dWpart, dbpart;
+  DevBuf X, H[kLayers], Z[kLayers], Y, dY, rowloss, dZ[kLayers], colpart[kLayers], wpart, dWpart, dbpart;
   Status ensure(int m) {
     if (m <= M) return Status();
     Status s;
     const size_t act = (size_t)m * kHidden;
     s = X.ensure(act * 2);
-    if (s.ok()) s = Xt.ensure(act * 2);
     for (int l = 0; l < kLayers && s.ok(); ++l) {
       s = H[l].ensure(act * 2);
-      if (s.ok()) s = Ht[l].ensure(act * 2);
       if (s.ok()) s = Z[l].ensure(act * 4);
       if (s.ok()) s = dZ[l].ensure(act * 2);
-      if (s.ok()) s = dZt[l].ensure(act * 2);
       // column sums per 128-row tile (GEMM epilogue) or per 32-row block (head)
       if (s.ok()) s = colpart[l].ensure((size_t)(m / (l == kLayers - 1 ? 32 : kBM)) * kHidden * 4);
     }
@@ -60,14 +56,14 @@ struct MlpBuffers {
 };
 
 struct SurrogateState {
-  DevBuf w, g, m1, m2, wb, wt;           // FP32 master, gradient, Adam moments; BF16 copies
+  DevBuf w, g, m1, m2, wb;               // FP32 master, gradient, Adam moments; BF16 weights
   DevBuf cal_amp, cal_pulse;             // agonist pulse by amplitude (calibrated nominal)
   MlpBuffers buf;
   MlpBuffers infer;                      // admission-time inference of the request loop
   // training data: two slots, so that one batch is generated (on a side
   // stream) while the network trains on the other
   struct DataSlot {
-    DevBuf sacs, traces, hidden, target, X, Xt;
+    DevBuf sacs, traces, hidden, target, X;
   } slot[2];
   DevBuf outoff, losses;
   DevBuf tstate;                         // device step state: next sample base per slot, step index
@@ -88,7 +84,6 @@ static Status ensure_state(opmm_ctx* ctx) {
   if (s.ok()) s = S.m1.ensure(sizeof(float) * kNumParams);
   if (s.ok()) s = S.m2.ensure(sizeof(float) * kNumParams);
   if (s.ok()) s = S.wb.ensure(sizeof(__nv_bfloat16) * kWbElems);
-  if (s.ok()) s = S.wt.ensure(sizeof(__nv_bfloat16) * kWtElems);
   if (s.ok()) s = S.cal_amp.ensure(sizeof(float) * kCal);
   if (s.ok()) s = S.cal_pulse.ensure(sizeof(float) * kCal);
   if (s.ok()) s = cuda_status(gemm_prepare(), "GEMM attributes");
@@ -128,12 +123,12 @@ static Status build_calibration(opmm_ctx* ctx) {
 
 static Status refresh_copies(opmm_ctx* ctx) {
   SurrogateState& S = *ctx->surrogate;
-  return cuda_status(pack_params(f32(S.w), (int)kNumParams, AdamLayout{}, bf(S.wb), bf(S.wt), ctx->stream), "pack");
+  return cuda_status(pack_params(f32(S.w), (int)kNumParams, AdamLayout{}, bf(S.wb), ctx->stream), "pack");
 }
 
 // Hidden layers of M rows from X on the tensor cores: H = GELU(Z) (BF16)
-// and, for training, Z (pre-activations, FP32) and H's transpose.
-static Status forward_hidden(opmm_ctx* ctx, MlpBuffers& B, int M, const __nv_bfloat16* X, bool keep_transposes,
+// and, for training, Z (pre-activations, FP32).
+static Status forward_hidden(opmm_ctx* ctx, MlpBuffers& B, int M, const __nv_bfloat16* X, bool train,
                              cudaStream_t st) {
   SurrogateState& S = *ctx->surrogate;
   for (int l = 0; l < kLayers; ++l) {
@@ -143,7 +138,6 @@ static Status forward_hidden(opmm_ctx* ctx, MlpBuffers& B, int M, const __nv_bfl
     L.K = kHidden;
     L.epi = kEpiBiasGelu;
     L.ldo = kHidden;
-    L.ldt = M;
     L.stages = 6;
     L.err = ctx->d_err.as<unsigned>();
     GemmProblem& p = L.p[0];
@@ -151,8 +145,7 @@ static Status forward_hidden(opmm_ctx* ctx, MlpBuffers& B, int M, const __nv_bfl
     p.B = bf(S.wb, (size_t)l * kHidden * kHidden);
     p.bias = f32(S.w, (size_t)l * kLayerParams + (size_t)kHidden * kHidden);
     p.out_bf16 = bf(B.H[l]);
-    p.out_f32 = keep_transposes ? f32(B.Z[l]) : nullptr;   // Z only for the backward pass
-    p.out_t = keep_transposes ? bf(B.Ht[l]) : nullptr;
+    p.out_f32 = train ? f32(B.Z[l]) : nullptr;   // Z only for the backward pass
     Status s = cuda_status(gemm(L, st), "GEMM fwd");
     if (!s.ok()) return s;
   }
@@ -182,16 +175,15 @@ static Status forward(opmm_ctx* ctx, MlpBuffers& B, int M, cudaStream_t st) {
 struct AdamStep {
   float lr, wd;
   const float* bc_tab;
-  int* t_idx;
+  int* t_idx;   // -1 before the first step; the head kernel advances it
 };
-static Status train_pass(opmm_ctx* ctx, MlpBuffers& B, int M, const __nv_bfloat16* X, const __nv_bfloat16* Xt,
-                         const float* T, float* loss, const AdamStep* adam, cudaStream_t st) {
+static Status train_pass(opmm_ctx* ctx, MlpBuffers& B, int M, const __nv_bfloat16* X, const float* T, float* loss, const AdamStep* adam, cudaStream_t st) {
   SurrogateState& S = *ctx->surrogate;
   Status s = forward_hidden(ctx, B, M, X, true, st);
   if (!s.ok()) return s;
   s = cuda_status(head_train(bf(B.H[kLayers - 1]), bf(S.wb, (size_t)kLayers * kHidden * kHidden), f32(S.w, kHeadB), T,
                              f32(B.Z[kLayers - 1]), M, f32(B.Y), f32(B.dY), f32(B.rowloss), bf(B.dZ[kLayers - 1]),
-                             bf(B.dZt[kLayers - 1]), f32(B.colpart[kLayers - 1]), f32(B.dWpart), f32(B.dbpart), st),
+                             f32(B.colpart[kLayers - 1]), f32(B.dWpart), f32(B.dbpart), adam ? adam->t_idx : nullptr, st),
                   "head");
   for (int l = kLayers - 1; l >= 1 && s.ok(); --l) {
     // dZ_{l-1} from dH_{l-1}[m][k] = sum_n dZ_l[m][n] W_l[n][k]
@@ -201,15 +193,14 @@ static Status train_pass(opmm_ctx* ctx, MlpBuffers& B, int M, const __nv_bfloat1
     L.K = kHidden;
     L.epi = kEpiGeluBwd;
     L.ldo = kHidden;
-    L.ldt = M;
     L.stages = 6;
     L.err = ctx->d_err.as<unsigned>();
     GemmProblem& p = L.p[0];
     p.A = bf(B.dZ[l]);
-    p.B = bf(S.wt, (size_t)l * kHidden * kHidden);
+    p.B = bf(S.wb, (size_t)l * kHidden * kHidden);
+    L.bmn = true;   // W_l [n][k]: stored across the sum's index n
     p.zin = f32(B.Z[l - 1]);
     p.out_bf16 = bf(B.dZ[l - 1]);
-    p.out_t = bf(B.dZt[l - 1]);
     p.colpart = f32(B.colpart[l - 1]);
     s = cuda_status(gemm(L, st), "GEMM dgrad");
   }
@@ -224,14 +215,15 @@ static Status train_pass(opmm_ctx* ctx, MlpBuffers& B, int M, const __nv_bfloat1
     L.ksplit = M % (4 * kBK) == 0 && M >= 1024 ? kWgradSplit : M >= 2 * kBM ? 2 : 1;
     L.epi = kEpiF32;
     L.bn = 256;
+    L.amn = L.bmn = true;   // dZ [m][n] and H [m][k]: stored across the sum's index m
     L.ldo = kHidden;
     L.zstride = (long long)kHidden * kHidden;
     L.stages = 4;
     L.err = ctx->d_err.as<unsigned>();
     for (int l = 0; l < kLayers; ++l) {
       GemmProblem& p = L.p[l];
-      p.A = bf(B.dZt[l]);
-      p.B = l == 0 ? Xt : bf(B.Ht[l - 1]);
+      p.A = bf(B.dZ[l]);
+      p.B = l == 0 ? X : bf(B.H[l - 1]);
       p.out_f32 = f32(B.wpart, (size_t)l * L.ksplit * kHidden * kHidden);
     }
     s = cuda_status(gemm(L, st), "GEMM wgrad");
@@ -263,7 +255,6 @@ static Status train_pass(opmm_ctx* ctx, MlpBuffers& B, int M, const __nv_bfloat1
         a.m1 = f32(S.m1);
         a.m2 = f32(S.m2);
         a.wb = bf(S.wb);
-        a.wt = bf(S.wt);
       }
       s = cuda_status(grad_finish(a, st), adam ? "gradient assembly and AdamW" : "gradient assembly");
     }
@@ -282,7 +273,7 @@ Status surrogate_centres(opmm_ctx* ctx, const DevSac* sacs, const float* traces,
     s = cuda_status(cudaMemsetAsync(B.X.ptr, 0, (size_t)M * kIn * 2, st), "clear features");
     if (!s.ok()) return s;
   }
-  Status s = cuda_status(featurize(sacs, traces, n, bf(B.X), nullptr, M, st), "featurize");
+  Status s = cuda_status(featurize(sacs, traces, n, bf(B.X), st), "featurize");
   if (s.ok()) s = forward(ctx, B, M, st);
   if (s.ok()) s = cuda_status(apply_centres(f32(B.Y), n, pc, st), "centres");
   return s;
@@ -314,7 +305,7 @@ Status surrogate_prepare_plan(opmm_ctx* ctx, opmm_plan* p, const opmm_saccade*, 
   p->pre_search_kernels = 1 + kLayers + 2;
   p->pre_search = [keep, M](opmm_plan* pl, cudaStream_t st) -> Status {
     opmm_ctx* c = pl->ctx;
-    Status r = cuda_status(featurize(pl->d_sacs.as<DevSac>(), pl->d_traces.as<float>(), pl->n, bf(keep->X), nullptr, M, st),
+    Status r = cuda_status(featurize(pl->d_sacs.as<DevSac>(), pl->d_traces.as<float>(), pl->n, bf(keep->X), st),
                            "featurize");
     if (r.ok()) r = forward(c, *keep, M, st);
     if (r.ok()) r = cuda_status(apply_centres(f32(keep->Y), pl->n, pl->d_pc.as<float>(), st), "centres");
@@ -398,21 +389,15 @@ extern "C" int opmm_surrogate_grad(opmm_ctx* ctx, const float* x, const float* t
   MlpBuffers& B = S.buf;
   STRY(B.ensure(m));
   cudaStream_t st = ctx->stream;
-  // host features -> BF16 (round to nearest even) and the transpose
-  std::vector<__nv_bfloat16> xb((size_t)m * kIn), xt((size_t)m * kIn);
-  for (int i = 0; i < m; ++i)
-    for (int k = 0; k < kIn; ++k) {
-      const __nv_bfloat16 v = __float2bfloat16_rn(x[(size_t)i * kIn + k]);
-      xb[(size_t)i * kIn + k] = v;
-      xt[(size_t)k * m + i] = v;
-    }
+  // host features -> BF16 (round to nearest even)
+  std::vector<__nv_bfloat16> xb((size_t)m * kIn);
+  for (size_t i = 0; i < xb.size(); ++i) xb[i] = __float2bfloat16_rn(x[i]);
   DevBuf dt;
   STRY(dt.ensure((size_t)m * kOut * 4));
   STRY(cuda_status(cudaMemcpyAsync(B.X.ptr, xb.data(), xb.size() * 2, cudaMemcpyHostToDevice, st), "H2D X"));
-  STRY(cuda_status(cudaMemcpyAsync(B.Xt.ptr, xt.data(), xt.size() * 2, cudaMemcpyHostToDevice, st), "H2D Xt"));
   STRY(cuda_status(cudaMemcpyAsync(dt.ptr, t, (size_t)m * kOut * 4, cudaMemcpyHostToDevice, st), "H2D T"));
   STRY(cuda_status(cudaMemsetAsync(ctx->d_err.ptr, 0, 4, st), "clear error"));
-  STRY(train_pass(ctx, B, m, bf(B.X), bf(B.Xt), f32(dt), nullptr, nullptr, st));
+  STRY(train_pass(ctx, B, m, bf(B.X), f32(dt), nullptr, nullptr, st));
   std::vector<float> rl((size_t)m);
   STRY(cuda_status(cudaMemcpyAsync(rl.data(), B.rowloss.ptr, (size_t)m * 4, cudaMemcpyDeviceToHost, st), "D2H loss"));
   STRY(cuda_status(cudaMemcpyAsync(grad, S.g.ptr, (size_t)kNumParams * 4, cudaMemcpyDeviceToHost, st), "D2H grad"));
@@ -438,7 +423,7 @@ extern "C" int opmm_surrogate_apply_grad(opmm_ctx* ctx, const float* grad, float
   STRY(cuda_status(cudaMemcpyAsync(S.g.ptr, grad, (size_t)kNumParams * 4, cudaMemcpyHostToDevice, st), "H2D grad"));
   S.step += 1;
   STRY(cuda_status(adamw(f32(S.w), f32(S.g), f32(S.m1), f32(S.m2), (int)kNumParams, lr, 0.9f, 0.999f, 1e-8f,
-                         weight_decay, S.step, AdamLayout{}, bf(S.wb), bf(S.wt), st), "AdamW"));
+                         weight_decay, S.step, AdamLayout{}, bf(S.wb), st), "AdamW"));
   STRY(cuda_status(cudaStreamSynchronize(st), "apply_grad"));
   return OPMM_OK;
 }
@@ -460,7 +445,6 @@ extern "C" int opmm_surrogate_train(opmm_ctx* ctx, int32_t steps, int32_t batch,
       STRY(D.hidden.ensure(sizeof(float) * (size_t)batch * kOut));
       STRY(D.target.ensure(sizeof(float) * (size_t)batch * kOut));
       STRY(D.X.ensure((size_t)batch * kIn * 2));
-      STRY(D.Xt.ensure((size_t)batch * kIn * 2));
     }
     STRY(S.outoff.ensure(sizeof(long long) * (size_t)batch));
     std::vector<long long> off((size_t)batch);
@@ -483,7 +467,7 @@ extern "C" int opmm_surrogate_train(opmm_ctx* ctx, int32_t steps, int32_t batch,
     for (int t = 0; t < steps; ++t) adam_corrections(0.9f, 0.999f, S.step + 1 + t, &tab[2 * (size_t)t], &tab[2 * (size_t)t + 1]);
     const long long init[2] = {(long long)sample_base, (long long)sample_base + batch};
     STRY(cuda_status(cudaMemcpyAsync(gbase, init, sizeof init, cudaMemcpyHostToDevice, st), "H2D step state"));
-    STRY(cuda_status(cudaMemsetAsync(t_idx, 0, sizeof(int), st), "clear step index"));
+    STRY(cuda_status(cudaMemsetAsync(t_idx, 0xff, sizeof(int), st), "step index -1"));
     STRY(cuda_status(cudaMemcpyAsync(S.bctab.ptr, tab.data(), tab.size() * 4, cudaMemcpyHostToDevice, st), "H2D corrections"));
     STRY(cuda_status(cudaStreamSynchronize(st), "stage step state"));
   }
@@ -525,14 +509,13 @@ extern "C" int opmm_surrogate_train(opmm_ctx* ctx, int32_t steps, int32_t batch,
                                       f32(D.traces), s2), "simulate");
     if (r.ok()) r = cuda_status(add_noise(data_seed, gbase + b, D.sacs.as<DevSac>(), batch, f32(D.traces), 0.05f, s2), "noise");
     if (r.ok())
-      r = cuda_status(featurize(D.sacs.as<DevSac>(), f32(D.traces), batch, bf(D.X), bf(D.Xt), batch, s2), "featurize");
+      r = cuda_status(featurize(D.sacs.as<DevSac>(), f32(D.traces), batch, bf(D.X), s2), "featurize");
     if (r.ok()) r = cuda_status(bump(gbase + b, 2LL * batch, nullptr, s2), "advance sample base");
     return r;
   };
   auto net = [&](int b, cudaStream_t s1) -> Status {
     SurrogateState::DataSlot& D = S.slot[b];
-    // the step index advances in the weight transposes that end the step
-    return train_pass(ctx, B, batch, bf(D.X), bf(D.Xt), f32(D.target), f32(S.losses), &adam, s1);
+    return train_pass(ctx, B, batch, bf(D.X), f32(D.target), f32(S.losses), &adam, s1);
   };
   if (steps > 0) STRY(gen(0, st));
   const int pairs = steps / 2;
@@ -644,7 +627,7 @@ extern "C" int opmm_featurize(opmm_ctx* ctx, const opmm_saccade* sacs, int32_t n
   STRY(plan_stage(ctx, sacs, n, o, &p));
   DevBuf X;
   STRY(X.ensure((size_t)n * kIn * 2));
-  STRY(cuda_status(featurize(p.d_sacs.as<DevSac>(), p.d_traces.as<float>(), n, bf(X), nullptr, n, ctx->stream),
+  STRY(cuda_status(featurize(p.d_sacs.as<DevSac>(), p.d_traces.as<float>(), n, bf(X), ctx->stream),
                    "featurize"));
   std::vector<__nv_bfloat16> h((size_t)n * kIn);
   STRY(cuda_status(cudaMemcpyAsync(h.data(), X.ptr, h.size() * 2, cudaMemcpyDeviceToHost, ctx->stream), "D2H"));
