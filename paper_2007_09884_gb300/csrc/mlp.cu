@@ -54,6 +54,14 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int 
                "r"(y), "r"(smem_u32(src))
                : "memory");
 }
+// Programmatic dependent launch.  A kernel launched as the next of a chain may
+// start while the one before it still runs; chain_wait returns once that one
+// has completed and its writes are visible (at once for any other launch),
+// and no thread touches global memory before it.  chain_go lets the next
+// kernel of the chain start.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 
@@ -265,6 +273,8 @@ __global__ void __launch_bounds__(gemm_threads(STAGES), STAGES <= 3 ? 2 : 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  chain_go();
+  chain_wait();
 
   if (warp == kTmaWarp) {
     if (lane == 0) {
@@ -496,6 +506,8 @@ __global__ void __launch_bounds__(kHeadThreads) k_head_train(const __nv_bfloat16
                                                              float* Y, float* dY, float* row_loss, __nv_bfloat16* dZ,
                                                              float* colpart, float* dWpart, float* dbpart,
                                                              int* step_idx) {
+  chain_go();
+  chain_wait();
   // the step index of a replayed training sequence advances here: the last
   // step's AdamW, its only reader, is over, and this step's is to come
   if (step_idx && blockIdx.x == 0 && threadIdx.x == 0) *step_idx += 1;
@@ -702,6 +714,7 @@ constexpr int kFinishRBlocks = kFinishBiasGroups + kFinishHeadWGroups + 1;   // 
 
 __global__ void __launch_bounds__(256) k_grad_finish(const __grid_constant__ FinishArgs a) {
   const int tid = threadIdx.x;
+  chain_wait();
   const int t = a.t_idx ? *a.t_idx : 0;            // step within a replayed sequence
   const float bc1 = a.bc_tab ? a.bc_tab[2 * t] : a.bc1;
   const float bc2 = a.bc_tab ? a.bc_tab[2 * t + 1] : a.bc2;
@@ -1012,6 +1025,24 @@ cudaError_t gemm_prepare() {
   return e;
 }
 
+// Launch; chained: as the next kernel of a chain (see chain_wait), after the
+// kernel launched last on the stream.
+template <class... P, class... A>
+static cudaError_t launch_chain(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, bool chained,
+                                const A&... args) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = dim3((unsigned)threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
 cudaError_t gemm(const GemmLaunch& L, cudaStream_t st) {
   if (L.np < 1 || L.np > kMaxGroup || L.ksplit < 1 || L.M <= 0 || L.N <= 0 || L.K <= 0) return cudaErrorInvalidValue;
   if (L.M % kBM || L.N % L.bn || L.K % (L.ksplit * kBK)) return cudaErrorInvalidValue;
@@ -1057,14 +1088,12 @@ cudaError_t gemm(const GemmLaunch& L, cudaStream_t st) {
   g.err = L.err;
   dim3 grid(L.N / L.bn, L.M / kBM, L.np * L.ksplit);
   if (kind == 0)
-    k_gemm_tn<3, kEpiF32, 128, false, false><<<grid, gemm_threads(3), gemm_smem(3, 128), st>>>(maps, g);
-  else if (kind == 1)
-    k_gemm_tn<6, kEpiBiasGelu, 128, false, false><<<grid, gemm_threads(6), gemm_smem(6, 128), st>>>(maps, g);
-  else if (kind == 2)
-    k_gemm_tn<6, kEpiGeluBwd, 128, false, true><<<grid, gemm_threads(6), gemm_smem(6, 128), st>>>(maps, g);
-  else
-    k_gemm_tn<4, kEpiF32, 256, true, true><<<grid, gemm_threads(4), gemm_smem(4, 256), st>>>(maps, g);
-  return cudaGetLastError();
+    return launch_chain(k_gemm_tn<3, kEpiF32, 128, false, false>, grid, gemm_threads(3), gemm_smem(3, 128), st, L.chained, maps, g);
+  if (kind == 1)
+    return launch_chain(k_gemm_tn<6, kEpiBiasGelu, 128, false, false>, grid, gemm_threads(6), gemm_smem(6, 128), st, L.chained, maps, g);
+  if (kind == 2)
+    return launch_chain(k_gemm_tn<6, kEpiGeluBwd, 128, false, true>, grid, gemm_threads(6), gemm_smem(6, 128), st, L.chained, maps, g);
+  return launch_chain(k_gemm_tn<4, kEpiF32, 256, true, true>, grid, gemm_threads(4), gemm_smem(4, 256), st, L.chained, maps, g);
 }
 
 cudaError_t head_fwd_loss(const __nv_bfloat16* H, const __nv_bfloat16* W5, const float* b5, const float* T, int M,
@@ -1077,16 +1106,14 @@ cudaError_t head_train(const __nv_bfloat16* H, const __nv_bfloat16* W5, const fl
                        int M, float* Y, float* dY, float* row_loss, __nv_bfloat16* dZ, float* colpart, float* dWpart,
                        float* dbpart, int* step_idx, cudaStream_t st) {
   if (M % kHeadRows) return cudaErrorInvalidValue;
-  k_head_train<<<M / kHeadRows, kHeadThreads, kHeadSmem, st>>>(H, W5, b5, T, Z, M, Y, dY, row_loss, dZ, colpart, dWpart,
-                                                               dbpart, step_idx);
-  return cudaGetLastError();
+  return launch_chain(k_head_train, dim3(M / kHeadRows), kHeadThreads, kHeadSmem, st, true, H, W5, b5, T, Z, M, Y, dY,
+                      row_loss, dZ, colpart, dWpart, dbpart, step_idx);
 }
 
 cudaError_t grad_finish(const FinishArgs& a, cudaStream_t st) {
   static_assert(kFinishW % 1024 == 0 && (long long)kFinishW + kFinishR == kNumParams, "every entry once");
   static_assert(kFinishBiasGroups * 32 + kFinishHeadWGroups * 32 + kOut == kFinishR, "every reduced entry once");
-  k_grad_finish<<<kFinishWBlocks + kFinishRBlocks + 1, 256, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_chain(k_grad_finish, dim3(kFinishWBlocks + kFinishRBlocks + 1), 256, 0, st, true, a);
 }
 
 cudaError_t adam_corrections(float b1, float b2, int step, float* bc1, float* bc2) {

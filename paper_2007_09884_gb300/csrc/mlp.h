@@ -67,6 +67,7 @@ struct GemmProblem {
 struct GemmLaunch {
   int np = 1, M = 0, N = 0, K = 0, ksplit = 1, epi = kEpiF32, bn = kBN;
   bool amn = false, bmn = false;
+  bool chained = false;        // may start before the stream's last kernel ends (that kernel's data is all it reads)
   int ldo = 0;
   long long zstride = 0;       // elements between the outputs of consecutive K slices
   int stages = 3;

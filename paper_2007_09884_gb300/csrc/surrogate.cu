@@ -139,6 +139,7 @@ static Status forward_hidden(opmm_ctx* ctx, MlpBuffers& B, int M, const __nv_bfl
     L.epi = kEpiBiasGelu;
     L.ldo = kHidden;
     L.stages = 6;
+    L.chained = l > 0;
     L.err = ctx->d_err.as<unsigned>();
     GemmProblem& p = L.p[0];
     p.A = l == 0 ? X : bf(B.H[l - 1]);
@@ -194,6 +195,7 @@ static Status train_pass(opmm_ctx* ctx, MlpBuffers& B, int M, const __nv_bfloat1
     L.epi = kEpiGeluBwd;
     L.ldo = kHidden;
     L.stages = 6;
+    L.chained = true;
     L.err = ctx->d_err.as<unsigned>();
     GemmProblem& p = L.p[0];
     p.A = bf(B.dZ[l]);
@@ -219,6 +221,7 @@ static Status train_pass(opmm_ctx* ctx, MlpBuffers& B, int M, const __nv_bfloat1
     L.ldo = kHidden;
     L.zstride = (long long)kHidden * kHidden;
     L.stages = 4;
+    L.chained = true;
     L.err = ctx->d_err.as<unsigned>();
     for (int l = 0; l < kLayers; ++l) {
       GemmProblem& p = L.p[l];
