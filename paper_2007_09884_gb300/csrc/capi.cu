@@ -86,6 +86,25 @@ Status HostBuf::ensure(size_t want) {
   return Status();
 }
 
+void FitBuffers::swap(FitBuffers& o) {
+  DevBuf* a[] = {&d_sacs, &d_traces, &d_pc, &d_sac_index, &d_units, &d_ustart, &d_unit_best, &d_counter, &d_results,
+                 &d_src, &d_pc_given};
+  DevBuf* b[] = {&o.d_sacs, &o.d_traces, &o.d_pc, &o.d_sac_index, &o.d_units, &o.d_ustart, &o.d_unit_best,
+                 &o.d_counter, &o.d_results, &o.d_src, &o.d_pc_given};
+  for (size_t i = 0; i < sizeof a / sizeof *a; ++i) a[i]->swap(*b[i]);
+  h_traces.swap(o.h_traces);
+  h_results.swap(o.h_results);
+  h_err.swap(o.h_err);
+}
+
+size_t FitBuffers::bytes() const {
+  size_t n = h_traces.bytes + h_results.bytes + h_err.bytes;
+  for (const DevBuf* b : {&d_sacs, &d_traces, &d_pc, &d_sac_index, &d_units, &d_ustart, &d_unit_best, &d_counter,
+                          &d_results, &d_src, &d_pc_given})
+    n += b->bytes;
+  return n;
+}
+
 int nsub_for(float fs) {
   const int n = (int)std::floor(1.0e4 / (double)fs + 0.5);
   return n < 1 ? 1 : n;
@@ -786,7 +805,9 @@ Status plan_stage(opmm_ctx* ctx, const opmm_saccade* sacs, int32_t n, const opmm
   P.counter = p->d_counter.as<int>();
   P.err = ctx->d_err.as<unsigned>();
 
-  // stage the traces and centres now (the tuner's probes and direct callers need them)
+  // stage the traces and centres now (the tuner's probes and direct callers
+  // need them; a one-shot fit stages them when it runs)
+  if (p->one_shot) return Status();
   if (!p->traces_on_device) pack_host_traces(p);
   s = enqueue_centres(p, st);
   if (s.ok()) s = cuda_status(cudaStreamSynchronize(st), "stage");
@@ -806,9 +827,11 @@ Status plan_build(opmm_ctx* ctx, const opmm_saccade* sacs, int32_t n, const opmm
   s = build_units(p, p->variant, p->blocks_per_sm);
   if (!s.ok()) return s;
   p->threads = search_variant_threads(p->variant);
-  s = cuda_status(cudaEventCreate(&p->ev_search[0]), "event");
-  if (s.ok()) s = cuda_status(cudaEventCreate(&p->ev_search[1]), "event");
-  if (!s.ok()) return s;
+  if (!p->one_shot) {
+    s = cuda_status(cudaEventCreate(&p->ev_search[0]), "event");
+    if (s.ok()) s = cuda_status(cudaEventCreate(&p->ev_search[1]), "event");
+    if (!s.ok()) return s;
+  }
   if (capture) {
     cudaStream_t cs = st;
     s = cuda_status(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal), "begin capture");
@@ -872,7 +895,7 @@ extern "C" int opmm_plan_create(opmm_ctx* ctx, const opmm_saccade* sacs, int32_t
   if (!p) return fail(ctx, Status(OPMM_ENOMEM, "plan allocation"));
   Status s;
   try {
-    if (opts->use_surrogate) s = surrogate_prepare_plan(ctx, p, sacs, n);
+    if (opts->use_surrogate) s = surrogate_prepare_plan(ctx, p, n, false);
     if (s.ok()) s = plan_build(ctx, sacs, n, *opts, true, true, p);
   } catch (const std::bad_alloc&) {
     s = Status(OPMM_ENOMEM, "host allocation failed");
@@ -945,9 +968,11 @@ extern "C" void opmm_plan_destroy(opmm_plan* plan) {
 static Status fit_once(opmm_ctx* ctx, const opmm_saccade* sacs, int32_t n, const opmm_fit_opts& o,
                        opmm_fit_result* out) {
   opmm_plan p;
+  BorrowBuffers lend(ctx, &p);
+  p.one_shot = true;
   Status s;
   try {
-    if (o.use_surrogate) s = surrogate_prepare_plan(ctx, &p, sacs, n);
+    if (o.use_surrogate) s = surrogate_prepare_plan(ctx, &p, n, true);
     if (s.ok()) s = plan_build(ctx, sacs, n, o, false, false, &p);
     if (s.ok()) s = plan_run(&p, out);
   } catch (const std::bad_alloc&) {
@@ -990,6 +1015,7 @@ extern "C" int opmm_refine_batch(opmm_ctx* ctx, const opmm_saccade* sacs, int32_
   fo.pulse_init = ro->pulse_init;
   fo.init_opc = ro->centre_opc;
   opmm_plan p;
+  BorrowBuffers lend(ctx, &p);
   TRY(plan_stage(ctx, sacs, n, fo, &p));
   cudaStream_t st = ctx->stream;
   DevBuf& b_start = ctx->scratch[8];

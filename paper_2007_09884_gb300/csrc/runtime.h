@@ -6,8 +6,10 @@
 #include <functional>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <tuple>
+#include <utility>
 #include <vector>
 
 #include "../../include/opmm.h"
@@ -45,6 +47,10 @@ struct DevBuf {
   ~DevBuf();
   Status ensure(size_t want);
   void release();
+  void swap(DevBuf& o) {
+    std::swap(ptr, o.ptr);
+    std::swap(bytes, o.bytes);
+  }
   template <class T> T* as() const { return static_cast<T*>(ptr); }
 };
 
@@ -58,7 +64,25 @@ struct HostBuf {
   ~HostBuf();
   Status ensure(size_t want);
   void release();
+  void swap(HostBuf& o) {
+    std::swap(ptr, o.ptr);
+    std::swap(bytes, o.bytes);
+  }
   template <class T> T* as() const { return static_cast<T*>(ptr); }
+};
+
+// Buffers of a fit of one batch: descriptors, traces, centres, work units and
+// results.  A plan owns its own; one-shot calls borrow the context's, which
+// keep their size from call to call up to kKeepBytes in all (allocating and
+// freeing them took 0.1 ms of a 1.1 ms single fit, and each free waits for
+// the device).
+struct FitBuffers {
+  DevBuf d_sacs, d_traces, d_pc, d_sac_index, d_units, d_ustart, d_unit_best, d_counter, d_results, d_src;
+  DevBuf d_pc_given;            // caller's centres when the surrogate rescales them
+  HostBuf h_traces, h_results, h_err;
+  static constexpr size_t kKeepBytes = (size_t)1 << 30;
+  void swap(FitBuffers& o);
+  size_t bytes() const;
 };
 
 struct SurrogateState;
@@ -81,6 +105,8 @@ struct opmm_ctx {
   opmm::DevBuf d_err;                 // device error word of the kernels
   opmm::DevBuf scratch[16];           // per-call scratch of the synchronous entry points
   opmm::HostBuf h_scratch[2];         // pinned host scratch of the synchronous entry points
+  opmm::FitBuffers once;              // buffers of the one-shot fit calls
+  std::mutex once_mu;                 // guards `once` and the surrogate's spare buffers while they change hands
   std::map<std::tuple<int, int, int, int>, std::pair<int, int>> tune_cache;
   std::map<std::tuple<int, int, int, int>, std::vector<opmm::TuneProbe>> tune_logs;
   opmm::SurrogateState* surrogate = nullptr;   // owned, released by surrogate_release
@@ -89,7 +115,7 @@ struct opmm_ctx {
   ~opmm_ctx();
 };
 
-struct opmm_plan {
+struct opmm_plan : opmm::FitBuffers {
   opmm_ctx* ctx = nullptr;
   int n = 0;
   opmm_fit_opts opts{};
@@ -104,6 +130,7 @@ struct opmm_plan {
   int lcap = 0;
   int sac_index_base = 0;             // Philox counter word of saccade 0
   bool autotune = false;
+  bool one_shot = false;              // runs once, right after it is built: nothing is staged ahead
   bool traces_on_device = false;
   bool centres_given = false;
   int pre_search_kernels = 0;
@@ -113,9 +140,6 @@ struct opmm_plan {
   std::vector<const float*> src;
   size_t trace_floats = 0;
   opmm::SearchParams params{};
-  opmm::DevBuf d_sacs, d_traces, d_pc, d_sac_index, d_units, d_ustart, d_unit_best, d_counter, d_results, d_src;
-  opmm::DevBuf d_pc_given;            // caller's centres when the surrogate rescales them
-  opmm::HostBuf h_traces, h_results, h_err;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaEvent_t ev_search[2] = {nullptr, nullptr};   // around the search kernel
@@ -135,7 +159,26 @@ void pack_host_traces(opmm_plan* p);
 
 // surrogate.cu
 void surrogate_release(opmm_ctx* ctx);
-Status surrogate_prepare_plan(opmm_ctx* ctx, opmm_plan* p, const opmm_saccade* sacs, int32_t n);
+// once: the plan is used by this call only and may borrow the context's buffers
+Status surrogate_prepare_plan(opmm_ctx* ctx, opmm_plan* p, int32_t n, bool once);
+
+// Lends the context's one-shot buffers to a plan for the length of a call.
+struct BorrowBuffers {
+  opmm_ctx* ctx;
+  opmm_plan* p;
+  BorrowBuffers(opmm_ctx* c, opmm_plan* q) : ctx(c), p(q) {
+    std::lock_guard<std::mutex> lock(ctx->once_mu);
+    p->swap(ctx->once);
+  }
+  ~BorrowBuffers() {
+    cudaStreamSynchronize(ctx->stream);   // a call that failed half way may have left work on them
+    if (p->bytes() > FitBuffers::kKeepBytes) return;   // freed with the plan
+    std::lock_guard<std::mutex> lock(ctx->once_mu);
+    p->swap(ctx->once);
+  }
+  BorrowBuffers(const BorrowBuffers&) = delete;
+  BorrowBuffers& operator=(const BorrowBuffers&) = delete;
+};
 
 // serve.cu
 void serve_shutdown(opmm_ctx* ctx);

@@ -30,7 +30,8 @@ constexpr int kTrainLcap = 400;         // longest training window
 // Activations and gradients of one batch of M rows (M a multiple of 128).
 constexpr int kWgradSplit = 4;          // largest number of K slices of the weight-gradient GEMM
 struct MlpBuffers {
-  int M = 0;
+  int M = 0;        // rows of a training pass
+  int rows = 0;     // rows of an inference pass (X, two layers' activations, Y)
   DevBuf X, H[kLayers], Z[kLayers], Y, dY, rowloss, dZ[kLayers], colpart[kLayers], wpart, dWpart, dbpart;
   Status ensure(int m) {
     if (m <= M) return Status();
@@ -50,7 +51,16 @@ struct MlpBuffers {
     if (s.ok()) s = wpart.ensure((size_t)kLayers * kWgradSplit * kHidden * kHidden * 4);
     if (s.ok()) s = dWpart.ensure((size_t)(m / 32) * kOut * kHidden * 4);
     if (s.ok()) s = dbpart.ensure((size_t)(m / 32) * kOut * 4);
-    if (s.ok()) M = m;
+    if (s.ok()) M = rows = m;
+    return s;
+  }
+  Status ensure_inference(int m) {
+    if (m <= rows) return Status();
+    const size_t act = (size_t)m * kHidden;
+    Status s = X.ensure(act * 2);
+    for (int l = 0; l < 2 && s.ok(); ++l) s = H[l].ensure(act * 2);
+    if (s.ok()) s = Y.ensure((size_t)m * kOut * 4);
+    if (s.ok()) rows = m;
     return s;
   }
 };
@@ -60,6 +70,7 @@ struct SurrogateState {
   DevBuf cal_amp, cal_pulse;             // agonist pulse by amplitude (calibrated nominal)
   MlpBuffers buf;
   MlpBuffers infer;                      // admission-time inference of the request loop
+  std::unique_ptr<MlpBuffers> spare;     // inference buffers of the last one-shot call (once_mu)
   // training data: two slots, so that one batch is generated (on a side
   // stream) while the network trains on the other
   struct DataSlot {
@@ -142,10 +153,11 @@ static Status forward_hidden(opmm_ctx* ctx, MlpBuffers& B, int M, const __nv_bfl
     L.chained = l > 0;
     L.err = ctx->d_err.as<unsigned>();
     GemmProblem& p = L.p[0];
-    p.A = l == 0 ? X : bf(B.H[l - 1]);
+    // inference needs no layer but the last: two activation buffers in turn
+    p.A = l == 0 ? X : bf(B.H[train ? l - 1 : (l - 1) & 1]);
     p.B = bf(S.wb, (size_t)l * kHidden * kHidden);
     p.bias = f32(S.w, (size_t)l * kLayerParams + (size_t)kHidden * kHidden);
-    p.out_bf16 = bf(B.H[l]);
+    p.out_bf16 = bf(B.H[train ? l : l & 1]);
     p.out_f32 = train ? f32(B.Z[l]) : nullptr;   // Z only for the backward pass
     Status s = cuda_status(gemm(L, st), "GEMM fwd");
     if (!s.ok()) return s;
@@ -158,8 +170,8 @@ static Status forward(opmm_ctx* ctx, MlpBuffers& B, int M, cudaStream_t st) {
   SurrogateState& S = *ctx->surrogate;
   Status s = forward_hidden(ctx, B, M, bf(B.X), false, st);
   if (!s.ok()) return s;
-  return cuda_status(head_fwd_loss(bf(B.H[kLayers - 1]), bf(S.wb, (size_t)kLayers * kHidden * kHidden),
-                                   f32(S.w, kHeadB), nullptr, M, f32(B.Y), f32(B.dY), nullptr, st),
+  return cuda_status(head_fwd_loss(bf(B.H[(kLayers - 1) & 1]), bf(S.wb, (size_t)kLayers * kHidden * kHidden),
+                                   f32(S.w, kHeadB), nullptr, M, f32(B.Y), nullptr, nullptr, st),
                      "head");
 }
 
@@ -270,8 +282,8 @@ Status surrogate_centres(opmm_ctx* ctx, const DevSac* sacs, const float* traces,
   if (!ctx->surrogate || !ctx->surrogate->ready) return Status(OPMM_EINVAL, "no surrogate");
   MlpBuffers& B = ctx->surrogate->infer;
   const int M = (n + kBM - 1) / kBM * kBM;
-  if (B.M < M) {
-    Status s = B.ensure(M);
+  if (B.rows < M) {
+    Status s = B.ensure_inference(M);
     if (!s.ok()) return s;
     s = cuda_status(cudaMemsetAsync(B.X.ptr, 0, (size_t)M * kIn * 2, st), "clear features");
     if (!s.ok()) return s;
@@ -289,22 +301,37 @@ void surrogate_release(opmm_ctx* ctx) {
 
 // Box centres of a plan from the network: featurize the staged traces, run the
 // forward pass, centre = nominal centre * exp(0.2 y).
-Status surrogate_prepare_plan(opmm_ctx* ctx, opmm_plan* p, const opmm_saccade*, int32_t n) {
+Status surrogate_prepare_plan(opmm_ctx* ctx, opmm_plan* p, int32_t n, bool once) {
   if (!ctx->surrogate || !ctx->surrogate->ready)
     return Status(OPMM_EINVAL, "use_surrogate set but no surrogate is initialised or loaded");
+  if (n < 1) return Status(OPMM_EINVAL, "empty batch");
   const int M = (n + kBM - 1) / kBM * kBM;
-  auto* bufs = new MlpBuffers();
-  Status s = bufs->ensure(M);
-  if (!s.ok()) {
-    delete bufs;
-    return s;
+  // a plan keeps its buffers; a one-shot call takes those the last one left
+  // and leaves them for the next
+  std::shared_ptr<MlpBuffers> keep;
+  if (once) {
+    MlpBuffers* b = nullptr;
+    {
+      std::lock_guard<std::mutex> lock(ctx->once_mu);
+      b = ctx->surrogate->spare.release();
+    }
+    keep = std::shared_ptr<MlpBuffers>(b ? b : new MlpBuffers(), [ctx](MlpBuffers* q) {
+      std::unique_ptr<MlpBuffers> own(q), old;   // `old` is freed outside the lock
+      if ((size_t)q->rows * kHidden * 6 > FitBuffers::kKeepBytes) return;
+      std::lock_guard<std::mutex> lock(ctx->once_mu);
+      old.swap(ctx->surrogate->spare);
+      ctx->surrogate->spare.swap(own);
+    });
+  } else {
+    keep = std::make_shared<MlpBuffers>();
   }
-  s = cuda_status(cudaMemset(bufs->X.ptr, 0, (size_t)M * kIn * 2), "clear features");
-  if (!s.ok()) {
-    delete bufs;
-    return s;
-  }
-  std::shared_ptr<MlpBuffers> keep(bufs);
+  Status s = keep->ensure_inference(M);
+  if (!s.ok()) return s;
+  // the rows past n that pad the last tile (of another call's features, else)
+  if (M > n)
+    s = cuda_status(cudaMemsetAsync(bf(keep->X, (size_t)n * kIn), 0, (size_t)(M - n) * kIn * 2, ctx->stream),
+                    "clear features");
+  if (!s.ok()) return s;
   p->pre_search_kernels = 1 + kLayers + 2;
   p->pre_search = [keep, M](opmm_plan* pl, cudaStream_t st) -> Status {
     opmm_ctx* c = pl->ctx;
@@ -567,7 +594,8 @@ extern "C" int opmm_surrogate_predict(opmm_ctx* ctx, const opmm_saccade* sacs, i
   o.pulse_init = pulse_init;
   o.use_surrogate = 1;
   opmm_plan p;
-  Status s = surrogate_prepare_plan(ctx, &p, sacs, n);
+  BorrowBuffers lend(ctx, &p);
+  Status s = surrogate_prepare_plan(ctx, &p, n, true);
   if (s.ok()) s = plan_stage(ctx, sacs, n, o, &p);   // stages traces and applies the surrogate
   if (s.ok())
     s = cuda_status(cudaMemcpyAsync(out_opc, p.d_pc.ptr, sizeof(float) * OPMM_NPARAM * (size_t)n, cudaMemcpyDeviceToHost,
@@ -627,6 +655,7 @@ extern "C" int opmm_featurize(opmm_ctx* ctx, const opmm_saccade* sacs, int32_t n
   std::vector<float> zero_centres((size_t)n * OPMM_NPARAM, 1.0f);
   o.init_opc = zero_centres.data();
   opmm_plan p;
+  BorrowBuffers lend(ctx, &p);
   STRY(plan_stage(ctx, sacs, n, o, &p));
   DevBuf X;
   STRY(X.ensure((size_t)n * kIn * 2));
