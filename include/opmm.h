@@ -388,6 +388,11 @@ typedef struct {
  * fails; OPMM_ECUDA for CUDA errors. */
 int opmm_detect_saccades(opmm_ctx* ctx, const float* stream_deg, int64_t n_samples, float sample_rate_hz,
                          const opmm_ivt_opts* opts, opmm_ivt_event* out, int32_t max_events, int32_t* n_events);
+/* The same without a copy: *events points at all *n_events kept events in the
+ * context's own array (NULL when there are none), which stays as it is until
+ * the next detection on this context or its destruction. */
+int opmm_detect_saccades_view(opmm_ctx* ctx, const float* stream_deg, int64_t n_samples, float sample_rate_hz,
+                              const opmm_ivt_opts* opts, const opmm_ivt_event** events, int32_t* n_events);
 
 /* Fresh weights (uniform +-1/sqrt(512), seeded) and zeroed AdamW state; builds
  * the amplitude -> agonist-pulse table the training data uses. */

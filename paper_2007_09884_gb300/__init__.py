@@ -133,6 +133,8 @@ def load_library(path: str = LIB_PATH):
                                       ctypes.POINTER(opmm_fit_result)]
     lib.opmm_detect_saccades.argtypes = [vp, vp, ctypes.c_int64, ctypes.c_float, ctypes.POINTER(opmm_ivt_opts), vp,
                                          i32, ctypes.POINTER(i32)]
+    lib.opmm_detect_saccades_view.argtypes = [vp, vp, ctypes.c_int64, ctypes.c_float, ctypes.POINTER(opmm_ivt_opts),
+                                              ctypes.POINTER(vp), ctypes.POINTER(i32)]
     lib.opmm_fit_batch_seeded.argtypes = [vp, ctypes.POINTER(opmm_saccade), i32, ctypes.POINTER(opmm_fit_opts),
                                           ctypes.POINTER(opmm_fit_opts), ctypes.c_float,
                                           ctypes.POINTER(opmm_fit_result), ctypes.POINTER(ctypes.c_int32)]
@@ -334,7 +336,6 @@ def opmm_create(device: int = 0):
 
 
 def opmm_destroy(ctx):
-    _IVT_OUT.pop(_ctx_key(ctx), None)
     load_library().opmm_destroy(ctx)
 
 
@@ -460,13 +461,6 @@ IVT_EVENT_DTYPE = np.dtype([("onset", "<i8"), ("end", "<i8"), ("window_start", "
                             ("reserved", "<i4")])
 
 
-_IVT_OUT = {}
-
-
-def _ctx_key(ctx) -> int:
-    return ctypes.cast(ctx, ctypes.c_void_p).value or 0
-
-
 def opmm_detect_saccades(ctx, stream, sample_rate_hz, threshold_dps=30.0, min_duration_ms=6.0,
                          min_amplitude_deg=4.0, valid_min_deg=-90.0, valid_max_deg=90.0, pre_samples=10,
                          post_samples=40, max_events=None) -> np.ndarray:
@@ -480,20 +474,16 @@ def opmm_detect_saccades(ctx, stream, sample_rate_hz, threshold_dps=30.0, min_du
         raise ValueError("stream tensor must be float32")
     ptr, keep = _ptr(stream)
     n = int(stream.numel()) if _is_torch(stream) else int(keep.size)
-    cap = int(max_events) if max_events is not None else max(16, n // 64)
-    # the event array is kept per context and reused (its pages are touched
-    # once); the caller gets a copy of the events found
-    out = _IVT_OUT.get(_ctx_key(ctx))
-    if out is None or out.size < cap:
-        out = np.zeros(cap, dtype=IVT_EVENT_DTYPE)
-        _IVT_OUT[_ctx_key(ctx)] = out
-    found = ctypes.c_int32()
-    _check(ctx, lib.opmm_detect_saccades(ctx, ptr, ctypes.c_int64(n), ctypes.c_float(sample_rate_hz),
-                                         ctypes.byref(o), out.ctypes.data, cap, ctypes.byref(found)))
-    if found.value > cap and max_events is None:
-        return opmm_detect_saccades(ctx, stream, sample_rate_hz, threshold_dps, min_duration_ms, min_amplitude_deg,
-                                    valid_min_deg, valid_max_deg, pre_samples, post_samples, found.value)
-    return out[:min(found.value, cap)].copy()
+    if max_events is not None and int(max_events) < 0:
+        raise OpmmError(OPMM_EINVAL, "opmm_detect_saccades: bad options")
+    view, found = ctypes.c_void_p(), ctypes.c_int32()
+    _check(ctx, lib.opmm_detect_saccades_view(ctx, ptr, ctypes.c_int64(n), ctypes.c_float(sample_rate_hz),
+                                              ctypes.byref(o), ctypes.byref(view), ctypes.byref(found)))
+    count = found.value if max_events is None else min(found.value, int(max_events))
+    if count == 0:
+        return np.zeros(0, IVT_EVENT_DTYPE)
+    raw = (ctypes.c_char * (count * IVT_EVENT_DTYPE.itemsize)).from_address(view.value)
+    return np.frombuffer(raw, IVT_EVENT_DTYPE).copy()
 
 
 def batch_from_events(stream, events, sample_rate_hz) -> SaccadeBatch:

@@ -21,7 +21,7 @@
 #include <cstdint>
 #include <cfloat>
 #include <cmath>
-#include <vector>
+#include <cstring>
 
 #include "../../include/opmm.h"
 #include "launch.h"
@@ -57,34 +57,54 @@ constexpr int kIvtIters = 8;
 constexpr int kVec = 4;                                                     // steps per thread and iteration
 constexpr long long kTile = (long long)kIvtThreads * kIvtIters * kVec;     // steps per tile (one block)
 
-// Run starts among steps 4m+1 .. 4m+4 (bit i for step 4m+1+i).  Group m's
-// samples 4m .. 4m+3 come in one 16-byte load when the stream is aligned;
-// sample 4m-1 (for step 4m) and sample 4m+4 from the neighbouring lanes.
-// Every lane of the warp calls it, with consecutive m on consecutive lanes.
-// FULL: every sample the group touches, 4m-1 .. 4m+4, lies in the stream
-// (sample -1 of the first group aside), so no load needs a bounds check.
+// Samples 4m .. 4m+3 of group m, in one 16-byte load when the stream is
+// aligned, and on lane 31 sample 4m+4 (the other lanes get theirs from the
+// next lane).  FULL: every sample the group touches, 4m-1 .. 4m+4, lies in the
+// stream (sample -1 of the first group aside), so no load needs a bounds check.
+struct IvtGroup {
+  float x0, x1, x2, x3, x4;
+};
+
 template <bool VEC, bool FULL>
-__device__ __forceinline__ unsigned ivt_group_starts(const IvtDev& P, long long m) {
+__device__ __forceinline__ IvtGroup ivt_load(const IvtDev& P, long long m) {
   const float nan = __int_as_float(0x7fc00000);
   const long long b = 4 * m;
   const float* xb = P.x + b;
-  float x0, x1, x2, x3;
+  IvtGroup g;
   if (VEC && (FULL || b + 3 < P.n)) {
     const float4 v = *reinterpret_cast<const float4*>(xb);
-    x0 = v.x; x1 = v.y; x2 = v.z; x3 = v.w;
+    g.x0 = v.x; g.x1 = v.y; g.x2 = v.z; g.x3 = v.w;
   } else if (FULL) {
-    x0 = xb[0]; x1 = xb[1]; x2 = xb[2]; x3 = xb[3];
+    g.x0 = xb[0]; g.x1 = xb[1]; g.x2 = xb[2]; g.x3 = xb[3];
   } else {
-    x0 = b < P.n ? xb[0] : nan;
-    x1 = b + 1 < P.n ? xb[1] : nan;
-    x2 = b + 2 < P.n ? xb[2] : nan;
-    x3 = b + 3 < P.n ? xb[3] : nan;
+    g.x0 = b < P.n ? xb[0] : nan;
+    g.x1 = b + 1 < P.n ? xb[1] : nan;
+    g.x2 = b + 2 < P.n ? xb[2] : nan;
+    g.x3 = b + 3 < P.n ? xb[3] : nan;
   }
+  g.x4 = nan;
+  if ((threadIdx.x & 31) == 31) g.x4 = (FULL || b + 4 < P.n) ? xb[4] : nan;
+  return g;
+}
+
+// Run starts among steps 4m+1 .. 4m+4 (bit i for step 4m+1+i) of a loaded
+// group.  Every lane of the warp calls it, with consecutive m on consecutive
+// lanes.  A start is a fast step, so a warp none of whose 128 steps is as
+// fast as the threshold (most of a recording is fixation) is done after one
+// test of its largest difference: multiplying by fs is monotonic in FP32, and
+// a NaN difference neither exceeds the threshold nor survives fmaxf.
+template <bool FULL>
+__device__ __forceinline__ unsigned ivt_group_starts(const IvtDev& P, long long m, const IvtGroup& g) {
+  const float x0 = g.x0, x1 = g.x1, x2 = g.x2, x3 = g.x3;
   const int lane = threadIdx.x & 31;
-  float xm = __shfl_up_sync(0xffffffffu, x3, 1);
   float x4 = __shfl_down_sync(0xffffffffu, x0, 1);
-  if (lane == 0) xm = (b >= 1 && (FULL || b - 1 < P.n)) ? xb[-1] : nan;
-  if (lane == 31) x4 = (FULL || b + 4 < P.n) ? xb[4] : nan;
+  if (lane == 31) x4 = g.x4;
+  const float top = fmaxf(fmaxf(fabsf(x1 - x0), fabsf(x2 - x1)), fmaxf(fabsf(x3 - x2), fabsf(x4 - x3)));
+  if (!__any_sync(0xffffffffu, top * P.fs > P.thr)) return 0u;
+  const float nan = __int_as_float(0x7fc00000);
+  const long long b = 4 * m;
+  float xm = __shfl_up_sync(0xffffffffu, x3, 1);
+  if (lane == 0) xm = (b >= 1 && (FULL || b - 1 < P.n)) ? P.x[b - 1] : nan;
   // per sample validity once, then fast steps 4m .. 4m+4 (step 0 does not
   // exist: sample -1 reads as NaN, which is not valid)
   const bool vm = ivt_valid(xm, P), v0 = ivt_valid(x0, P), v1 = ivt_valid(x1, P), v2 = ivt_valid(x2, P);
@@ -109,24 +129,27 @@ constexpr int kIvtRec = 64;   // run starts a tile records during the count pass
 
 // Pass 1a: run starts per tile; the first kIvtRec found are recorded as
 // tile-local step indices (step - first step of the tile, < kTile), in the
-// order the warps happen to claim slots.  The loop over the stream only
-// loads and tests (each thread's eight 4-bit start masks packed in one
-// word); the records collect in shared memory afterwards and go out at the
-// end.
+// order the warps happen to claim slots.  A thread's eight loads are issued
+// together, then tested (eight 4-bit start masks packed in one word); the
+// records collect in shared memory afterwards and go out at the end.
+template <bool VEC, bool FULL>
+__device__ __forceinline__ unsigned ivt_tile_starts(const IvtDev& P) {
+  IvtGroup g[kIvtIters];
+#pragma unroll
+  for (int it = 0; it < kIvtIters; ++it) g[it] = ivt_load<VEC, FULL>(P, ivt_group(it));
+  unsigned packed = 0;
+#pragma unroll
+  for (int it = 0; it < kIvtIters; ++it) packed |= ivt_group_starts<FULL>(P, ivt_group(it), g[it]) << (kVec * it);
+  return packed;
+}
+
 template <bool VEC>
 __global__ void __launch_bounds__(kIvtThreads) k_ivt_count(IvtDev P, int* tile_count, unsigned short* rec) {
   static_assert(kIvtIters * kVec <= 32, "start masks packed in one word");
   __shared__ int n_found;
   __shared__ unsigned short found[kIvtRec];
   if (threadIdx.x == 0) n_found = 0;
-  unsigned packed = 0;
-  if (ivt_tile_full(P)) {   // block-uniform
-#pragma unroll 4
-    for (int it = 0; it < kIvtIters; ++it) packed |= ivt_group_starts<VEC, true>(P, ivt_group(it)) << (kVec * it);
-  } else {
-#pragma unroll 4
-    for (int it = 0; it < kIvtIters; ++it) packed |= ivt_group_starts<VEC, false>(P, ivt_group(it)) << (kVec * it);
-  }
+  const unsigned packed = ivt_tile_full(P) ? ivt_tile_starts<VEC, true>(P) : ivt_tile_starts<VEC, false>(P);
   __syncthreads();
   const int lane = threadIdx.x & 31;
   if (__syncthreads_or(packed != 0u)) {             // block-uniform: most tiles of a fixation start nothing
@@ -157,15 +180,26 @@ __global__ void __launch_bounds__(kIvtThreads) k_ivt_count(IvtDev P, int* tile_c
   if (threadIdx.x == 0) tile_count[blockIdx.x] = c;
 }
 
-// Exclusive scan of the tile counts (one block of 1024 threads, each taking
-// a contiguous run of tiles); the total goes to *total.
-__global__ void __launch_bounds__(1024) k_ivt_scan(const int* tile_count, int ntiles, long long* tile_off,
-                                                   long long* total) {
+// Exclusive scan of n counts (one block of 1024 threads, each taking a
+// contiguous run of them).  The total and the largest count go to res, which
+// the host reads (pinned memory).
+struct ScanResult {
+  long long total;
+  long long largest;
+};
+
+__global__ void __launch_bounds__(1024) k_ivt_scan(const int* count, int n, long long* offset, ScanResult* res) {
   __shared__ long long warp_tot[32];
-  const int per = (ntiles + 1023) / 1024;
+  __shared__ int warp_max[32];
+  const int per = (n + 1023) / 1024;
   const int t0 = (int)threadIdx.x * per;
   long long mine = 0;
-  for (int i = t0; i < t0 + per && i < ntiles; ++i) mine += tile_count[i];
+  int most = 0;
+#pragma unroll 8
+  for (int i = t0; i < min(t0 + per, n); ++i) {
+    mine += count[i];
+    most = max(most, count[i]);
+  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   long long inc = mine;
 #pragma unroll
@@ -173,7 +207,11 @@ __global__ void __launch_bounds__(1024) k_ivt_scan(const int* tile_count, int nt
     const long long y = __shfl_up_sync(0xffffffffu, inc, o);
     if (lane >= o) inc += y;
   }
-  if (lane == 31) warp_tot[warp] = inc;
+  most = __reduce_max_sync(0xffffffffu, most);
+  if (lane == 31) {
+    warp_tot[warp] = inc;
+    warp_max[warp] = most;
+  }
   __syncthreads();
   if (warp == 0) {
     long long v = warp_tot[lane], wi = v;
@@ -183,13 +221,17 @@ __global__ void __launch_bounds__(1024) k_ivt_scan(const int* tile_count, int nt
       if (lane >= o) wi += y;
     }
     warp_tot[lane] = wi - v;   // exclusive prefix of the warps
-    if (lane == 31) *total = wi;
+    most = __reduce_max_sync(0xffffffffu, warp_max[lane]);
+    if (lane == 31) {
+      res->total = wi;
+      res->largest = most;
+    }
   }
   __syncthreads();
   long long run = warp_tot[warp] + inc - mine;
-  for (int i = t0; i < t0 + per && i < ntiles; ++i) {
-    tile_off[i] = run;
-    run += tile_count[i];
+  for (int i = t0; i < min(t0 + per, n); ++i) {
+    offset[i] = run;
+    run += count[i];
   }
 }
 
@@ -231,7 +273,7 @@ __global__ void __launch_bounds__(kIvtThreads) k_ivt_write(IvtDev P, const int* 
   long long run = tile_off[blockIdx.x];
   for (int it = 0; it < kIvtIters; ++it) {
     const long long m = ivt_group(it);
-    const unsigned bits = ivt_group_starts<VEC, false>(P, m);
+    const unsigned bits = ivt_group_starts<false>(P, m, ivt_load<VEC, false>(P, m));
     const int c = __popc(bits);
     int inc = c;
 #pragma unroll
@@ -256,8 +298,11 @@ __global__ void __launch_bounds__(kIvtThreads) k_ivt_write(IvtDev P, const int* 
 
 // Pass 2: one warp per run: the run's end (the first slow step, found 32
 // steps at a time), peak velocity, the window check, the event record;
-// keep[i] = 1 for a kept saccade.
-__global__ void k_ivt_events(IvtDev P, const long long* starts, int m, opmm_ivt_event* ev, int* keep) {
+// keep[i] = 1 for a kept saccade, counted in its group of kPackRuns runs.
+constexpr int kPackRuns = 1024;
+
+__global__ void k_ivt_events(IvtDev P, const long long* starts, int m, opmm_ivt_event* ev, unsigned char* keep,
+                             int* kept) {
   const int i = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (i >= m) return;
@@ -303,9 +348,36 @@ __global__ void k_ivt_events(IvtDev P, const long long* starts, int m, opmm_ivt_
     r.duration_ms = dur;
     r.peak_velocity_dps = peak;
     r.reserved = 0;
-    ev[i] = r;
+    if (ok) ev[i] = r;
     keep[i] = ok ? 1 : 0;
+    if (ok) atomicAdd(&kept[i / kPackRuns], 1);
   }
+}
+
+// Pass 3: the kept records of each group of kPackRuns runs at the group's
+// offset, in onset order, straight into the host's (pinned) array: the host
+// then copies whole ranges instead of picking records one by one.
+__global__ void __launch_bounds__(kPackRuns) k_ivt_pack(const opmm_ivt_event* ev, const unsigned char* keep, int m,
+                                                        const long long* offset, opmm_ivt_event* out) {
+  __shared__ int warp_cnt[kPackRuns / 32];
+  __shared__ unsigned short src[kPackRuns];
+  const int i = blockIdx.x * kPackRuns + (int)threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool ok = i < m && keep[i] != 0;
+  const unsigned mask = __ballot_sync(0xffffffffu, ok);
+  if (lane == 0) warp_cnt[warp] = __popc(mask);
+  __syncthreads();
+  int before = 0, all = 0;
+  for (int w = 0; w < kPackRuns / 32; ++w) {
+    before += w < warp ? warp_cnt[w] : 0;
+    all += warp_cnt[w];
+  }
+  if (ok) src[before + __popc(mask & ((1u << lane) - 1u))] = (unsigned short)threadIdx.x;
+  __syncthreads();
+  static_assert(sizeof(opmm_ivt_event) % 8 == 0, "records copied in 8-byte pieces");
+  constexpr int kPieces = (int)sizeof(opmm_ivt_event) / 8;
+  const uint2* from = reinterpret_cast<const uint2*>(ev + (size_t)blockIdx.x * kPackRuns);
+  uint2* to = reinterpret_cast<uint2*>(out + offset[blockIdx.x]);
+  for (int t = threadIdx.x; t < all * kPieces; t += kPackRuns) to[t] = from[src[t / kPieces] * kPieces + t % kPieces];
 }
 
 int ivt_fail(const Status& s) {
@@ -319,21 +391,20 @@ int ivt_fail(const Status& s) {
 
 using namespace opmm;
 
-extern "C" int opmm_detect_saccades(opmm_ctx* ctx, const float* stream_deg, int64_t n_samples, float sample_rate_hz,
-                                    const opmm_ivt_opts* opts, opmm_ivt_event* out, int32_t max_events,
-                                    int32_t* n_events) {
-  if (!ctx) return OPMM_EINVAL;
-  if (!stream_deg || !opts || !n_events || (max_events > 0 && !out))
-    return ivt_fail(Status(OPMM_EINVAL, "opmm_detect_saccades: null argument"));
+// The kept events in the context's pinned array, valid until the next call.
+static Status detect(opmm_ctx* ctx, const float* stream_deg, int64_t n_samples, float sample_rate_hz,
+                     const opmm_ivt_opts* opts, const opmm_ivt_event** events, size_t* found) {
+  if (!stream_deg || !opts) return Status(OPMM_EINVAL, "opmm_detect_saccades: null argument");
   if (n_samples < 2 || n_samples > (int64_t)1 << 40)
-    return ivt_fail(Status(OPMM_EINVAL, "opmm_detect_saccades: n_samples outside [2, 2^40]"));
+    return Status(OPMM_EINVAL, "opmm_detect_saccades: n_samples outside [2, 2^40]");
   if (!(sample_rate_hz > 0.0f) || !std::isfinite(sample_rate_hz) || !(opts->threshold_dps > 0.0f) ||
       !std::isfinite(opts->threshold_dps) || !(opts->min_duration_ms >= 0.0f) || !(opts->min_amplitude_deg >= 0.0f) ||
-      !(opts->valid_min_deg <= opts->valid_max_deg) || opts->pre_samples < 0 || opts->post_samples < 0 ||
-      max_events < 0)
-    return ivt_fail(Status(OPMM_EINVAL, "opmm_detect_saccades: bad options"));
+      !(opts->valid_min_deg <= opts->valid_max_deg) || opts->pre_samples < 0 || opts->post_samples < 0)
+    return Status(OPMM_EINVAL, "opmm_detect_saccades: bad options");
+  *events = nullptr;
+  *found = 0;
   Status s = cuda_status(cudaSetDevice(ctx->device), "cudaSetDevice");
-  if (!s.ok()) return ivt_fail(s);
+  if (!s.ok()) return s;
   cudaStream_t st = ctx->stream;
   const float* x = stream_deg;
   DevBuf& b_x = ctx->scratch[11];
@@ -343,12 +414,14 @@ extern "C" int opmm_detect_saccades(opmm_ctx* ctx, const float* stream_deg, int6
   DevBuf& b_count = ctx->scratch[15];
   DevBuf& b_off = ctx->scratch[10];
   DevBuf& b_rec = ctx->scratch[9];
+  HostBuf& h_ev = ctx->h_scratch[0];
+  HostBuf& h_res = ctx->h_scratch[1];
   if (!is_device_ptr(stream_deg)) {
     s = b_x.ensure(sizeof(float) * (size_t)n_samples);
     if (s.ok())
       s = cuda_status(cudaMemcpyAsync(b_x.ptr, stream_deg, sizeof(float) * (size_t)n_samples, cudaMemcpyHostToDevice, st),
                       "H2D stream");
-    if (!s.ok()) return ivt_fail(s);
+    if (!s.ok()) return s;
     x = b_x.as<float>();
   }
   IvtDev P{x, (long long)n_samples, sample_rate_hz, opts->threshold_dps, std::max(opts->valid_min_deg, -FLT_MAX),
@@ -356,63 +429,82 @@ extern "C" int opmm_detect_saccades(opmm_ctx* ctx, const float* stream_deg, int6
            opts->min_duration_ms, opts->min_amplitude_deg, opts->pre_samples, opts->post_samples};
   // run starts in stream order: count per tile, scan, write
   const long long ntiles_ll = (n_samples - 1 + kTile - 1) / kTile;
-  if (ntiles_ll > 0x7fffffffLL) return ivt_fail(Status(OPMM_EINVAL, "opmm_detect_saccades: stream too long"));
+  if (ntiles_ll > 0x7fffffffLL) return Status(OPMM_EINVAL, "opmm_detect_saccades: stream too long");
   const int ntiles = (int)ntiles_ll;
   s = b_count.ensure(sizeof(int) * (size_t)ntiles);
-  if (s.ok()) s = b_off.ensure(sizeof(long long) * ((size_t)ntiles + 1));
-  if (!s.ok()) return ivt_fail(s);
+  if (s.ok()) s = b_off.ensure(sizeof(long long) * (size_t)ntiles);
+  if (s.ok()) s = b_rec.ensure(sizeof(unsigned short) * kIvtRec * (size_t)ntiles);
+  if (s.ok()) s = h_res.ensure(2 * sizeof(ScanResult));
+  if (!s.ok()) return s;
   long long* d_off = b_off.as<long long>();
-  s = b_rec.ensure(sizeof(unsigned short) * kIvtRec * (size_t)ntiles);
-  if (!s.ok()) return ivt_fail(s);
   unsigned short* d_rec = b_rec.as<unsigned short>();
+  ScanResult* res = h_res.as<ScanResult>();   // [0] runs per tile, [1] kept runs per group
   const bool vec = (reinterpret_cast<uintptr_t>(x) & 15u) == 0;   // 16-byte loads need an aligned stream
   if (vec) k_ivt_count<true><<<ntiles, kIvtThreads, 0, st>>>(P, b_count.as<int>(), d_rec);
   else k_ivt_count<false><<<ntiles, kIvtThreads, 0, st>>>(P, b_count.as<int>(), d_rec);
-  k_ivt_scan<<<1, 1024, 0, st>>>(b_count.as<int>(), ntiles, d_off, d_off + ntiles);
+  k_ivt_scan<<<1, 1024, 0, st>>>(b_count.as<int>(), ntiles, d_off, &res[0]);
   s = cuda_status(cudaGetLastError(), "launch I-VT count");
-  long long total = 0;
-  if (s.ok()) s = cuda_status(cudaMemcpyAsync(&total, d_off + ntiles, sizeof total, cudaMemcpyDeviceToHost, st), "D2H runs");
   if (s.ok()) s = cuda_status(cudaStreamSynchronize(st), "I-VT count");
-  if (!s.ok()) return ivt_fail(s);
-  if (total > (1LL << 26))
-    return ivt_fail(Status(OPMM_ENOMEM, "opmm_detect_saccades: more than 2^26 velocity runs (raise the threshold)"));
-  const int m = (int)total;
-  // run records come back through pinned staging
-  HostBuf& h_ev = ctx->h_scratch[0];
-  HostBuf& h_keep = ctx->h_scratch[1];
-  if (m > 0) {
-    s = b_starts.ensure(sizeof(long long) * (size_t)m);
-    if (s.ok()) s = b_ev.ensure(sizeof(opmm_ivt_event) * (size_t)m);
-    if (s.ok()) s = b_keep.ensure(sizeof(int) * (size_t)m);
-    if (s.ok()) s = h_ev.ensure(sizeof(opmm_ivt_event) * (size_t)m);
-    if (s.ok()) s = h_keep.ensure(sizeof(int) * (size_t)m);
-    if (!s.ok()) return ivt_fail(s);
-    const long long warps_per_block = 4;
-    k_ivt_place<<<(unsigned)((ntiles + warps_per_block - 1) / warps_per_block), 32 * warps_per_block, 0, st>>>(
-        b_count.as<int>(), d_rec, d_off, ntiles, b_starts.as<long long>());
+  if (!s.ok()) return s;
+  if (res[0].total > (1LL << 26))
+    return Status(OPMM_ENOMEM, "opmm_detect_saccades: more than 2^26 velocity runs (raise the threshold)");
+  const int m = (int)res[0].total;
+  if (m == 0) return Status();
+  const int npack = (m + kPackRuns - 1) / kPackRuns;
+  s = b_starts.ensure(sizeof(long long) * (size_t)m);
+  if (s.ok()) s = b_ev.ensure(sizeof(opmm_ivt_event) * (size_t)m);
+  if (s.ok()) s = b_keep.ensure((size_t)npack * (sizeof(long long) + sizeof(int)) + (size_t)m);
+  if (s.ok()) s = h_ev.ensure(sizeof(opmm_ivt_event) * (size_t)m);
+  if (!s.ok()) return s;
+  long long* d_koff = b_keep.as<long long>();
+  int* d_kept = reinterpret_cast<int*>(d_koff + npack);
+  unsigned char* d_keep = reinterpret_cast<unsigned char*>(d_kept + npack);
+  const long long warps_per_block = 4;
+  k_ivt_place<<<(unsigned)((ntiles + warps_per_block - 1) / warps_per_block), 32 * warps_per_block, 0, st>>>(
+      b_count.as<int>(), d_rec, d_off, ntiles, b_starts.as<long long>());
+  if (res[0].largest > kIvtRec) {   // some tile has more starts than it records
     if (vec) k_ivt_write<true><<<ntiles, kIvtThreads, 0, st>>>(P, b_count.as<int>(), d_off, b_starts.as<long long>());
     else k_ivt_write<false><<<ntiles, kIvtThreads, 0, st>>>(P, b_count.as<int>(), d_off, b_starts.as<long long>());
-    k_ivt_events<<<(unsigned)((m + warps_per_block - 1) / warps_per_block), 32 * warps_per_block, 0, st>>>(
-        P, b_starts.as<long long>(), m, b_ev.as<opmm_ivt_event>(), b_keep.as<int>());
-    s = cuda_status(cudaGetLastError(), "launch I-VT events");
-    if (s.ok())
-      s = cuda_status(cudaMemcpyAsync(h_ev.ptr, b_ev.ptr, sizeof(opmm_ivt_event) * (size_t)m, cudaMemcpyDeviceToHost, st),
-                      "D2H events");
-    if (s.ok())
-      s = cuda_status(cudaMemcpyAsync(h_keep.ptr, b_keep.ptr, sizeof(int) * (size_t)m, cudaMemcpyDeviceToHost, st),
-                      "D2H keep");
-    if (s.ok()) s = cuda_status(cudaStreamSynchronize(st), "I-VT events");
-    if (!s.ok()) return ivt_fail(s);
   }
-  // kept events, already in onset order
+  s = cuda_status(cudaMemsetAsync(d_kept, 0, sizeof(int) * (size_t)npack, st), "clear kept counts");
+  if (!s.ok()) return s;
+  k_ivt_events<<<(unsigned)((m + warps_per_block - 1) / warps_per_block), 32 * warps_per_block, 0, st>>>(
+      P, b_starts.as<long long>(), m, b_ev.as<opmm_ivt_event>(), d_keep, d_kept);
+  k_ivt_scan<<<1, 1024, 0, st>>>(d_kept, npack, d_koff, &res[1]);
+  k_ivt_pack<<<npack, kPackRuns, 0, st>>>(b_ev.as<opmm_ivt_event>(), d_keep, m, d_koff, h_ev.as<opmm_ivt_event>());
+  s = cuda_status(cudaGetLastError(), "launch I-VT events");
+  if (s.ok()) s = cuda_status(cudaStreamSynchronize(st), "I-VT events");
+  if (!s.ok()) return s;
+  *events = h_ev.as<opmm_ivt_event>();
+  *found = (size_t)res[1].total;
+  return Status();
+}
+
+extern "C" int opmm_detect_saccades(opmm_ctx* ctx, const float* stream_deg, int64_t n_samples, float sample_rate_hz,
+                                    const opmm_ivt_opts* opts, opmm_ivt_event* out, int32_t max_events,
+                                    int32_t* n_events) {
+  if (!ctx) return OPMM_EINVAL;
+  if (!n_events || (max_events > 0 && !out))
+    return ivt_fail(Status(OPMM_EINVAL, "opmm_detect_saccades: null argument"));
+  if (max_events < 0) return ivt_fail(Status(OPMM_EINVAL, "opmm_detect_saccades: bad options"));
+  const opmm_ivt_event* ev = nullptr;
   size_t found = 0;
-  const opmm_ivt_event* hev = h_ev.as<opmm_ivt_event>();
-  const int* hkeep = h_keep.as<int>();
-  for (int i = 0; i < m; ++i) {
-    if (!hkeep[i]) continue;
-    if (found < (size_t)max_events) out[found] = hev[i];
-    ++found;
-  }
+  const Status s = detect(ctx, stream_deg, n_samples, sample_rate_hz, opts, &ev, &found);
+  if (!s.ok()) return ivt_fail(s);
+  const size_t n = std::min<size_t>(found, (size_t)max_events);
+  if (n > 0) std::memcpy(out, ev, n * sizeof(opmm_ivt_event));
   *n_events = (int32_t)std::min<size_t>(found, (size_t)0x7fffffff);
+  return OPMM_OK;
+}
+
+extern "C" int opmm_detect_saccades_view(opmm_ctx* ctx, const float* stream_deg, int64_t n_samples,
+                                         float sample_rate_hz, const opmm_ivt_opts* opts, const opmm_ivt_event** events,
+                                         int32_t* n_events) {
+  if (!ctx) return OPMM_EINVAL;
+  if (!events || !n_events) return ivt_fail(Status(OPMM_EINVAL, "opmm_detect_saccades: null argument"));
+  size_t found = 0;
+  const Status s = detect(ctx, stream_deg, n_samples, sample_rate_hz, opts, events, &found);
+  if (!s.ok()) return ivt_fail(s);
+  *n_events = (int32_t)found;
   return OPMM_OK;
 }
