@@ -182,16 +182,6 @@ static int fail(opmm_ctx* ctx, const Status& s) {
 
 static Status ctx_bind(opmm_ctx* ctx) { return cuda_status(cudaSetDevice(ctx->device), "cudaSetDevice"); }
 
-static Status ctx_check_error_word(opmm_ctx* ctx) {
-  unsigned h = 0;
-  Status s = cuda_status(cudaMemcpy(&h, ctx->d_err.as<unsigned>(), sizeof h, cudaMemcpyDeviceToHost),
-                         "read error word");
-  if (!s.ok()) return s;
-  if (h & kErrWaitTimeout) return Status(OPMM_ETIMEDOUT, "a kernel's bounded TMA wait expired");
-  if (h) return Status(OPMM_ECUDA, "kernel error bits " + std::to_string(h));
-  return Status();
-}
-
 extern "C" int opmm_create(int device_ordinal, opmm_ctx** out) {
   if (!out) return OPMM_EINVAL;
   *out = nullptr;
@@ -326,19 +316,6 @@ extern "C" int opmm_simulate(opmm_ctx* ctx, const float* opc, int32_t n, const o
   return OPMM_OK;
 }
 
-// Stage one saccade's trace into scratch slot `slot` (16-byte aligned,
-// zero-padded to a multiple of 4 samples).
-static Status stage_one(opmm_ctx* ctx, const opmm_saccade& s, DevBuf& buf, cudaStream_t st) {
-  const size_t lp = (size_t)((s.n_samples + 3) & ~3);
-  Status r = buf.ensure(lp * sizeof(float));
-  if (!r.ok()) return r;
-  r = cuda_status(cudaMemsetAsync(buf.ptr, 0, lp * sizeof(float), st), "clear trace");
-  if (!r.ok()) return r;
-  const cudaMemcpyKind kind = is_device_ptr(s.trace_deg) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  return cuda_status(cudaMemcpyAsync(buf.ptr, s.trace_deg, sizeof(float) * (size_t)s.n_samples, kind, st),
-                     "copy trace");
-}
-
 extern "C" int opmm_score(opmm_ctx* ctx, const float* opc, int32_t m, const opmm_saccade* sac, float* out_f) {
   if (!ctx) return OPMM_EINVAL;
   if (m < 0 || !sac || (m > 0 && (!opc || !out_f)) || !sac->trace_deg)
@@ -349,13 +326,15 @@ extern "C" int opmm_score(opmm_ctx* ctx, const float* opc, int32_t m, const opmm
   cudaStream_t st = ctx->stream;
   DevSac d = make_devsac(*sac);
   d.off = 0;
-  DevBuf& b_sac = ctx->scratch[0];
   DevBuf& b_opc = ctx->scratch[1];
   DevBuf& b_tr = ctx->scratch[5];
   DevBuf& b_f = ctx->scratch[6];
-  TRY(b_sac.ensure(sizeof(DevSac)));
-  CUDA_TRY(cudaMemcpyAsync(b_sac.ptr, &d, sizeof d, cudaMemcpyHostToDevice, st), "H2D descriptor");
-  TRY(stage_one(ctx, *sac, b_tr, st));
+  const float* d_trace = sac->trace_deg;
+  if (!is_device_ptr(d_trace)) {
+    TRY(b_tr.ensure(sizeof(float) * (size_t)d.L));
+    CUDA_TRY(cudaMemcpyAsync(b_tr.ptr, sac->trace_deg, sizeof(float) * (size_t)d.L, cudaMemcpyHostToDevice, st), "copy trace");
+    d_trace = b_tr.as<float>();
+  }
   const bool opc_dev = is_device_ptr(opc), f_dev = is_device_ptr(out_f);
   if (!opc_dev)
     for (int i = 0; i < m; ++i) TRY(check_opc(opc + (size_t)i * OPMM_NPARAM));
@@ -370,12 +349,9 @@ extern "C" int opmm_score(opmm_ctx* ctx, const float* opc, int32_t m, const opmm
     TRY(b_f.ensure(sizeof(float) * (size_t)m));
     d_f = b_f.as<float>();
   }
-  CUDA_TRY(cudaMemsetAsync(ctx->d_err.ptr, 0, sizeof(unsigned), st), "clear error word");
-  CUDA_TRY(launch_score(d_opc, m, b_sac.as<DevSac>(), d.L, b_tr.as<float>(), d_f, ctx->d_err.as<unsigned>(),
-                        ctx->num_sms, st), "launch score");
+  CUDA_TRY(launch_score(d_opc, m, d, d_trace, d_f, ctx->num_sms, st), "launch score");
   if (!f_dev) CUDA_TRY(cudaMemcpyAsync(out_f, d_f, sizeof(float) * (size_t)m, cudaMemcpyDeviceToHost, st), "D2H scores");
   CUDA_TRY(cudaStreamSynchronize(st), "score");
-  TRY(ctx_check_error_word(ctx));
   return OPMM_OK;
 }
 

@@ -69,13 +69,47 @@ struct KahanSink {
     sum = t;
     part = 0.0f;
   }
+  // mean over L samples, +inf when it is not finite
+  __device__ __forceinline__ float mean(int L) {
+    block_end();
+    const float f = (sum - c) / (float)L;
+    return isfinite(f) ? f : INFINITY;
+  }
 };
 
+// Writes a trajectory's samples, which come in order from k = 0, four at a
+// time where they fill an aligned 16-byte group.  Every thread of a warp
+// writes its own row, so a store of single samples touches 32 sectors for 128
+// bytes; in groups it takes a quarter of the transactions.
 struct WriteSink {
   float* out;
   float sign, thf;
-  __device__ __forceinline__ void emit(int k, float dth) { out[k] = sign * (thf + dth); }
+  int lead;            // samples by which out is past an aligned group
+  float b0, b1, b2;
+  __device__ __forceinline__ WriteSink(float* o, float sg, float th) : out(o), sign(sg), thf(th), b0(0), b1(0), b2(0) {
+    lead = (int)((reinterpret_cast<uintptr_t>(o) >> 2) & 3);
+  }
+  __device__ __forceinline__ void put(int k, float v) {
+    const int s = (lead + k) & 3;
+    if (k < s) {
+      out[k] = v;      // the row's first group is not whole
+      return;
+    }
+    if (s == 3) *reinterpret_cast<float4*>(out + k - 3) = make_float4(b0, b1, b2, v);
+    b0 = s == 0 ? v : b0;
+    b1 = s == 1 ? v : b1;
+    b2 = s == 2 ? v : b2;
+  }
+  __device__ __forceinline__ void emit(int k, float dth) { put(k, sign * (thf + dth)); }
   __device__ __forceinline__ void block_end() {}
+  // the n samples' last, partial group
+  __device__ __forceinline__ void finish(int n) {
+    const int s = (lead + n) & 3;
+    if (n < s) return;
+    if (s > 0) out[n - s] = b0;
+    if (s > 1) out[n - s + 1] = b1;
+    if (s > 2) out[n - s + 2] = b2;
+  }
 };
 
 struct PeakSink {
@@ -87,15 +121,12 @@ struct PeakSink {
 // Objective of one OPC vector: mean squared error over the window; the
 // samples up to onset (the plant at rest) are folded into (sum0, c0).
 // pe (optional): set to 1 when the pulse ends inside the window.
-template <bool SYNC = false, bool PACK = false>
+template <bool PACK>
 __device__ __forceinline__ float objective(const float* p, const SacConst& sc, const float* z,
-                                           float sum0, float c0, float* qs = nullptr, int qstride = 0,
-                                           int* pe = nullptr, unsigned mask = 0xffffffffu) {
+                                           float sum0, float c0, float* qs, int qstride, int* pe, unsigned mask) {
   KahanSink s{z, sum0, c0, 0.0f};
-  if (walk<KahanSink, SYNC, PACK>(p, sc, s, qs, qstride, true, pe, mask) < 0) return INFINITY;
-  s.block_end();
-  const float f = (s.sum - s.c) / (float)sc.L;
-  return isfinite(f) ? f : INFINITY;
+  if (walk<KahanSink, true, PACK>(p, sc, s, qs, qstride, true, pe, mask) < 0) return INFINITY;
+  return s.mean(sc.L);
 }
 
 // Parameter sources of the register-lean walk: each load() re-derives the
@@ -129,6 +160,26 @@ struct TraceStage {
   float sum0, c0;
 };
 
+// The positive-frame trace minus the end fixation into z, and the compensated
+// sum of the rest samples (all threads; y in shared or global memory).
+__device__ __forceinline__ void shift_trace(const DevSac& d, const float* y, float* z, TraceStage* st) {
+  for (int k = threadIdx.x; k < d.L; k += blockDim.x) z[k] = d.sign * y[k] - d.thf;
+  if (threadIdx.x == 0) {
+    float sum = 0.0f, c = 0.0f;
+    const int kend = min(d.onset, d.L - 1);
+    for (int k = 0; k <= kend; ++k) {
+      const float e = d.th0 - d.sign * y[k];
+      const float q = fmaf(e, e, -c);
+      const float t = sum + q;
+      c = (t - sum) - q;
+      sum = t;
+    }
+    st->sum0 = sum;
+    st->c0 = c;
+  }
+  __syncthreads();
+}
+
 __device__ bool stage_trace(const DevSac& d, const float* traces, float* yraw, float* z, uint64_t* bar,
                             uint32_t& phase, TraceStage* st) {
   if (threadIdx.x == 0) {
@@ -140,35 +191,30 @@ __device__ bool stage_trace(const DevSac& d, const float* traces, float* yraw, f
   const bool ok = mbar_wait(bar, phase, kMaxWaitTries);
   phase ^= 1u;
   if (__syncthreads_or(!ok)) return false;
-  for (int k = threadIdx.x; k < d.L; k += blockDim.x) z[k] = d.sign * yraw[k] - d.thf;
-  if (threadIdx.x == 0) {
-    float sum = 0.0f, c = 0.0f;
-    const int kend = min(d.onset, d.L - 1);
-    for (int k = 0; k <= kend; ++k) {
-      const float e = d.th0 - d.sign * yraw[k];
-      const float y = fmaf(e, e, -c);
-      const float t = sum + y;
-      c = (t - sum) - y;
-      sum = t;
-    }
-    st->sum0 = sum;
-    st->c0 = c;
-  }
-  __syncthreads();
+  shift_trace(d, yraw, z, st);
   return true;
 }
 
 // ------------------------------------------------------------------ nominal
-// Largest sample of the default plant's saccade from 0 to A with agonist
-// pulse nsac, 1 kHz grid, 250 ms after onset.
-__device__ float nominal_peak(float* p, float A, float nsac) {
-  p[kNsacAg] = nsac;
+// The default plant's saccade from 0 to A, 1 kHz grid, 250 ms after onset; its
+// propagators do not depend on the agonist pulse, so one set-up serves all the
+// pulses tried (a set-up per pulse, in scalar arithmetic: 615 us against 507 for
+// 10,000 saccades).
+struct NominalWalk {
   SacConst sc;
-  sc.L = 251; sc.onset = 0; sc.nsub = 10; sc.fs = 1000.0f; sc.h = 1.0e-4f; sc.th0 = 0.0f; sc.thf = A;
-  PeakSink pk{-A};
-  walk(p, sc, pk);
-  return A + pk.m;
-}
+  PackedWalk w;
+  __device__ __forceinline__ NominalWalk(const float* p, float A) {
+    sc.L = 251; sc.onset = 0; sc.nsub = 10; sc.fs = 1000.0f; sc.h = 1.0e-4f; sc.th0 = 0.0f; sc.thf = A;
+    w.setup(p, sc);
+  }
+  // largest sample with agonist pulse nsac
+  __device__ __forceinline__ float peak(float* p, float nsac) {
+    p[kNsacAg] = nsac;
+    PeakSink pk{-sc.thf};
+    w.samples(p, sc, pk);
+    return sc.thf + pk.m;
+  }
+};
 
 // One warp per saccade.  Calibrated mode: the agonist pulse for which the
 // default plant's saccade peaks at its amplitude A; round 0 brackets the
@@ -195,7 +241,8 @@ __global__ void k_nominal(const DevSac* sacs, int n, int pulse_mode, const float
     float s[6];
     rest_state(p, A, s);
     const float lo = s[4];
-    float pk = nominal_peak(p, A, lo * ldexpf(1.0f, lane));
+    NominalWalk nw(p, A);
+    float pk = nw.peak(p, lo * ldexpf(1.0f, lane));
     unsigned hit = __ballot_sync(0xffffffffu, pk >= A);
     if (hit & 1u) {
       nsac = lo;
@@ -205,9 +252,10 @@ __global__ void k_nominal(const DevSac* sacs, int n, int pulse_mode, const float
       const int i0 = __ffs(hit) - 1;
       float a = lo * ldexpf(1.0f, i0 - 1);
       float bb = lo * ldexpf(1.0f, i0);
+#pragma unroll 1
       for (int round = 0; round < 6; ++round) {
         const float x = a + (bb - a) * ((float)(lane + 1) * (1.0f / 33.0f));
-        pk = nominal_peak(p, A, x);
+        pk = nw.peak(p, x);
         const unsigned h = __ballot_sync(0xffffffffu, pk >= A);
         const int i = h ? __ffs(h) - 1 : 32;
         const float xlo = __shfl_sync(0xffffffffu, x, i > 0 ? i - 1 : 0);
@@ -237,36 +285,35 @@ __global__ void k_simulate(const float* opc, int n, const DevSac* sacs, const in
   for (int j = 0; j < kNumParams; ++j) p[j] = opc[(size_t)i * kNumParams + j];
   const DevSac d = sacs[sac_of ? sac_of[i] : i];
   const SacConst sc = sac_const(d);
-  float* o = out + out_off[i];
+  WriteSink w(out + out_off[i], d.sign, d.thf);
   const int kend = min(d.onset, d.L - 1);
-  for (int k = 0; k <= kend; ++k) o[k] = d.sign * d.th0;
-  WriteSink w{o, d.sign, d.thf};
-  walk(p, sc, w);
+  for (int k = 0; k <= kend; ++k) w.put(k, d.sign * d.th0);
+  PackedWalk pw;
+  pw.setup(p, sc);
+  pw.samples(p, sc, w);
+  w.finish(d.L);
 }
 
 // ------------------------------------------------------------------ score
-__global__ void k_score(const float* opc, int m, const DevSac* sac, const float* traces, float* f,
-                        unsigned* err) {
+constexpr int kScoreThreads = 128;
+
+// One launch and nothing around it: the descriptor is an argument, and each
+// block reads the trace where the caller keeps it (any alignment, a few
+// hundred samples) instead of a padded copy by TMA, whose staging, error word
+// and second synchronisation were half of a call's time.
+__global__ void __launch_bounds__(kScoreThreads) k_score(const float* opc, int m, const __grid_constant__ DevSac d,
+                                                         const float* trace, float* f) {
   extern __shared__ __align__(128) unsigned char smraw[];
-  __shared__ __align__(8) uint64_t bar;
   __shared__ TraceStage st;
-  const DevSac d = *sac;
-  const int lp = (d.L + 3) & ~3;
-  float* yraw = reinterpret_cast<float*>(smraw);
-  float* z = yraw + lp;
-  if (threadIdx.x == 0) { mbar_init(&bar, 1); fence_mbar_init(); }
-  __syncthreads();
-  uint32_t phase = 0;
-  if (!stage_trace(d, traces, yraw, z, &bar, phase, &st)) {
-    if (threadIdx.x == 0) raise_error(err, kErrWaitTimeout);
-    return;
-  }
+  float* z = reinterpret_cast<float*>(smraw);
+  shift_trace(d, trace, z, &st);
   const SacConst sc = sac_const(d);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
     float p[kNumParams];
 #pragma unroll
     for (int j = 0; j < kNumParams; ++j) p[j] = opc[(size_t)i * kNumParams + j];
-    f[i] = objective(p, sc, z, st.sum0, st.c0);
+    KahanSink s{z, st.sum0, st.c0, 0.0f};
+    f[i] = walk(p, sc, s, nullptr, 0, true) < 0 ? INFINITY : s.mean(sc.L);
   }
 }
 
@@ -431,9 +478,7 @@ __device__ __forceinline__ float objective_lean(const ULinSrc& src, const SacCon
   }
   KahanSink s{z, sum0, c0, 0.0f};
   walk_lean(src, sc, s, pe);
-  s.block_end();
-  const float f = (s.sum - s.c) / (float)sc.L;
-  return isfinite(f) ? f : INFINITY;
+  return s.mean(sc.L);
 }
 
 // Objective of search point u; the lanes in `mask` call it together and
@@ -444,7 +489,7 @@ __device__ __forceinline__ float eval_u(const float (&u)[N], const float* pc, fl
                                         float c0, float* qs, int qstride, int* pe, unsigned mask) {
   float p[kNumParams];
   u_to_p<N>(u, pc, lnlo, lnhi, p);
-  return objective<true, PACK>(p, sc, z, sum0, c0, qs, qstride, pe, mask);
+  return objective<PACK>(p, sc, z, sum0, c0, qs, qstride, pe, mask);
 }
 
 // Rows of trial point q of simplex gi, as u = a + (b - a) / 2 coordinate by
@@ -1920,18 +1965,17 @@ cudaError_t launch_simulate(const float* opc, int n, const DevSac* sacs, const i
   return cudaGetLastError();
 }
 
-cudaError_t launch_score(const float* opc, int m, const DevSac* sac, int L, const float* traces, float* f,
-                         unsigned* err, int num_sms, cudaStream_t st) {
+cudaError_t launch_score(const float* opc, int m, const DevSac& sac, const float* trace, float* f, int num_sms,
+                         cudaStream_t st) {
   if (m <= 0) return cudaSuccess;
-  const int threads = 256;
-  int blocks = (m + threads - 1) / threads;
-  if (blocks > 4 * num_sms) blocks = 4 * num_sms;
-  const size_t smem = 2 * (size_t)((L + 3) & ~3) * sizeof(float);
+  int blocks = (m + kScoreThreads - 1) / kScoreThreads;
+  if (blocks > 8 * num_sms) blocks = 8 * num_sms;
+  const size_t smem = (size_t)sac.L * sizeof(float);
   if (smem > 48 * 1024) {
     cudaError_t e = allow_dynamic_smem(k_score, smem);
     if (e != cudaSuccess) return e;
   }
-  k_score<<<blocks, threads, smem, st>>>(opc, m, sac, traces, f, err);
+  k_score<<<blocks, kScoreThreads, smem, st>>>(opc, m, sac, trace, f);
   return cudaGetLastError();
 }
 

@@ -47,8 +47,8 @@ cudaError_t launch_nominal(const DevSac* sacs, int n, int pulse_mode, const floa
                            cudaStream_t st);
 cudaError_t launch_simulate(const float* opc, int n, const DevSac* sacs, const int* sac_of,
                             const long long* out_off, float* out, cudaStream_t st);
-cudaError_t launch_score(const float* opc, int m, const DevSac* sac, int L, const float* traces, float* f,
-                         unsigned* err, int num_sms, cudaStream_t st);
+cudaError_t launch_score(const float* opc, int m, const DevSac& sac, const float* trace, float* f, int num_sms,
+                         cudaStream_t st);   // trace: the saccade's samples, any alignment
 // Search kernel variants (see kernels.cu): unit size (simplices per block),
 // search coordinates (18, or 9 for the 9-parameter model), threads and
 // dynamic shared memory per block.

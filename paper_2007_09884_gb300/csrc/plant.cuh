@@ -409,6 +409,66 @@ __device__ __forceinline__ void prop_pow(const Prop2& q, int n, Prop2& out) {
   }
 }
 
+// r = a + b + a b (increment form of (I + a)(I + b)), two columns per packed
+// FP32 instruction; r may alias neither.
+__device__ __forceinline__ void prop_mul_x2(const Prop2& a, const Prop2& b, Prop2& r) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+#pragma unroll
+    for (int j = 0; j < 4; j += 2) {
+      float2 acc = __fadd2_rn(f2(a.m[i][j], a.m[i][j + 1]), f2(b.m[i][j], b.m[i][j + 1]));
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) acc = __ffma2_rn(bc(a.m[i][kk]), f2(b.m[kk][j], b.m[kk][j + 1]), acc);
+      r.m[i][j] = acc.x;
+      r.m[i][j + 1] = acc.y;
+    }
+#pragma unroll
+    for (int ph = 0; ph < 2; ++ph) {
+      const float (&ac)[4][2] = ph == 0 ? a.c1 : a.c2;
+      const float (&bb)[4][2] = ph == 0 ? b.c1 : b.c2;
+      const float (&bd)[2] = ph == 0 ? b.d1 : b.d2;
+      float (&rc)[4][2] = ph == 0 ? r.c1 : r.c2;
+      const float2 ai = f2(ac[i][0], ac[i][1]);
+      float2 acc = __ffma2_rn(ai, f2(bd[0], bd[1]), __fadd2_rn(ai, f2(bb[i][0], bb[i][1])));
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) acc = __ffma2_rn(bc(a.m[i][kk]), f2(bb[kk][0], bb[kk][1]), acc);
+      rc[i][0] = acc.x;
+      rc[i][1] = acc.y;
+    }
+  }
+#pragma unroll
+  for (int ph = 0; ph < 2; ++ph) {
+    const float (&ad)[2] = ph == 0 ? a.d1 : a.d2;
+    const float (&bd)[2] = ph == 0 ? b.d1 : b.d2;
+    float (&rd)[2] = ph == 0 ? r.d1 : r.d2;
+    const float2 x = f2(ad[0], ad[1]), y = f2(bd[0], bd[1]);
+    const float2 d = __ffma2_rn(x, y, __fadd2_rn(x, y));
+    rd[0] = d.x;
+    rd[1] = d.y;
+  }
+}
+
+// out = (I + q)^n - I by binary powering (n >= 1).
+__device__ __forceinline__ void prop_pow_x2(const Prop2& q, int n, Prop2& out) {
+  Prop2 base = q, tmp;
+  bool have = false;
+  while (true) {
+    if (n & 1) {
+      if (have) {
+        prop_mul_x2(out, base, tmp);
+        out = tmp;
+      } else {
+        out = base;
+        have = true;
+      }
+    }
+    n >>= 1;
+    if (!n) break;
+    prop_mul_x2(base, base, tmp);
+    base = tmp;
+  }
+}
+
 // Single-phase increment propagator: the mechanical block plus one phase's
 // coupling and activation blocks (26 floats).
 struct Prop1 {
@@ -936,6 +996,87 @@ __device__ __forceinline__ int walk(const float* p, const SacConst& sc0, Sink& s
   }
   return ntot;
 }
+
+// Where the pulse ends: n1 whole pulse-phase samples, then (when it ends
+// inside the window) jsw whole substeps and the fraction frac of the next.
+struct PulseEnd {
+  int n1, jsw;
+  float frac;
+  bool sw;
+  __device__ __forceinline__ PulseEnd(float pw, const SacConst& sc, int nsub) {
+    const int ntot = sc.L - 1 - sc.onset;
+    float tau = pw * sc.fs * (float)nsub * 1e-3f;   // in substeps after onset
+    tau = fminf(fmaxf(tau, 0.0f), 1.0e9f);
+    const float jf = floorf(tau);
+    frac = tau - jf;
+    const float span = (float)ntot * (float)nsub;
+    jsw = 0;
+    if (jf >= span) {
+      n1 = ntot;
+      sw = false;
+    } else {
+      const int J = (int)jf;
+      n1 = J / nsub;
+      jsw = J - n1 * nsub;
+      sw = true;
+    }
+  }
+};
+
+// The walk without a slot in packed arithmetic (trajectories, calibration):
+// bit for bit the walk called without one.  It is a second copy because the
+// search kernel's walk loses a quarter of its speed when these steps are shared
+// functions (a batch fit 420 -> 465 ms: the compiler then no longer keeps the
+// row pairs together).  The set-up (coefficients, propagators) and the samples
+// are separate, so that one set-up serves several pulse heights.
+struct PackedWalk {
+  Coef k;
+  Prop2 q, phi;   // single substep, one sample
+  float h;
+  int nsub;
+  // false: too stiff even for the finest substep
+  __device__ __forceinline__ bool setup(const float* p, const SacConst& sc) {
+    make_coef(p, k);
+    const int rs = refine_shift(k, sc.h);
+    const int sh = rs < 0 ? kMaxRefine : rs;
+    nsub = sc.nsub << sh;
+    h = sc.h * pow2neg(sh);
+    step_increment_x2(k, h, q);
+    prop_pow_x2(q, nsub, phi);
+    return rs >= 0;
+  }
+  template <class Sink>
+  __device__ __forceinline__ void samples(const float* p, const SacConst& sc, Sink& sink) const {
+    const int ntot = sc.L - 1 - sc.onset;
+    if (ntot <= 0) return;
+    const PulseEnd pe(p[kPw], sc, nsub);
+    float s0[6], s1[6], s2[6];
+    rest_state_k(p, k, sc.th0, s0);
+    drive_equilibrium_k(p, k, p[kNsacAg], p[kNsacAnt], s1);
+    rest_state_k(p, k, sc.thf, s2);
+    float e[6], dl[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      e[i] = s0[i] - s1[i];
+      dl[i] = s1[i] - s2[i];
+    }
+    int kk = sc.onset + 1;
+    run_samples_v<1, true>(phi, e, s1[0] - sc.thf, kk, pe.n1, sink);
+    if (!pe.sw) return;
+    const float h1 = pe.frac * h;
+    PropX2 x;
+    pack_phase<1>(q, x);
+    for (int s = 0; s < pe.jsw; ++s) prop_apply_x2(x, e);
+    rk4_vec(k, k.da1, k.dn1, h1, e);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) e[i] += dl[i];
+    rk4_vec(k, k.da2, k.dn2, h - h1, e);
+    pack_phase<2>(q, x);
+    for (int s = pe.jsw + 1; s < nsub; ++s) prop_apply_x2(x, e);
+    sink.emit(kk++, e[0]);
+    run_samples_v<2, true>(phi, e, 0.0f, kk, ntot - pe.n1 - 1, sink);
+  }
+};
 
 // Single-phase version of run_samples.
 template <class Sink>
