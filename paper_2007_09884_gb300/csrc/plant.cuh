@@ -296,28 +296,40 @@ __device__ __forceinline__ void zm_mul_x2(const float2 (&Z)[9], const float2 (&w
   o[3] = __ffma2_rn(Z[8], w[3], __fmul2_rn(Z[7], w[0]));
 }
 
+// The first Horner level multiplies the identity (mechanical block) or two
+// single entries (coupling), so its products are Zm's own entries or a few
+// products; those are written out, since a packed multiplication by 0 or 1 is
+// not folded away.  (A dropped product with 0 can only change the sign of a
+// zero, which the next level's sum absorbs.)
 __device__ __forceinline__ void step_increment_x2(const Coef& k, float h, Prop2& q) {
-  const float2 Z[9] = {bc(h), bc(h * k.m10), bc(h * k.m11), bc(h * k.m12), bc(h * k.m13),
-                       bc(h * k.m20), bc(h * k.m22), bc(h * k.m30), bc(h * k.m33)};
+  const float z10 = h * k.m10, z11 = h * k.m11, z12 = h * k.m12, z13 = h * k.m13;
+  const float z20 = h * k.m20, z22 = h * k.m22, z30 = h * k.m30, z33 = h * k.m33;
+  const float2 Z[9] = {bc(h), bc(z10), bc(z11), bc(z12), bc(z13), bc(z20), bc(z22), bc(z30), bc(z33)};
   const float zcx = h * k.cx, zcy = h * k.cy;
   // mechanical block, column pairs jp = 0 (columns 0, 1) and 1 (columns 2, 3)
 #pragma unroll
   for (int jp = 0; jp < 2; ++jp) {
     float2 id[4], w[4], t[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      id[i] = f2(i == 2 * jp ? 1.0f : 0.0f, i == 2 * jp + 1 ? 1.0f : 0.0f);
-      w[i] = id[i];
+    for (int i = 0; i < 4; ++i) id[i] = f2(i == 2 * jp ? 1.0f : 0.0f, i == 2 * jp + 1 ? 1.0f : 0.0f);
+    // W3 = I + Zm / 4
+    if (jp == 0) {
+      w[0] = f2(1.0f, 0.25f * h);
+      w[1] = f2(0.25f * z10, __fadd_rn(1.0f, 0.25f * z11));
+      w[2] = f2(0.25f * z20, 0.0f);
+      w[3] = f2(0.25f * z30, 0.0f);
+    } else {
+      w[0] = f2(0.0f, 0.0f);
+      w[1] = f2(0.25f * z12, 0.25f * z13);
+      w[2] = f2(__fadd_rn(1.0f, 0.25f * z22), 0.0f);
+      w[3] = f2(0.0f, __fadd_rn(1.0f, 0.25f * z33));
     }
-    zm_mul_x2(Z, w, t);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) w[i] = __fadd2_rn(id[i], __fmul2_rn(bc(0.25f), t[i]));
     zm_mul_x2(Z, w, t);
 #pragma unroll
     for (int i = 0; i < 4; ++i) w[i] = __ffma2_rn(t[i], bc(1.0f / 3.0f), id[i]);
     zm_mul_x2(Z, w, t);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) w[i] = __fadd2_rn(id[i], __fmul2_rn(bc(0.5f), t[i]));
+    for (int i = 0; i < 4; ++i) w[i] = __ffma2_rn(t[i], bc(0.5f), id[i]);
     zm_mul_x2(Z, w, t);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -325,40 +337,42 @@ __device__ __forceinline__ void step_increment_x2(const Coef& k, float h, Prop2&
       q.m[i][2 * jp + 1] = t[i].y;
     }
   }
-  // coupling and activation blocks, per phase; the pair is (column Fa, column Fn)
+  // coupling and activation blocks, per phase; the pair is (column Fa, column
+  // Fn).  Rows 2 and 3 of the coupling hold one entry each until the last
+  // level: dg is the pair (row 2 column Fa, row 3 column Fn).
+  const float2 zc = f2(zcx, zcy), zo = f2(z12, z13), zd = f2(z22, z33);
 #pragma unroll
   for (int ph = 0; ph < 2; ++ph) {
-    const float zda = h * (ph == 0 ? k.da1 : k.da2);
-    const float zdn = h * (ph == 0 ? k.dn1 : k.dn2);
-    float2 wc[4] = {f2(0.f, 0.f), f2(0.f, 0.f), f2(0.25f * zcx, 0.f), f2(0.f, 0.25f * zcy)};
-    float wda = 1.0f + 0.25f * zda, wdn = 1.0f + 0.25f * zdn;
-    float2 tc[4];
-    zm_mul_x2(Z, wc, tc);
-    tc[2].x = fmaf(zcx, wda, tc[2].x);
-    tc[3].y = fmaf(zcy, wdn, tc[3].y);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) wc[i] = __fmul2_rn(tc[i], bc(1.0f / 3.0f));
-    wda = __fmaf_rn(__fmul_rn(zda, wda), 1.0f / 3.0f, 1.0f);
-    wdn = __fmaf_rn(__fmul_rn(zdn, wdn), 1.0f / 3.0f, 1.0f);
-    zm_mul_x2(Z, wc, tc);
-    tc[2].x = fmaf(zcx, wda, tc[2].x);
-    tc[3].y = fmaf(zcy, wdn, tc[3].y);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) wc[i] = __fmul2_rn(bc(0.5f), tc[i]);
-    wda = __fmaf_rn(0.5f * zda, wda, 1.0f);
-    wdn = __fmaf_rn(0.5f * zdn, wdn, 1.0f);
-    zm_mul_x2(Z, wc, tc);
-    tc[2].x = fmaf(zcx, wda, tc[2].x);
-    tc[3].y = fmaf(zcy, wdn, tc[3].y);
+    const float2 za = __fmul2_rn(bc(h), ph == 0 ? f2(k.da1, k.dn1) : f2(k.da2, k.dn2));
+    float2 dg = __fmul2_rn(bc(0.25f), zc);                        // level 3: Wc3 = Zc / 4
+    float2 wd = __ffma2_rn(bc(0.25f), za, bc(1.0f));              // Wd3 = 1 + Zd / 4
+    // level 2: Wc2 = (Zm Wc3 + Zc Wd3) / 3, Wd2 = 1 + Zd Wd3 / 3
+    float2 w1 = __fmul2_rn(__fmul2_rn(zo, dg), bc(1.0f / 3.0f));
+    dg = __fmul2_rn(__ffma2_rn(zc, wd, __fmul2_rn(zd, dg)), bc(1.0f / 3.0f));
+    wd = __ffma2_rn(__fmul2_rn(za, wd), bc(1.0f / 3.0f), bc(1.0f));
+    // level 1: Wc1 = (Zm Wc2 + Zc Wd2) / 2, Wd1 = 1 + Zd Wd2 / 2
+    const float2 w0 = __fmul2_rn(bc(0.5f), __fmul2_rn(Z[0], w1));
+    w1 = __fmul2_rn(bc(0.5f), __ffma2_rn(zo, dg, __fmul2_rn(Z[2], w1)));
+    dg = __fmul2_rn(bc(0.5f), __ffma2_rn(zc, wd, __fmul2_rn(zd, dg)));
+    wd = __ffma2_rn(__fmul2_rn(bc(0.5f), za), wd, bc(1.0f));
+    // Q: Qc = Zm Wc1 + Zc Wd1, Qd = Zd Wd1
+    const float2 c0 = __fmul2_rn(Z[0], w1);
+    const float2 c1 = __ffma2_rn(zo, dg, __ffma2_rn(Z[2], w1, __fmul2_rn(Z[1], w0)));
+    const float2 r2 = __fmul2_rn(Z[5], w0), r3 = __fmul2_rn(Z[7], w0);
+    dg = __ffma2_rn(zc, wd, __ffma2_rn(zd, dg, f2(r2.x, r3.y)));
+    const float2 d2 = __fmul2_rn(za, wd);
     float (&c)[4][2] = ph == 0 ? q.c1 : q.c2;
     float (&d)[2] = ph == 0 ? q.d1 : q.d2;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      c[i][0] = tc[i].x;
-      c[i][1] = tc[i].y;
-    }
-    d[0] = zda * wda;
-    d[1] = zdn * wdn;
+    c[0][0] = c0.x;
+    c[0][1] = c0.y;
+    c[1][0] = c1.x;
+    c[1][1] = c1.y;
+    c[2][0] = dg.x;
+    c[2][1] = r2.y;
+    c[3][0] = r3.x;
+    c[3][1] = dg.y;
+    d[0] = d2.x;
+    d[1] = d2.y;
   }
 }
 
