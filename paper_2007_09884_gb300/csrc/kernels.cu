@@ -1161,15 +1161,17 @@ __global__ void __launch_bounds__(search_threads<G, N>(), MINB) k_search(SearchP
 // into two RK4 steps.  Independent of the FP32 search formulation (double
 // precision, matrix powers instead of substeps, its own equilibria).
 //
-// The FP64 pipe bounds it (two lanes per SM and clock: a warp instruction
-// holds the SM's pipe for about 16 cycles however many lanes it uses), so
-// every lane carries work.  Matrices keep the plant's block form (a 4x4
-// mechanical block, a 4x2 coupling, a diagonal activation pair: 26 entries)
-// with one entry per lane, five FMAs a product; and a phase's samples go 32
-// at a time, lane l holding the state after sample l + 1: five predicated
-// steps by (I + P)^1, ^2, ^4, ^8, ^16 start the lanes, (I + P)^32 moves them.
-// One thread per saccade with dense 6x6 matrices in local memory took 365 us
-// for one saccade of 150 samples and 880 us for 2,000 uneven ones.
+// The FP64 pipes bound it: a warp instruction holds its sub-partition's for
+// about 64 cycles however many lanes it uses, so the count of warp
+// instructions is what is kept small and every lane carries work.  Matrices
+// keep the plant's block form (a 4x4 mechanical block, a 4x2 coupling, a
+// diagonal activation pair: 26 entries) with one entry per lane, five FMAs a
+// product; vectors go one row per lane; and a phase's samples go 32 at a
+// time, lane l holding the state after sample l + 1: the first 32 states come
+// by doubling ((I + P)^c takes states 1 .. c to c + 1 .. 2 c, one row of one
+// state per lane), (I + P)^32 moves them on.  One thread per saccade with
+// dense 6x6 matrices in local memory took 365 us for one saccade of 150
+// samples and 880 us for 2,000 uneven ones.
 
 // Products by entry: entry e of a 32-double matrix is m[e / 4][e % 4] for
 // e < 16, c[(e - 16) / 2][(e - 16) % 2] for e < 24, d[e - 24] for e < 26 and
@@ -1214,6 +1216,8 @@ struct Lane64 {
 
 struct Warp64 {
   double A[32], Q[32], W[32], B[32], P[6][32];
+  double E[32][6];               // states after samples 1 .. 32 of a phase
+  double v[6];                   // the walk's current state
   double par[kNumParams], rcp[12];
   float opc[kNumParams];
 };
@@ -1221,7 +1225,7 @@ struct Warp64 {
 // out = T4(h A) - I by Horner (w: scratch).
 __device__ void step_inc64(const Lane64& L, const double* A, double h, double* w, double* out) {
   L.put(w, fma(0.25 * h, A[L.e], L.unit));
-  L.put(w, fma(h / 3.0, L.mul(A, w), L.unit));
+  L.put(w, fma(h * (1.0 / 3.0), L.mul(A, w), L.unit));
   L.put(w, fma(0.5 * h, L.mul(A, w), L.unit));
   L.put(out, h * L.mul(A, w));
 }
@@ -1231,10 +1235,10 @@ __device__ __forceinline__ void mul_inc64(const Lane64& L, const double* a, cons
   L.put(r, a[L.e] + b[L.e] + L.mul(a, b));
 }
 
-// out = (I + q)^n - I for n >= 0 (left to right; out is not q).
+// out = (I + q)^n - I for n >= 1 (left to right; out is not q).
 __device__ void pow_inc64(const Lane64& L, const double* q, int n, double* out) {
-  L.put(out, n > 0 ? q[L.e] : 0.0);
-  for (int b = 30 - __clz(max(n, 1)); b >= 0; --b) {
+  L.put(out, q[L.e]);
+  for (int b = 30 - __clz(n); b >= 0; --b) {
     mul_inc64(L, out, out, out);
     if ((n >> b) & 1) mul_inc64(L, out, q, out);
   }
@@ -1256,6 +1260,24 @@ __device__ __forceinline__ void apply_inc64(const double* q, double (&e)[6]) {
   e[5] = fma(q[25], e[5], e[5]);
 }
 
+// Row i of (I + q) v (the zero entries past 25 pad the activation rows).
+__device__ __forceinline__ double row_inc64(const double* q, const double* v, int i) {
+  const bool mech = i < 4;
+  double t = fma(q[mech ? 16 + 2 * i : i == 4 ? 24 : 26], v[4], v[i]);
+  t = fma(q[mech ? 17 + 2 * i : i == 5 ? 25 : 26], v[5], t);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) t = fma(q[mech ? 4 * i + k : 26], v[k], t);
+  return t;
+}
+
+// v <- (I + q) v for the warp's vector in shared memory.
+__device__ __forceinline__ void apply_vec64(const Lane64& L, const double* q, double* v) {
+  const double t = row_inc64(q, v, L.e < 6 ? L.e : 0);
+  __syncwarp();
+  if (L.e < 6) v[L.e] = t;
+  __syncwarp();
+}
+
 __device__ __forceinline__ double warp_sum64(double v) {
 #pragma unroll
   for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -1270,32 +1292,38 @@ struct Err64 {
   }
 };
 
-// n samples of one phase from the state e (the same on every lane), the first
-// of them sample k0, around the equilibrium angle th; leaves the state after
-// the last one in e.  W.P[0] holds the one-sample propagator.
-__device__ void run_phase64(const Lane64& L, Warp64& W, double (&e)[6], int k0, int n, double th, double sg,
-                            const float* y, Err64& err) {
+// n samples of one phase from the state W.v, the first of them sample k0,
+// around the equilibrium angle th; leaves the state after the last one in
+// W.v.  W.P[0] holds the one-sample propagator.
+__device__ void run_phase64(const Lane64& L, Warp64& W, int k0, int n, double th, double sg, const float* y, Err64& err) {
   if (n <= 0) return;
-  for (int b = 1; b < 6; ++b) mul_inc64(L, W.P[b - 1], W.P[b - 1], W.P[b]);
-  apply_inc64(W.P[0], e);
+  apply_vec64(L, W.P[0], W.v);
+  if (L.e < 6) W.E[0][L.e] = W.v[L.e];
+  __syncwarp();
 #pragma unroll 1
-  for (int b = 0; b < 5; ++b) {
-    double t[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) t[i] = e[i];
-    apply_inc64(W.P[b], t);
-    if ((L.e >> b) & 1)
-#pragma unroll
-      for (int i = 0; i < 6; ++i) e[i] = t[i];
+  for (int b = 0; b < 5 && (1 << b) < n; ++b) {
+    // states 1 .. c give c + 1 .. 2 c by P[b], whose square is P[b + 1]
+    for (int t = L.e; t < 6 << b; t += 32) {
+      const int st = t / 6, i = t - 6 * st;
+      W.E[st + (1 << b)][i] = row_inc64(W.P[b], W.E[st], i);
+    }
+    if ((2 << b) < n) mul_inc64(L, W.P[b], W.P[b], W.P[b + 1]);
+    __syncwarp();
   }
+  double e[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) e[i] = W.E[L.e][i];   // (lanes past n hold nothing that is used)
 #pragma unroll 1
   for (int i = L.e;; i += 32) {
     if (i < n) err.add(sg * (th + e[0]) - (double)y[k0 + i]);
     if (i - L.e + 32 >= n) break;   // warp-uniform
     apply_inc64(W.P[5], e);
   }
+  __syncwarp();
+  if (L.e == ((n - 1) & 31))
 #pragma unroll
-  for (int i = 0; i < 6; ++i) e[i] = __shfl_sync(0xffffffffu, e[i], (n - 1) & 31);
+    for (int i = 0; i < 6; ++i) W.v[i] = e[i];
+  __syncwarp();
 }
 
 // Mean squared and mean absolute error of the OPC vector W.opc's trajectory
@@ -1394,33 +1422,38 @@ __device__ void errors64(const Lane64& L, Warp64& W, const DevSac& d, const floa
       jsw = J - n1 * nsub;
       sw = true;
     }
-    double e[6];
+    if (L.e == 0)
 #pragma unroll
-    for (int i = 0; i < 6; ++i) e[i] = s0[i] - s1[i];
+      for (int i = 0; i < 6; ++i) W.v[i] = s0[i] - s1[i];
     step_inc64(L, W.A, h, W.W, W.Q);
     if (n1 > 0) {
       pow_inc64(L, W.Q, nsub, W.P[0]);
-      run_phase64(L, W, e, d.onset + 1, n1, s1[0], sg, y, err);
+      run_phase64(L, W, d.onset + 1, n1, s1[0], sg, y, err);
     }
     if (sw) {
       // the sample that holds the pulse end
-      pow_inc64(L, W.Q, jsw, W.B);
-      apply_inc64(W.B, e);
+      if (jsw > 0) {
+        pow_inc64(L, W.Q, jsw, W.B);
+        apply_vec64(L, W.B, W.v);
+      }
       step_inc64(L, W.A, frac * h, W.W, W.B);
-      apply_inc64(W.B, e);
+      apply_vec64(L, W.B, W.v);
+      if (L.e == 0)
 #pragma unroll
-      for (int i = 0; i < 6; ++i) e[i] += s1[i] - s2[i];
+        for (int i = 0; i < 6; ++i) W.v[i] += s1[i] - s2[i];
       L.put(W.A, L.e == 24 ? -r[iTdA] : L.e == 25 ? -r[iTaN] : W.A[L.e]);
       step_inc64(L, W.A, h - frac * h, W.W, W.B);
-      apply_inc64(W.B, e);
+      apply_vec64(L, W.B, W.v);
       step_inc64(L, W.A, h, W.W, W.Q);
-      pow_inc64(L, W.Q, nsub - 1 - jsw, W.B);
-      apply_inc64(W.B, e);
+      if (jsw + 1 < nsub) {
+        pow_inc64(L, W.Q, nsub - 1 - jsw, W.B);
+        apply_vec64(L, W.B, W.v);
+      }
       const int k = d.onset + 1 + n1;
-      if (L.e == 0) err.add(sg * (s2[0] + e[0]) - (double)y[k]);
+      if (L.e == 0) err.add(sg * (s2[0] + W.v[0]) - (double)y[k]);
       if (k + 1 < d.L) {
         pow_inc64(L, W.Q, nsub, W.P[0]);
-        run_phase64(L, W, e, k + 1, d.L - 1 - k, s2[0], sg, y, err);
+        run_phase64(L, W, k + 1, d.L - 1 - k, s2[0], sg, y, err);
       }
     }
   }
