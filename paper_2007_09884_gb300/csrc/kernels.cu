@@ -1532,9 +1532,7 @@ __global__ void __launch_bounds__(32) k_finalize(const DevSac* sacs, const float
 // max_i A_ii)) solved by Cholesky in FP64; u' = clamp(u + du); accept when
 // f(u') < f(u) (lambda / 10, floor 1e-12, new Jacobian), else lambda * 10
 // (ceiling 1e12).  f = sum_k r_k^2 / L over every sample.  Stops early when
-// A is zero or the system is not positive definite.  Trajectories (2N + 2
-// rows of lcap floats) go to shared memory when they fit, else to a per-block
-// scratch area in global memory.
+// A is zero or the system is not positive definite.
 constexpr int kRefineThreads = 64;
 
 // Floats between trajectory rows: an odd number, so that threads that write
@@ -1602,14 +1600,20 @@ __device__ double refine_f(RefineSmem<N>& S, const float* row, const float* z, i
   return refine_sum<N>(S, acc) / (double)L;
 }
 
-// rows_in_smem: the 2N + 2 trajectory rows live in dynamic shared memory after
-// the staged trace (short windows; the dot products of J^T J then read shared
-// memory), else in the per-block global scratch area.
-template <int N>
+// SMEM: the N + 2 rows that the dot products of J^T J read (the
+// Jacobian's columns, formed in place of the trajectories at u + delta, and
+// the current and the trial point's trajectory) live in dynamic shared memory
+// after the staged trace (short windows), else in the per-block global scratch
+// area, where the N trajectories at u - delta always go: they are written and
+// read once per Jacobian, and without them four blocks fit on an SM instead of
+// two (windows of 400 samples), which is what hides the FP64 factorisation of
+// one block (40 k of an iteration's 107 k cycles, on one warp) behind the
+// others.
+template <int N, bool SMEM>
 __global__ void __launch_bounds__(kRefineThreads) k_refine(const DevSac* sacs, const float* traces, const float* pcs,
                                                             const float* start, int K, float lnlo, float lnhi,
                                                             float delta, float lambda0, int lcap, float* scratch,
-                                                            int rows_in_smem, opmm_fit_result* out, unsigned* err) {
+                                                            opmm_fit_result* out, unsigned* err) {
   __shared__ RefineSmem<N> S;
   extern __shared__ __align__(128) unsigned char smraw[];
   float* yraw = reinterpret_cast<float*>(smraw);
@@ -1618,8 +1622,8 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(const DevSac* sacs, c
   const int b = blockIdx.x, tid = threadIdx.x;
   const DevSac d = sacs[b];
   const int pitch = refine_pitch(lcap);
-  float* rows = rows_in_smem ? qslot + kQSlotFloats * kRefineThreads
-                             : scratch + (size_t)b * (2 * N + 2) * (size_t)pitch;
+  float* minus = scratch + (size_t)b * (SMEM ? N : 2 * N + 2) * (size_t)pitch;
+  float* rows = SMEM ? qslot + kQSlotFloats * kRefineThreads : minus + (size_t)N * pitch;
   if (tid == 0) {
     mbar_init(&S.bar, 1);
     fence_mbar_init();
@@ -1651,7 +1655,7 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(const DevSac* sacs, c
   }
   __syncthreads();
   const SacConst sc = S.sc;
-  float* rcur[2] = {rows + (size_t)(2 * N) * pitch, rows + (size_t)(2 * N + 1) * pitch};
+  float* rcur[2] = {rows + (size_t)N * pitch, rows + (size_t)(N + 1) * pitch};
   if (tid == 0) {
     float p[kNumParams];
     u_to_p<N>(S.u, S.pc, lnlo, lnhi, p);
@@ -1679,7 +1683,7 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(const DevSac* sacs, c
         float p[kNumParams];
         u_to_p<N>(ut, S.pc, lnlo, lnhi, p);
         int pe = 0;
-        S.bad[tid] = refine_row(p, sc, rows + (size_t)tid * pitch, &pe, qslot + tid) ? 0 : 1;
+        S.bad[tid] = refine_row(p, sc, ((tid & 1) ? minus : rows) + (size_t)j * pitch, &pe, qslot + tid) ? 0 : 1;
         if (pe) atomicAdd(&S.pe, 1);
       }
       __syncthreads();
@@ -1690,8 +1694,8 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(const DevSac* sacs, c
       for (int k = tid; k < sc.L; k += kRefineThreads) {
 #pragma unroll 6
         for (int j = 0; j < N; ++j) {
-          float* jp = rows + (size_t)(2 * j) * pitch + k;
-          *jp = (*jp - jp[pitch]) * inv2d;
+          float* jp = rows + (size_t)j * pitch + k;
+          *jp = (*jp - minus[(size_t)j * pitch + k]) * inv2d;
         }
       }
       __syncthreads();
@@ -1718,11 +1722,11 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(const DevSac* sacs, c
         }
         ea[q] = a;
         eb[q] = bb;
-        ja[q] = rows + (size_t)(a < 0 ? 0 : 2 * a) * pitch;
-        jb[q] = bb < 0 ? r0 : rows + (size_t)(2 * bb) * pitch;
+        ja[q] = rows + (size_t)(a < 0 ? 0 : a) * pitch;
+        jb[q] = bb < 0 ? r0 : rows + (size_t)bb * pitch;
         sum[q] = c[q] = 0.0f;
       }
-#pragma unroll 2
+#pragma unroll 4
       for (int k = 0; k < sc.L; ++k) {
         const float zk = z[k];
 #pragma unroll
@@ -1776,7 +1780,7 @@ __global__ void __launch_bounds__(kRefineThreads) k_refine(const DevSac* sacs, c
             go = 0;
             break;
           }
-          const double ljj = sqrt(sjj), il = 1.0 / ljj;
+          const double ljj = sqrt(sjj), il = __drcp_rn(ljj);
           __syncwarp();
           if (tid == 0) {
             M[j * N + j] = ljj;
@@ -1909,26 +1913,22 @@ cudaError_t launch_refine(int dim, const DevSac* sacs, const float* traces, cons
                           int n, int K, float lnlo, float lnhi, float delta, float lambda0, int lcap, float* scratch,
                           opmm_fit_result* out, unsigned* err, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  // the trajectory rows go to shared memory when they fit in 96 KB (windows up
-  // to about 600 samples with 18 coordinates), leaving room for two blocks
-  const size_t rows_bytes = (2 * (size_t)dim + 2) * (size_t)refine_pitch(lcap) * sizeof(float);
-  const int in_smem = rows_bytes <= (size_t)96 * 1024 ? 1 : 0;
+  // the rows of the dot products go to shared memory when they fit in 96 KB
+  // (windows up to about 1,200 samples with 18 coordinates)
+  const size_t rows_bytes = ((size_t)dim + 2) * (size_t)refine_pitch(lcap) * sizeof(float);
+  const bool in_smem = rows_bytes <= (size_t)96 * 1024;
   const size_t smem = 2 * (size_t)lcap * sizeof(float) + (size_t)kQSlotFloats * kRefineThreads * sizeof(float) +
                       (in_smem ? rows_bytes : 0);
-  if (dim == 9) {
-    cudaError_t e = allow_dynamic_smem(k_refine<9>, smem);
+  auto run = [&](auto kernel) -> cudaError_t {
+    const cudaError_t e = allow_dynamic_smem(kernel, smem);
     if (e != cudaSuccess) return e;
-    k_refine<9><<<n, kRefineThreads, smem, st>>>(sacs, traces, pcs, start, K, lnlo, lnhi, delta, lambda0, lcap,
-                                                 scratch, in_smem, out, err);
-  } else if (dim == kNumParams) {
-    cudaError_t e = allow_dynamic_smem(k_refine<kNumParams>, smem);
-    if (e != cudaSuccess) return e;
-    k_refine<kNumParams><<<n, kRefineThreads, smem, st>>>(sacs, traces, pcs, start, K, lnlo, lnhi, delta, lambda0,
-                                                          lcap, scratch, in_smem, out, err);
-  } else {
-    return cudaErrorInvalidValue;
-  }
-  cudaError_t e = cudaGetLastError();
+    kernel<<<n, kRefineThreads, smem, st>>>(sacs, traces, pcs, start, K, lnlo, lnhi, delta, lambda0, lcap, scratch, out,
+                                            err);
+    return cudaGetLastError();
+  };
+  cudaError_t e = cudaErrorInvalidValue;
+  if (dim == 9) e = in_smem ? run(k_refine<9, true>) : run(k_refine<9, false>);
+  else if (dim == kNumParams) e = in_smem ? run(k_refine<kNumParams, true>) : run(k_refine<kNumParams, false>);
   if (e != cudaSuccess) return e;
   k_refine_check<<<n, 32, 0, st>>>(sacs, traces, n, out);
   return cudaGetLastError();
