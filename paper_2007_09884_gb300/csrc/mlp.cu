@@ -19,7 +19,7 @@
 //
 // Around it: the training head (output layer, loss, the layer-3 error, the
 // output layer's gradient partials), the gradient assembly fused with AdamW,
-// the inference head, the on-device training data generator and the
+// the inference head (output layer and box centres), the on-device training data generator and the
 // featurizer.
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -449,38 +449,65 @@ __global__ void __launch_bounds__(gemm_threads(STAGES), STAGES <= 3 ? 2 : 1)
 }
 
 // ------------------------------------------------------------------ elementwise / reductions
-// Output layer and loss: Y[m][o] = H[m] . W5[o] + b5[o] (o < 18, CUDA cores);
-// loss contribution and dY = 2 (Y - T) / (M * 18).  One warp per row.
-__global__ void k_head_fwd_loss(const __nv_bfloat16* H, const __nv_bfloat16* W5, const float* b5, const float* T, int M,
-                                float* Y, float* dY, float* row_loss) {
+// Inference head: the output layer y[o] = H[m] . W5[o] + b5[o] (o < 18) of
+// rows m < n on CUDA cores, straight into the box centres, centre[o] *=
+// exp(scale y[o]).  One warp per kHeadWarpRows rows, whose H it takes through
+// one pass over W5 (staged in shared memory as FP32); a row's lane partials
+// are summed by a reduce-scatter (31 shuffles, output o on lane o), the same
+// pairwise sums as 18 butterflies of five.  Bound by latency: a few hundred
+// instructions a warp.
+constexpr int kHeadWarps = 8, kHeadWarpRows = 4;
+constexpr size_t kHeadCentresSmem = (size_t)kOut * kHidden * 4;
+
+__global__ void __launch_bounds__(32 * kHeadWarps) k_head_centres(const __nv_bfloat16* H, const __nv_bfloat16* W5,
+                                                                  const float* b5, int n, float scale, float* pc) {
+  extern __shared__ __align__(16) unsigned char hsm[];
+  float* sw = reinterpret_cast<float*>(hsm);   // [18][512]
+  for (int i = threadIdx.x; i < kOut * kHidden / 2; i += 32 * kHeadWarps)
+    reinterpret_cast<float2*>(sw)[i] = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(W5)[i]);
+  __syncthreads();
   const int lane = threadIdx.x & 31;
-  const int m = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  if (m >= M) return;
-  float acc[kOut];
+  const int m0 = (int)(blockIdx.x * kHeadWarps + (threadIdx.x >> 5)) * kHeadWarpRows;
+  if (m0 >= n) return;   // the rows past n of the last group exist (H is padded to the GEMM's tile)
+  float acc[kHeadWarpRows][kOut];
 #pragma unroll
-  for (int o = 0; o < kOut; ++o) acc[o] = 0.0f;
+  for (int r = 0; r < kHeadWarpRows; ++r)
+#pragma unroll
+    for (int o = 0; o < kOut; ++o) acc[r][o] = 0.0f;
+#pragma unroll 4
   for (int k = lane; k < kHidden; k += 32) {
-    const float h = __bfloat162float(H[(size_t)m * kHidden + k]);
+    float h[kHeadWarpRows];
 #pragma unroll
-    for (int o = 0; o < kOut; ++o) acc[o] = fmaf(h, __bfloat162float(W5[(size_t)o * kHidden + k]), acc[o]);
-  }
-  float l = 0.0f;
+    for (int r = 0; r < kHeadWarpRows; ++r) h[r] = __bfloat162float(H[(size_t)(m0 + r) * kHidden + k]);
 #pragma unroll
-  for (int o = 0; o < kOut; ++o) {
-    float v = acc[o];
+    for (int o = 0; o < kOut; ++o) {
+      const float w = sw[o * kHidden + k];
 #pragma unroll
-    for (int s = 16; s; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
-    v += b5[o];
-    if (lane == 0) {
-      Y[(size_t)m * kOut + o] = v;
-      if (T) {
-        const float d = v - T[(size_t)m * kOut + o];
-        l += d * d;
-        dY[(size_t)m * kOut + o] = 2.0f * d / (float)(M * kOut);
-      }
+      for (int r = 0; r < kHeadWarpRows; ++r) acc[r][o] = fmaf(h[r], w, acc[r][o]);
     }
   }
-  if (lane == 0 && row_loss) row_loss[m] = l / (float)(M * kOut);
+  const float b = lane < kOut ? b5[lane] : 0.0f;
+#pragma unroll
+  for (int r = 0; r < kHeadWarpRows; ++r) {
+    float v[32];
+#pragma unroll
+    for (int o = 0; o < 32; ++o) v[o] = o < kOut ? acc[r][o < kOut ? o : 0] : 0.0f;
+#pragma unroll
+    for (int lev = 0; lev < 5; ++lev) {
+      const int off = 16 >> lev;
+      const bool up = (lane & off) != 0;
+#pragma unroll
+      for (int q = 0; q < off; ++q) {
+        const float send = up ? v[q] : v[q + off];
+        const float keep = up ? v[q + off] : v[q];
+        v[q] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+      }
+    }
+    if (lane < kOut && m0 + r < n) {
+      float* c = pc + (size_t)(m0 + r) * kOut + lane;
+      *c *= __expf(scale * (v[0] + b));
+    }
+  }
 }
 
 // Output layer, loss and the first steps of the backward pass for 32 rows
@@ -875,13 +902,6 @@ __global__ void k_bump(long long* p64, long long by64, int* p32) {
   }
 }
 
-// Box centres from the network's output: centre = nominal * exp(scale * y).
-__global__ void k_apply_centres(const float* Y, int n, float scale, float* pc) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n * kOut) return;
-  pc[i] *= __expf(scale * Y[i]);
-}
-
 // Training data: per sample g = base + i, Philox4x32-10 (key = seed,
 // counter = (g, word, 0, 0)) draws the rate (250/500/1000 Hz), the window
 // (40-400 samples, redrawn until a 1 deg saccade fits), the amplitude
@@ -1096,9 +1116,11 @@ cudaError_t gemm(const GemmLaunch& L, cudaStream_t st) {
   return launch_chain(k_gemm_tn<4, kEpiF32, 256, true, true>, grid, gemm_threads(4), gemm_smem(4, 256), st, L.chained, maps, g);
 }
 
-cudaError_t head_fwd_loss(const __nv_bfloat16* H, const __nv_bfloat16* W5, const float* b5, const float* T, int M,
-                          float* Y, float* dY, float* row_loss, cudaStream_t st) {
-  k_head_fwd_loss<<<(M * 32 + 255) / 256, 256, 0, st>>>(H, W5, b5, T, M, Y, dY, row_loss);
+cudaError_t head_centres(const __nv_bfloat16* H, const __nv_bfloat16* W5, const float* b5, int n, float* pc,
+                         cudaStream_t st) {
+  constexpr int rows = kHeadWarps * kHeadWarpRows;
+  static_assert(kBM % rows == 0, "the padded rows cover the last group");
+  k_head_centres<<<(n + rows - 1) / rows, 32 * kHeadWarps, kHeadCentresSmem, st>>>(H, W5, b5, n, kTargetScale, pc);
   return cudaGetLastError();
 }
 
@@ -1145,11 +1167,6 @@ cudaError_t featurize(const DevSac* sacs, const float* traces, int n, __nv_bfloa
 
 cudaError_t bump(long long* p64, long long by64, int* p32, cudaStream_t st) {
   k_bump<<<1, 32, 0, st>>>(p64, by64, p32);
-  return cudaGetLastError();
-}
-
-cudaError_t apply_centres(const float* Y, int n, float* pc, cudaStream_t st) {
-  k_apply_centres<<<(n * kOut + 255) / 256, 256, 0, st>>>(Y, n, kTargetScale, pc);
   return cudaGetLastError();
 }
 

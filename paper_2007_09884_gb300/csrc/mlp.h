@@ -138,8 +138,10 @@ struct FinishArgs {
 
 cudaError_t gemm_prepare();
 cudaError_t gemm(const GemmLaunch& L, cudaStream_t st);
-cudaError_t head_fwd_loss(const __nv_bfloat16* H, const __nv_bfloat16* W5, const float* b5, const float* T, int M,
-                          float* Y, float* dY, float* row_loss, cudaStream_t st);
+// Inference head of rows m < n: pc[m][o] *= exp(kTargetScale y[m][o]).  H holds
+// whole tiles of kBM rows.
+cudaError_t head_centres(const __nv_bfloat16* H, const __nv_bfloat16* W5, const float* b5, int n, float* pc,
+                         cudaStream_t st);
 // Training head: output layer, loss terms, dY, the layer-3 error dZ3 (and
 // its per-32-row column sums), output-layer gradient partials per 32-row
 // block.  M a multiple of 32.  step_idx (optional): advanced by one.
@@ -152,7 +154,6 @@ cudaError_t adamw(float* w, const float* g, float* m1, float* m2, int n, float l
                   float wd, int step, const AdamLayout& L, __nv_bfloat16* wb, cudaStream_t st);
 cudaError_t pack_params(const float* w, int n, const AdamLayout& L, __nv_bfloat16* wb, cudaStream_t st);
 cudaError_t featurize(const DevSac* sacs, const float* traces, int n, __nv_bfloat16* X, cudaStream_t st);
-cudaError_t apply_centres(const float* Y, int n, float* pc, cudaStream_t st);
 cudaError_t bump(long long* p64, long long by64, int* p32, cudaStream_t st);
 cudaError_t gen_desc(uint64_t seed, const long long* base, int n, const float* cal_amp, const float* cal_pulse, int ncal,
                      DevSac* sacs, float* hidden, float* target, int lcap, cudaStream_t st);

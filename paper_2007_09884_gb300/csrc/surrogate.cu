@@ -31,7 +31,7 @@ constexpr int kTrainLcap = 400;         // longest training window
 constexpr int kWgradSplit = 4;          // largest number of K slices of the weight-gradient GEMM
 struct MlpBuffers {
   int M = 0;        // rows of a training pass
-  int rows = 0;     // rows of an inference pass (X, two layers' activations, Y)
+  int rows = 0;     // rows of an inference pass (X, two layers' activations)
   DevBuf X, H[kLayers], Z[kLayers], Y, dY, rowloss, dZ[kLayers], colpart[kLayers], wpart, dWpart, dbpart;
   Status ensure(int m) {
     if (m <= M) return Status();
@@ -59,7 +59,6 @@ struct MlpBuffers {
     const size_t act = (size_t)m * kHidden;
     Status s = X.ensure(act * 2);
     for (int l = 0; l < 2 && s.ok(); ++l) s = H[l].ensure(act * 2);
-    if (s.ok()) s = Y.ensure((size_t)m * kOut * 4);
     if (s.ok()) rows = m;
     return s;
   }
@@ -165,13 +164,14 @@ static Status forward_hidden(opmm_ctx* ctx, MlpBuffers& B, int M, const __nv_bfl
   return Status();
 }
 
-// Inference: hidden layers, then the output layer on CUDA cores into B.Y.
-static Status forward(opmm_ctx* ctx, MlpBuffers& B, int M, cudaStream_t st) {
+// Inference of n rows of B.X (padded to M): hidden layers, then the output
+// layer into the n box centres at pc.
+static Status forward_centres(opmm_ctx* ctx, MlpBuffers& B, int n, int M, float* pc, cudaStream_t st) {
   SurrogateState& S = *ctx->surrogate;
   Status s = forward_hidden(ctx, B, M, bf(B.X), false, st);
   if (!s.ok()) return s;
-  return cuda_status(head_fwd_loss(bf(B.H[(kLayers - 1) & 1]), bf(S.wb, (size_t)kLayers * kHidden * kHidden),
-                                   f32(S.w, kHeadB), nullptr, M, f32(B.Y), nullptr, nullptr, st),
+  return cuda_status(head_centres(bf(B.H[(kLayers - 1) & 1]), bf(S.wb, (size_t)kLayers * kHidden * kHidden),
+                                  f32(S.w, kHeadB), n, pc, st),
                      "head");
 }
 
@@ -289,8 +289,7 @@ Status surrogate_centres(opmm_ctx* ctx, const DevSac* sacs, const float* traces,
     if (!s.ok()) return s;
   }
   Status s = cuda_status(featurize(sacs, traces, n, bf(B.X), st), "featurize");
-  if (s.ok()) s = forward(ctx, B, M, st);
-  if (s.ok()) s = cuda_status(apply_centres(f32(B.Y), n, pc, st), "centres");
+  if (s.ok()) s = forward_centres(ctx, B, n, M, pc, st);
   return s;
 }
 
@@ -332,13 +331,12 @@ Status surrogate_prepare_plan(opmm_ctx* ctx, opmm_plan* p, int32_t n, bool once)
     s = cuda_status(cudaMemsetAsync(bf(keep->X, (size_t)n * kIn), 0, (size_t)(M - n) * kIn * 2, ctx->stream),
                     "clear features");
   if (!s.ok()) return s;
-  p->pre_search_kernels = 1 + kLayers + 2;
+  p->pre_search_kernels = 1 + kLayers + 1;
   p->pre_search = [keep, M](opmm_plan* pl, cudaStream_t st) -> Status {
     opmm_ctx* c = pl->ctx;
     Status r = cuda_status(featurize(pl->d_sacs.as<DevSac>(), pl->d_traces.as<float>(), pl->n, bf(keep->X), st),
                            "featurize");
-    if (r.ok()) r = forward(c, *keep, M, st);
-    if (r.ok()) r = cuda_status(apply_centres(f32(keep->Y), pl->n, pl->d_pc.as<float>(), st), "centres");
+    if (r.ok()) r = forward_centres(c, *keep, pl->n, M, pl->d_pc.as<float>(), st);
     return r;
   };
   return Status();
