@@ -276,7 +276,7 @@ __global__ void k_nominal(const DevSac* sacs, int n, int pulse_mode, const float
 }
 
 // ------------------------------------------------------------------ simulate
-__global__ void k_simulate(const float* opc, int n, const DevSac* sacs, const int* sac_of,
+__global__ void __launch_bounds__(256) k_simulate(const float* opc, int n, const DevSac* sacs, const int* sac_of,
                            const long long* out_off, float* out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -1992,9 +1992,9 @@ cudaError_t launch_nominal(const DevSac* sacs, int n, int pulse_mode, const floa
 }
 
 cudaError_t launch_simulate(const float* opc, int n, const DevSac* sacs, const int* sac_of,
-                            const long long* out_off, float* out, cudaStream_t st) {
+                            const long long* out_off, float* out, cudaStream_t st, int threads) {
   if (n <= 0) return cudaSuccess;
-  k_simulate<<<(n + 127) / 128, 128, 0, st>>>(opc, n, sacs, sac_of, out_off, out);
+  k_simulate<<<(n + threads - 1) / threads, threads, 0, st>>>(opc, n, sacs, sac_of, out_off, out);
   return cudaGetLastError();
 }
 

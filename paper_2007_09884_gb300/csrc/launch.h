@@ -46,7 +46,7 @@ cudaError_t launch_gather(const float* const* src, const DevSac* sacs, float* ds
 cudaError_t launch_nominal(const DevSac* sacs, int n, int pulse_mode, const float* init_opc, float* pc,
                            cudaStream_t st);
 cudaError_t launch_simulate(const float* opc, int n, const DevSac* sacs, const int* sac_of,
-                            const long long* out_off, float* out, cudaStream_t st);
+                            const long long* out_off, float* out, cudaStream_t st, int threads = 128);
 cudaError_t launch_score(const float* opc, int m, const DevSac& sac, const float* trace, float* f, int num_sms,
                          cudaStream_t st);   // trace: the saccade's samples, any alignment
 // Search kernel variants (see kernels.cu): unit size (simplices per block),

@@ -775,8 +775,9 @@ __global__ void __launch_bounds__(256) k_grad_finish(const __grid_constant__ Fin
       v[3] += x.w;
     }
     const long long i = (long long)l * kLayerParams + r;
-    *reinterpret_cast<float4*>(a.g + i) = make_float4(v[0], v[1], v[2], v[3]);
-    if (a.adam) {
+    if (!a.adam) {   // a training step takes the gradient from registers
+      *reinterpret_cast<float4*>(a.g + i) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
       const float4 m1 = *reinterpret_cast<const float4*>(a.m1 + i);
       const float4 m2 = *reinterpret_cast<const float4*>(a.m2 + i);
       const float4 w = *reinterpret_cast<const float4*>(a.w + i);

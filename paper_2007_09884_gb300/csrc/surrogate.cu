@@ -25,6 +25,12 @@ namespace {
 constexpr int kCal = 512;               // calibration table points
 constexpr float kCalLo = 0.5f, kCalHi = 45.0f;
 constexpr int kTrainLcap = 400;         // longest training window
+// Threads per block of the training data's trajectories: 256, so that a batch
+// of 4,096 takes 16 SMs.  The kernel's registers leave no room for a GEMM
+// block beside it, and the network's GEMMs need 128 of the 152 SMs at once: in
+// blocks of 128 threads on 32 SMs it sent eight of their blocks into a second
+// wave for as long as it ran.
+constexpr int kSimThreads = 256;
 }  // namespace
 
 // Activations and gradients of one batch of M rows (M a multiple of 128).
@@ -534,7 +540,7 @@ extern "C" int opmm_surrogate_train(opmm_ctx* ctx, int32_t steps, int32_t batch,
                                     D.sacs.as<DevSac>(), f32(D.hidden), f32(D.target), kTrainLcap, s2), "generate");
     if (r.ok())
       r = cuda_status(launch_simulate(f32(D.hidden), batch, D.sacs.as<DevSac>(), nullptr, S.outoff.as<long long>(),
-                                      f32(D.traces), s2), "simulate");
+                                      f32(D.traces), s2, kSimThreads), "simulate");
     if (r.ok()) r = cuda_status(add_noise(data_seed, gbase + b, D.sacs.as<DevSac>(), batch, f32(D.traces), 0.05f, s2), "noise");
     if (r.ok())
       r = cuda_status(featurize(D.sacs.as<DevSac>(), f32(D.traces), batch, bf(D.X), s2), "featurize");
