@@ -838,59 +838,81 @@ __global__ void __launch_bounds__(256) k_grad_finish(const __grid_constant__ Fin
 }
 
 // ------------------------------------------------------------------ data
+__device__ __forceinline__ float u01(uint32_t x) { return (float)(x >> 8) * (1.0f / 16777216.0f); }
+
 // Featurizer: resample the trace on a 1 ms grid from onset (256 points, linear
 // interpolation, held after the window end) in the positive frame, position
 // normalised by the amplitude (start fixation = 0, end fixation = 1) and
 // velocity as 10 x the per-millisecond difference.  Output BF16 [n][512].
-// A block of 4 warps takes 32 saccades (a warp per saccade at a time) and
-// stages their features in shared memory, then writes whole rows of X.
-constexpr int kFeatRows = 32;
-constexpr int kSxPitch = kIn + 2;          // BF16 elements: rows one bank apart
+// One warp per saccade, lane l the point pairs 2 l + 64 j, stored as they are
+// formed: nothing is staged, so a block needs no shared memory and runs
+// beside a network block that takes nearly all of an SM's (training data are
+// made while the network trains), and 4,096 saccades are 1,024 blocks at once
+// instead of 128 that take eight saccades per warp in turn.  Bound by the
+// chain descriptor -> samples -> store: 4,096 training
+// saccades with their noise 6.2 us, where noise (8 us) and features (12 us)
+// took two kernels; 96 training steps 11.6 -> 10.7 ms, since the network's
+// blocks no longer wait for an SM whose shared memory features hold.
+constexpr int kFeatWarps = 4;
+static_assert(kFeatPoints % 64 == 0 && kIn == 2 * kFeatPoints, "whole pairs per lane");
 
-__global__ void __launch_bounds__(128) k_featurize(const DevSac* sacs, const float* traces, int n, __nv_bfloat16* X) {
-  __shared__ __align__(16) __nv_bfloat16 sx[kFeatRows * kSxPitch];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int b0 = blockIdx.x * kFeatRows;
-  for (int rb = warp; rb < kFeatRows; rb += 4) {
-    const int b = b0 + rb;
-    if (b >= n) break;
-    const DevSac d = sacs[b];
-    const float* y = traces + d.off;
-    const float amp = fmaxf(d.thf - d.th0, 0.5f);
-    const float inv = 1.0f / amp;
-    float pos[kFeatPoints / 32 + 1];
-#pragma unroll
-    for (int j = 0; j <= kFeatPoints / 32; ++j) {
-      const int i = lane + 32 * j;
-      float v = 0.0f;
-      if (i <= kFeatPoints) {
-        float s = (float)d.onset + (float)i * d.fs * 1e-3f;
-        s = fminf(s, (float)(d.L - 1));
-        const int k0 = (int)floorf(s);
-        const int k1 = min(k0 + 1, d.L - 1);
-        const float w = s - (float)k0;
-        const float yy = (1.0f - w) * y[k0] + w * y[k1];
-        v = (d.sign * yy - d.th0) * inv;
-      }
-      pos[j] = v;
+// NOISE: training data.  The warp first takes its trajectory to shared memory
+// with N(0, sigma^2) deg of noise added (Philox stream 3 of sample *base + b,
+// a Box-Muller pair per two samples), as far as the features reach; a noise
+// kernel of its own wrote and read every trajectory once more.
+template <bool NOISE>
+__global__ void __launch_bounds__(32 * kFeatWarps) k_featurize(const DevSac* sacs, const float* traces, int n,
+                                                               __nv_bfloat16* X, uint64_t seed,
+                                                               const long long* base_ptr, float sigma) {
+  __shared__ float noisy[NOISE ? kFeatWarps : 1][NOISE ? kTrainLcap : 1];
+  const int lane = threadIdx.x & 31;
+  const int b = blockIdx.x * kFeatWarps + (threadIdx.x >> 5);
+  if (b >= n) return;
+  const DevSac d = sacs[b];
+  const float* y = traces + d.off;
+  if constexpr (NOISE) {   // d.L <= kTrainLcap (k_gen_desc)
+    float* z = noisy[threadIdx.x >> 5];
+    const long long g = *base_ptr + b;
+    const int end = min(d.L, (int)((float)d.onset + (float)kFeatPoints * d.fs * 1e-3f) + 2);
+    for (int k2 = 2 * lane; k2 < end; k2 += 64) {
+      const float y0 = y[k2], y1 = k2 + 1 < d.L ? y[k2 + 1] : 0.0f;
+      uint32_t q[4];
+      philox4x32_10((uint32_t)g, (uint32_t)(g >> 32), 3u, (uint32_t)k2, (uint32_t)seed, (uint32_t)(seed >> 32), q);
+      const float u1 = fmaxf(u01(q[0]), 1e-7f), u2 = u01(q[1]);
+      const float rad = sqrtf(-2.0f * __logf(u1));
+      z[k2] = y0 + sigma * rad * __cosf(6.283185307f * u2);
+      if (k2 + 1 < d.L) z[k2 + 1] = y1 + sigma * rad * __sinf(6.283185307f * u2);
     }
-#pragma unroll
-    for (int j = 0; j < kFeatPoints / 32; ++j) {
-      const int i = lane + 32 * j;
-      const float nxt = __shfl_down_sync(0xffffffffu, pos[j], 1);
-      const float nxt2 = __shfl_sync(0xffffffffu, pos[j + 1], 0);
-      const float p1 = lane == 31 ? nxt2 : nxt;
-      const float vel = (i == kFeatPoints - 1) ? 0.0f : 10.0f * (p1 - pos[j]);
-      sx[rb * kSxPitch + i] = __float2bfloat16_rn(pos[j]);
-      sx[rb * kSxPitch + kFeatPoints + i] = __float2bfloat16_rn(vel);
-    }
+    __syncwarp();
+    y = z;
   }
-  __syncthreads();
-  const int nr = min(kFeatRows, n - b0);
-  for (int q = tid; q < nr * (kIn / 2); q += 128) {
-    const int i = q / (kIn / 2), c2 = q - i * (kIn / 2);
-    *reinterpret_cast<__nv_bfloat162*>(X + (size_t)(b0 + i) * kIn + 2 * c2) =
-        *reinterpret_cast<const __nv_bfloat162*>(sx + i * kSxPitch + 2 * c2);
+  const float amp = fmaxf(d.thf - d.th0, 0.5f);
+  const float inv = 1.0f / amp;
+  auto point = [&](int i) {
+    float s = (float)d.onset + (float)i * d.fs * 1e-3f;
+    s = fminf(s, (float)(d.L - 1));
+    const int k0 = (int)floorf(s);
+    const int k1 = min(k0 + 1, d.L - 1);
+    const float w = s - (float)k0;
+    const float yy = (1.0f - w) * y[k0] + w * y[k1];
+    return (d.sign * yy - d.th0) * inv;
+  };
+  constexpr int kPairs = kFeatPoints / 64;
+  float p0[kPairs], p1[kPairs];
+#pragma unroll
+  for (int j = 0; j < kPairs; ++j) {
+    p0[j] = point(2 * lane + 64 * j);
+    p1[j] = point(2 * lane + 64 * j + 1);
+  }
+  __nv_bfloat162* x = reinterpret_cast<__nv_bfloat162*>(X + (size_t)b * kIn) + lane;
+#pragma unroll
+  for (int j = 0; j < kPairs; ++j) {
+    const float same = __shfl_down_sync(0xffffffffu, p0[j], 1);
+    const float wrap = __shfl_sync(0xffffffffu, p0[j + 1 < kPairs ? j + 1 : j], 0);
+    const float nxt = lane == 31 ? wrap : same;                         // point 2 l + 64 j + 2
+    const bool last = j + 1 == kPairs && lane == 31;                    // the last point's velocity is 0
+    x[32 * j] = __floats2bfloat162_rn(p0[j], p1[j]);
+    x[kFeatPoints / 2 + 32 * j] = __floats2bfloat162_rn(10.0f * (p1[j] - p0[j]), last ? 0.0f : 10.0f * (nxt - p1[j]));
   }
 }
 
@@ -909,8 +931,6 @@ __global__ void k_bump(long long* p64, long long by64, int* p32) {
 // (log-uniform up to 40 deg, capped by the window), the direction, the 18
 // hidden multipliers U(0.8, 1.2) and N(0, 0.05^2) noise (Box-Muller).  The
 // hidden OPC is the interpolated nominal centre times the multipliers.
-__device__ __forceinline__ float u01(uint32_t x) { return (float)(x >> 8) * (1.0f / 16777216.0f); }
-
 __global__ void k_gen_desc(uint64_t seed, const long long* base_ptr, int n, const float* cal_amp, const float* cal_pulse,
                            int ncal, DevSac* sacs, float* hidden, float* target, int lcap) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -969,23 +989,6 @@ __global__ void k_gen_desc(uint64_t seed, const long long* base_ptr, int n, cons
         target[(size_t)i * kOut + j] = __logf(mult) * (1.0f / kTargetScale);
       }
     }
-  }
-}
-
-// Noisy trace: simulated trajectory plus N(0, 0.05^2) deg noise, in place.
-__global__ void k_add_noise(uint64_t seed, const long long* base_ptr, const DevSac* sacs, int n, float* traces,
-                            float sigma) {
-  const int b = blockIdx.x;
-  if (b >= n) return;
-  const DevSac d = sacs[b];
-  const long long g = *base_ptr + b;
-  for (int k2 = threadIdx.x * 2; k2 < d.L; k2 += 2 * blockDim.x) {
-    uint32_t q[4];
-    philox4x32_10((uint32_t)g, (uint32_t)(g >> 32), 3u, (uint32_t)k2, (uint32_t)seed, (uint32_t)(seed >> 32), q);
-    const float u1 = fmaxf(u01(q[0]), 1e-7f), u2 = u01(q[1]);
-    const float rad = sqrtf(-2.0f * __logf(u1));
-    traces[d.off + k2] += sigma * rad * __cosf(6.283185307f * u2);
-    if (k2 + 1 < d.L) traces[d.off + k2 + 1] += sigma * rad * __sinf(6.283185307f * u2);
   }
 }
 
@@ -1162,7 +1165,13 @@ cudaError_t pack_params(const float* w, int n, const AdamLayout& L, __nv_bfloat1
 }
 
 cudaError_t featurize(const DevSac* sacs, const float* traces, int n, __nv_bfloat16* X, cudaStream_t st) {
-  k_featurize<<<(n + kFeatRows - 1) / kFeatRows, 128, 0, st>>>(sacs, traces, n, X);
+  k_featurize<false><<<(n + kFeatWarps - 1) / kFeatWarps, 32 * kFeatWarps, 0, st>>>(sacs, traces, n, X, 0, nullptr, 0.0f);
+  return cudaGetLastError();
+}
+
+cudaError_t featurize_noisy(uint64_t seed, const long long* base, const DevSac* sacs, const float* traces, int n,
+                            float sigma, __nv_bfloat16* X, cudaStream_t st) {
+  k_featurize<true><<<(n + kFeatWarps - 1) / kFeatWarps, 32 * kFeatWarps, 0, st>>>(sacs, traces, n, X, seed, base, sigma);
   return cudaGetLastError();
 }
 
@@ -1174,12 +1183,6 @@ cudaError_t bump(long long* p64, long long by64, int* p32, cudaStream_t st) {
 cudaError_t gen_desc(uint64_t seed, const long long* base, int n, const float* cal_amp, const float* cal_pulse, int ncal,
                      DevSac* sacs, float* hidden, float* target, int lcap, cudaStream_t st) {
   k_gen_desc<<<(n + 127) / 128, 128, 0, st>>>(seed, base, n, cal_amp, cal_pulse, ncal, sacs, hidden, target, lcap);
-  return cudaGetLastError();
-}
-
-cudaError_t add_noise(uint64_t seed, const long long* base, const DevSac* sacs, int n, float* traces, float sigma,
-                      cudaStream_t st) {
-  k_add_noise<<<n, 128, 0, st>>>(seed, base, sacs, n, traces, sigma);
   return cudaGetLastError();
 }
 

@@ -33,6 +33,7 @@ constexpr int gemm_threads(int stages) { return gemm_epi_warps(stages) * 32 + 64
 // ring, then 256 bytes of barriers and the tile's bias (512 bytes), plus the
 // 1024-byte alignment of the ring
 constexpr size_t gemm_smem(int stages, int bn) { return (size_t)stages * stage_bytes(bn) + 1024 + 256 + 512; }
+constexpr int kTrainLcap = 400;           // longest training window
 constexpr int kMaxGroup = 4;              // GEMM problems of one launch
 
 // Epilogues: kEpiBiasGelu  z = acc + bias -> out_f32 (z, optional), out_bf16
@@ -157,8 +158,8 @@ cudaError_t featurize(const DevSac* sacs, const float* traces, int n, __nv_bfloa
 cudaError_t bump(long long* p64, long long by64, int* p32, cudaStream_t st);
 cudaError_t gen_desc(uint64_t seed, const long long* base, int n, const float* cal_amp, const float* cal_pulse, int ncal,
                      DevSac* sacs, float* hidden, float* target, int lcap, cudaStream_t st);
-cudaError_t add_noise(uint64_t seed, const long long* base, const DevSac* sacs, int n, float* traces, float sigma,
-                      cudaStream_t st);
+cudaError_t featurize_noisy(uint64_t seed, const long long* base, const DevSac* sacs, const float* traces, int n,
+                            float sigma, __nv_bfloat16* X, cudaStream_t st);
 
 }  // namespace mlp
 }  // namespace opmm

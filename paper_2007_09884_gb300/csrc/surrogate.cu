@@ -24,7 +24,6 @@ using namespace mlp;
 namespace {
 constexpr int kCal = 512;               // calibration table points
 constexpr float kCalLo = 0.5f, kCalHi = 45.0f;
-constexpr int kTrainLcap = 400;         // longest training window
 // Threads per block of the training data's trajectories: 256, so that a batch
 // of 4,096 takes 16 SMs.  The kernel's registers leave no room for a GEMM
 // block beside it, and the network's GEMMs need 128 of the 152 SMs at once: in
@@ -541,9 +540,9 @@ extern "C" int opmm_surrogate_train(opmm_ctx* ctx, int32_t steps, int32_t batch,
     if (r.ok())
       r = cuda_status(launch_simulate(f32(D.hidden), batch, D.sacs.as<DevSac>(), nullptr, S.outoff.as<long long>(),
                                       f32(D.traces), s2, kSimThreads), "simulate");
-    if (r.ok()) r = cuda_status(add_noise(data_seed, gbase + b, D.sacs.as<DevSac>(), batch, f32(D.traces), 0.05f, s2), "noise");
     if (r.ok())
-      r = cuda_status(featurize(D.sacs.as<DevSac>(), f32(D.traces), batch, bf(D.X), s2), "featurize");
+      r = cuda_status(featurize_noisy(data_seed, gbase + b, D.sacs.as<DevSac>(), f32(D.traces), batch, 0.05f, bf(D.X), s2),
+                      "featurize");
     if (r.ok()) r = cuda_status(bump(gbase + b, 2LL * batch, nullptr, s2), "advance sample base");
     return r;
   };
