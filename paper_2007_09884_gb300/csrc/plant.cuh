@@ -135,7 +135,10 @@ __device__ __forceinline__ void rest_state_k(const float* p, const Coef& k, floa
   s[5] = fmaf(tn, fmaf(p[kLtAnt], k.iKn, 1.0f), -p[kLtAnt] * th);
 }
 
-// Equilibrium under constant active-state tensions, precomputed 1/K_SE.
+// Equilibrium under constant active-state tensions (fa, fn): from x' = y' = 0
+// the series tensions are Ta = a_g (fa - K_LT_AG th), Tn = a_n (fn + K_LT_ANT th)
+// with a = K_SE / (K_SE + K_LT); the globe balance Ta - Tn = K_P th fixes th.
+// The coefficients' 1 / K_SE are at hand.
 __device__ __forceinline__ void drive_equilibrium_k(const float* p, const Coef& k, float fa, float fn, float* s) {
   const float ag = __fdividef(1.0f, fmaf(p[kLtAg], k.iKa, 1.0f));     // K_SE / (K_SE + K_LT)
   const float an = __fdividef(1.0f, fmaf(p[kLtAnt], k.iKn, 1.0f));
@@ -164,24 +167,6 @@ __device__ __forceinline__ void rest_state(const float* p, float th, float* s) {
   s[3] = tn / p[kSeAnt] - th;
   s[4] = ta * (1.0f + p[kLtAg] / p[kSeAg]) + p[kLtAg] * th;
   s[5] = tn * (1.0f + p[kLtAnt] / p[kSeAnt]) - p[kLtAnt] * th;
-}
-
-// Equilibrium under constant active-state tensions (fa, fn): from x' = y' = 0
-// the series tensions are Ta = a_g (fa - K_LT_AG th), Tn = a_n (fn + K_LT_ANT th)
-// with a = K_SE / (K_SE + K_LT); the globe balance Ta - Tn = K_P th fixes th.
-__device__ __forceinline__ void drive_equilibrium(const float* p, float fa, float fn, float* s) {
-  const float ag = p[kSeAg] / (p[kSeAg] + p[kLtAg]);
-  const float an = p[kSeAnt] / (p[kSeAnt] + p[kLtAnt]);
-  const float kp = p[kNcAg] + p[kNcAnt];
-  const float th = (ag * fa - an * fn) / (kp + ag * p[kLtAg] + an * p[kLtAnt]);
-  const float ta = ag * (fa - p[kLtAg] * th);
-  const float tn = an * (fn + p[kLtAnt] * th);
-  s[0] = th;
-  s[1] = 0.0f;
-  s[2] = th + ta / p[kSeAg];
-  s[3] = tn / p[kSeAnt] - th;
-  s[4] = fa;
-  s[5] = fn;
 }
 
 // out = Zm * w for the sparse mechanical block Zm = h * A_mech, w dense 4x4
