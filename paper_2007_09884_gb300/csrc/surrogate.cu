@@ -34,12 +34,16 @@ constexpr int kSimThreads = 256;
 
 // Activations and gradients of one batch of M rows (M a multiple of 128).
 constexpr int kWgradSplit = 4;          // largest number of K slices of the weight-gradient GEMM
+// M and rows say what the buffers hold, so they are 0 while the buffers grow: an
+// allocation that fails leaves one of them gone (DevBuf::ensure frees before it
+// allocates), and the next call, of any size, allocates what is missing.
 struct MlpBuffers {
   int M = 0;        // rows of a training pass
   int rows = 0;     // rows of an inference pass (X, two layers' activations)
   DevBuf X, H[kLayers], Z[kLayers], Y, dY, rowloss, dZ[kLayers], colpart[kLayers], wpart, dWpart, dbpart;
   Status ensure(int m) {
     if (m <= M) return Status();
+    M = rows = 0;
     Status s;
     const size_t act = (size_t)m * kHidden;
     s = X.ensure(act * 2);
@@ -61,6 +65,7 @@ struct MlpBuffers {
   }
   Status ensure_inference(int m) {
     if (m <= rows) return Status();
+    M = rows = 0;
     const size_t act = (size_t)m * kHidden;
     Status s = X.ensure(act * 2);
     for (int l = 0; l < 2 && s.ok(); ++l) s = H[l].ensure(act * 2);
@@ -472,6 +477,7 @@ extern "C" int opmm_surrogate_train(opmm_ctx* ctx, int32_t steps, int32_t batch,
   MlpBuffers& B = S.buf;
   STRY(B.ensure(batch));
   if (S.train_M < batch) {
+    S.train_M = 0;   // until every slot has grown
     for (auto& D : S.slot) {
       STRY(D.sacs.ensure(sizeof(DevSac) * (size_t)batch));
       STRY(D.traces.ensure(sizeof(float) * (size_t)batch * kTrainLcap));

@@ -1,0 +1,87 @@
+"""The host code of the library on a CPU, over a CUDA runtime in host memory
+(tests/host/fake_cuda.cpp): after an allocation that failed, a later call of
+any size gets buffers that are there and large enough.  Every allocation of a
+call is made to fail in turn; a buffer that a launch is given and that is not
+live device memory of its size is counted."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import paper_2007_09884_gb300 as G
+from paper_2007_09884_gb300 import build as B
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="session")
+def lib(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("host") / "libopmm_host.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(B.nvcc()))), "include")
+    if not os.path.exists(os.path.join(cuda, "cuda_runtime.h")):
+        cuda = "/usr/local/cuda/include"
+    src = [os.path.join(B.CSRC, f) for f in ("capi.cu", "surrogate.cu", "serve.cu")]
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-pthread", "-Wl,-Bsymbolic", "-I", cuda, "-I", B.CSRC, "-include",
+                    os.path.join(HERE, "host", "device_names.h"), "-x", "c++", *src,
+                    os.path.join(HERE, "host", "fake_cuda.cpp"), "-o", out], check=True)
+    lib = ctypes.CDLL(out)
+    for f in ("fake_allocs", "fake_bad", "fake_in_use"):
+        getattr(lib, f).restype = ctypes.c_longlong
+    for f in ("fake_fail_alloc", "fake_capacity"):
+        getattr(lib, f).argtypes = [ctypes.c_longlong]
+    lib.opmm_destroy.restype = None
+    return lib
+
+
+@pytest.fixture
+def ctx(lib):
+    h = ctypes.c_void_p()
+    assert lib.opmm_create(0, ctypes.byref(h)) == G.OPMM_OK
+    assert lib.opmm_surrogate_init(h, ctypes.c_uint64(1)) == G.OPMM_OK
+    yield h
+    lib.fake_fail_alloc(-1)
+    lib.opmm_destroy(h)
+
+
+def _batch(n, L=60):
+    y = np.zeros(L, np.float32)
+    return G.make_batch([y] * n, [1000.0] * n, [10] * n, [0.0] * n, [10.0] * n, [43.0] * n)
+
+
+def _predict(lib, ctx, n):
+    descs, keep = _batch(n).descriptors()
+    out = np.zeros((n, 18), np.float32)
+    return lib.opmm_surrogate_predict(ctx, descs, n, G.OPMM_PULSE_CALIBRATED, out.ctypes.data_as(ctypes.c_void_p))
+
+
+def _train(lib, ctx, batch):
+    return lib.opmm_surrogate_train(ctx, 1, batch, ctypes.c_float(1e-3), ctypes.c_float(0.0), ctypes.c_uint64(1),
+                                    ctypes.c_int64(0), None)
+
+
+def _grad(lib, ctx, m):
+    x, t = np.zeros((m, 512), np.float32), np.zeros((m, 18), np.float32)
+    g, loss = np.zeros(4 * (512 * 512 + 512) + 18 * 513, np.float32), ctypes.c_float()
+    return lib.opmm_surrogate_grad(ctx, *(v.ctypes.data_as(ctypes.c_void_p) for v in (x, t)), m, ctypes.byref(loss),
+                                   g.ctypes.data_as(ctypes.c_void_p), None)
+
+
+@pytest.mark.parametrize("call", [_predict, _train, _grad], ids=["predict", "train", "grad"])
+def test_buffers_after_a_failed_allocation(lib, ctx, call):
+    bad = lib.fake_bad()
+    for nth in range(60):
+        assert call(lib, ctx, 256 * (1 + 3 * nth)) == G.OPMM_OK     # what a first call leaves behind
+        before = lib.fake_allocs()
+        lib.fake_fail_alloc(nth)
+        rc = call(lib, ctx, 256 * (3 + 3 * nth))                    # grows, and its nth allocation fails
+        hit = lib.fake_allocs() - before > nth
+        lib.fake_fail_alloc(-1)
+        assert rc == (G.OPMM_ENOMEM if hit else G.OPMM_OK)
+        assert call(lib, ctx, 256) == G.OPMM_OK                     # smaller than what was there
+        assert lib.fake_bad() == bad, f"allocation {nth} failed: a later launch got a buffer that is not there"
+        if not hit:
+            break
+    else:
+        pytest.fail("the call allocates more often than this test fails it")
