@@ -46,6 +46,22 @@ bool is_device_ptr(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Where a caller's floats are: kInPlace when a kernel on `device` may read them
+// there (that device's own memory, on a float's boundary), else what the
+// runtime copies them from.  Memory of another device (unreachable without
+// peer access), managed memory and odd addresses are copied, which takes all
+// of them.
+enum Place { kInPlace, kOnDevice, kOnHost };
+static Place place_of(const float* p, int device) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return kOnHost;
+  }
+  if (a.type != cudaMemoryTypeDevice) return a.type == cudaMemoryTypeManaged ? kOnDevice : kOnHost;
+  return a.device == device && (reinterpret_cast<uintptr_t>(p) & 3u) == 0 ? kInPlace : kOnDevice;
+}
+
 DevBuf::~DevBuf() { release(); }
 void DevBuf::release() {
   if (ptr) cudaFree(ptr);
@@ -330,9 +346,11 @@ extern "C" int opmm_score(opmm_ctx* ctx, const float* opc, int32_t m, const opmm
   DevBuf& b_tr = ctx->scratch[5];
   DevBuf& b_f = ctx->scratch[6];
   const float* d_trace = sac->trace_deg;
-  if (!is_device_ptr(d_trace)) {
+  const Place place = place_of(d_trace, ctx->device);
+  if (place != kInPlace) {
     TRY(b_tr.ensure(sizeof(float) * (size_t)d.L));
-    CUDA_TRY(cudaMemcpyAsync(b_tr.ptr, sac->trace_deg, sizeof(float) * (size_t)d.L, cudaMemcpyHostToDevice, st), "copy trace");
+    const cudaMemcpyKind kind = place == kOnDevice ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    CUDA_TRY(cudaMemcpyAsync(b_tr.ptr, sac->trace_deg, sizeof(float) * (size_t)d.L, kind, st), "copy trace");
     d_trace = b_tr.as<float>();
   }
   const bool opc_dev = is_device_ptr(opc), f_dev = is_device_ptr(out_f);

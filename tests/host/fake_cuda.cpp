@@ -24,17 +24,20 @@ struct Block {
 std::map<char*, Block> live;
 long long allocs = 0, fail_at = -1, bad = 0, in_use = 0;
 long long capacity = 1LL << 40;
+const void* scored_at = nullptr;
 
-bool inside(const void* p, size_t bytes, int device = 0) {
+// Inside one block of live memory, of the given device (-1: of any).
+bool inside(const void* p, size_t bytes, int device = -1) {
   std::lock_guard<std::mutex> lock(mu);
   char* c = (char*)p;
   auto it = live.upper_bound(c);
   if (it == live.begin()) return false;
   --it;
-  return it->second.device == device && c + bytes <= it->first + it->second.bytes;
+  return (device < 0 || it->second.device == device) && c + bytes <= it->first + it->second.bytes;
 }
+// A kernel of device 0 would access [p, p + bytes).
 void touch(const void* p, size_t bytes) {
-  if (!p || !inside(p, bytes)) ++bad;
+  if (!p || !inside(p, bytes, 0)) ++bad;
 }
 
 }  // namespace
@@ -43,7 +46,9 @@ extern "C" {
 void fake_fail_alloc(long long nth) { fail_at = nth < 0 ? -1 : allocs + nth; }   // the nth allocation from now (0: the next)
 long long fake_allocs() { return allocs; }
 long long fake_bad() { return bad; }
+const void* fake_scored_at() { return scored_at; }   // the trace that the last score kernel was given
 long long fake_in_use() { return in_use; }
+void fake_move(void* p, int device) { live[(char*)p].device = device; }   // as memory of another device
 void fake_capacity(long long c) { capacity = c; }
 
 cudaError_t cudaMalloc(void** p, size_t n) {
@@ -103,7 +108,7 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
   a->device = -2;
   if (inside(p, 1)) {
     a->type = cudaMemoryTypeDevice;
-    a->device = 0;
+    a->device = inside(p, 1, 0) ? 0 : 1;
   }
   return cudaSuccess;
 }
@@ -159,6 +164,8 @@ cudaError_t launch_simulate(const float* opc, int n, const DevSac*, const int*, 
 cudaError_t launch_score(const float* opc, int m, const DevSac& sac, const float* trace, float* f, int, cudaStream_t) {
   touch(opc, 72 * (size_t)m);
   touch(trace, 4 * (size_t)sac.L);
+  if ((uintptr_t)trace & 3) ++bad;
+  scored_at = trace;
   touch(f, 4 * (size_t)m);
   return cudaSuccess;
 }

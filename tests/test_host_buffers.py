@@ -1,8 +1,9 @@
 """The host code of the library on a CPU, over a CUDA runtime in host memory
-(tests/host/fake_cuda.cpp): after an allocation that failed, a later call of
-any size gets buffers that are there and large enough.  Every allocation of a
-call is made to fail in turn; a buffer that a launch is given and that is not
-live device memory of its size is counted."""
+(tests/host/fake_cuda.cpp), where a buffer that a launch is given and that is
+not live memory of the context's device, large enough, is counted: after an
+allocation that failed (every one of a call in turn), a later call of any size
+gets buffers that are there; a caller's memory is given to a kernel only where
+that can read it."""
 import ctypes
 import os
 import subprocess
@@ -29,6 +30,8 @@ def lib(tmp_path_factory):
     lib = ctypes.CDLL(out)
     for f in ("fake_allocs", "fake_bad", "fake_in_use"):
         getattr(lib, f).restype = ctypes.c_longlong
+    lib.fake_scored_at.restype = ctypes.c_void_p
+    lib.fake_move.argtypes = [ctypes.c_void_p, ctypes.c_int]
     for f in ("fake_fail_alloc", "fake_capacity"):
         getattr(lib, f).argtypes = [ctypes.c_longlong]
     lib.opmm_destroy.restype = None
@@ -85,3 +88,27 @@ def test_buffers_after_a_failed_allocation(lib, ctx, call):
             break
     else:
         pytest.fail("the call allocates more often than this test fails it")
+
+
+# where the caller keeps the trace: host memory, this device's, this device's off a float's boundary, another device's
+@pytest.mark.parametrize("where,in_place", [("host", False), ("device", True), ("odd", False), ("other", False)])
+def test_score_reads_a_trace_in_place_only_where_its_kernel_can(lib, ctx, where, in_place):
+    L, m = 61, 5
+    y = np.arange(L, dtype=np.float32)
+    block = ctypes.c_void_p()
+    assert lib.cudaMalloc(ctypes.byref(block), ctypes.c_size_t(4 * L + 4)) == 0
+    at = block.value + (2 if where == "odd" else 0)
+    ctypes.memmove(at, y.ctypes.data, 4 * L)
+    if where == "other":
+        lib.fake_move(block, 1)
+    if where == "host":
+        at = y.ctypes.data
+    sac = G.opmm_saccade(at, L, 1000.0, 10, 0.0, 10.0, 43.0)
+    opc, f = np.full((m, 18), 1.0, np.float32), np.zeros(m, np.float32)
+    bad = lib.fake_bad()
+    assert lib.opmm_score(ctx, opc.ctypes.data_as(ctypes.c_void_p), m, ctypes.byref(sac),
+                          f.ctypes.data_as(ctypes.c_void_p)) == G.OPMM_OK
+    assert lib.fake_bad() == bad
+    assert (lib.fake_scored_at() == at) == in_place
+    np.testing.assert_array_equal(np.frombuffer(ctypes.string_at(lib.fake_scored_at(), 4 * L), np.float32), y)
+    assert lib.cudaFree(block) == 0
