@@ -2005,7 +2005,11 @@ cudaError_t launch_score(const float* opc, int m, const DevSac& sac, const float
   int blocks = (m + kScoreThreads - 1) / kScoreThreads;
   if (blocks > 8 * num_sms) blocks = 8 * num_sms;
   const size_t smem = (size_t)sac.L * sizeof(float);
-  if (smem > 48 * 1024) {
+  // without asking a block gets 48 KB of static and dynamic shared memory
+  // together; asking costs four runtime calls, so short windows do without.
+  // The static part is TraceStage, at most one alignment of the dynamic part.
+  static_assert(sizeof(TraceStage) <= 128, "static shared memory of k_score");
+  if (smem + 128 > 48 * 1024) {
     cudaError_t e = allow_dynamic_smem(k_score, smem);
     if (e != cudaSuccess) return e;
   }
