@@ -77,40 +77,52 @@ struct KahanSink {
   }
 };
 
-// Writes a trajectory's samples, which come in order from k = 0, four at a
-// time where they fill an aligned 16-byte group.  Every thread of a warp
-// writes its own row, so a store of single samples touches 32 sectors for 128
-// bytes; in groups it takes a quarter of the transactions.
+// Writes a trajectory after its samples at rest.  Every thread of a warp writes
+// its own row, so a store of single samples touches 32 sectors for 128 bytes;
+// GROUPS: four at a time where they fill an aligned 16-byte group, which takes
+// a quarter of the transactions (rows with three samples at rest or more: no
+// later group then begins before the row).  The last three samples shift
+// through registers, which the unrolled sample loops resolve by renaming; an
+// array position chosen per sample (compares, selects and a branch) took 65 ns
+// a sample where these take 27, and more than the whole walk of one row.
+template <bool GROUPS>
 struct WriteSink {
   float* out;
   float sign, thf;
-  int lead;            // samples by which out is past an aligned group
-  float b0, b1, b2;
-  __device__ __forceinline__ WriteSink(float* o, float sg, float th) : out(o), sign(sg), thf(th), b0(0), b1(0), b2(0) {
-    lead = (int)((reinterpret_cast<uintptr_t>(o) >> 2) & 3);
-  }
-  __device__ __forceinline__ void put(int k, float v) {
-    const int s = (lead + k) & 3;
-    if (k < s) {
-      out[k] = v;      // the row's first group is not whole
-      return;
+  float b1, b2, b3;    // the last three samples
+  // all samples so far have the value v
+  __device__ __forceinline__ WriteSink(float* o, float sg, float th, float v) : out(o), sign(sg), thf(th), b1(v), b2(v), b3(v) {}
+  __device__ __forceinline__ void emit(int k, float dth) {
+    const float v = sign * (thf + dth);
+    float* o = out + k;
+    if constexpr (!GROUPS) {
+      *o = v;
+    } else {
+      if ((~(unsigned)reinterpret_cast<uintptr_t>(o) & 12u) == 0) *reinterpret_cast<float4*>(o - 3) = make_float4(b1, b2, b3, v);
+      b1 = b2;
+      b2 = b3;
+      b3 = v;
     }
-    if (s == 3) *reinterpret_cast<float4*>(out + k - 3) = make_float4(b0, b1, b2, v);
-    b0 = s == 0 ? v : b0;
-    b1 = s == 1 ? v : b1;
-    b2 = s == 2 ? v : b2;
   }
-  __device__ __forceinline__ void emit(int k, float dth) { put(k, sign * (thf + dth)); }
   __device__ __forceinline__ void block_end() {}
   // the n samples' last, partial group
   __device__ __forceinline__ void finish(int n) {
-    const int s = (lead + n) & 3;
-    if (n < s) return;
-    if (s > 0) out[n - s] = b0;
-    if (s > 1) out[n - s + 1] = b1;
-    if (s > 2) out[n - s + 2] = b2;
+    if constexpr (GROUPS) {
+      const int s = (int)((reinterpret_cast<uintptr_t>(out + n) >> 2) & 3);
+      if (s > 0) out[n - 1] = b3;
+      if (s > 1) out[n - 2] = b2;
+      if (s > 2) out[n - 3] = b1;
+    }
   }
 };
+
+// Samples 0 .. n - 1 of a row have the value v.
+__device__ __forceinline__ void write_rest(float* out, int n, float v) {
+  int k = 0;
+  for (; k < n && (reinterpret_cast<uintptr_t>(out + k) & 15u); ++k) out[k] = v;
+  for (; k + 4 <= n; k += 4) *reinterpret_cast<float4*>(out + k) = make_float4(v, v, v, v);
+  for (; k < n; ++k) out[k] = v;
+}
 
 struct PeakSink {
   float m;
@@ -277,7 +289,7 @@ __global__ void k_nominal(const DevSac* sacs, int n, int pulse_mode, const float
 
 // ------------------------------------------------------------------ simulate
 __global__ void __launch_bounds__(256) k_simulate(const float* opc, int n, const DevSac* sacs, const int* sac_of,
-                           const long long* out_off, float* out) {
+                           const long long* out_off, float* out, bool groups) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   float p[kNumParams];
@@ -285,13 +297,20 @@ __global__ void __launch_bounds__(256) k_simulate(const float* opc, int n, const
   for (int j = 0; j < kNumParams; ++j) p[j] = opc[(size_t)i * kNumParams + j];
   const DevSac d = sacs[sac_of ? sac_of[i] : i];
   const SacConst sc = sac_const(d);
-  WriteSink w(out + out_off[i], d.sign, d.thf);
-  const int kend = min(d.onset, d.L - 1);
-  for (int k = 0; k <= kend; ++k) w.put(k, d.sign * d.th0);
+  float* row = out + out_off[i];
+  const int rest = min(d.onset, d.L - 1) + 1;
+  const float v0 = d.sign * d.th0;
+  write_rest(row, rest, v0);
   PackedWalk pw;
   pw.setup(p, sc);
-  pw.samples(p, sc, w);
-  w.finish(d.L);
+  if (groups && rest >= 3) {
+    WriteSink<true> w(row, d.sign, d.thf, v0);
+    pw.samples(p, sc, w);
+    w.finish(d.L);
+  } else {
+    WriteSink<false> w(row, d.sign, d.thf, v0);
+    pw.samples(p, sc, w);
+  }
 }
 
 // ------------------------------------------------------------------ score
@@ -1995,7 +2014,12 @@ cudaError_t launch_nominal(const DevSac* sacs, int n, int pulse_mode, const floa
 cudaError_t launch_simulate(const float* opc, int n, const DevSac* sacs, const int* sac_of,
                             const long long* out_off, float* out, cudaStream_t st, int threads) {
   if (n <= 0) return cudaSuccess;
-  k_simulate<<<(n + threads - 1) / threads, threads, 0, st>>>(opc, n, sacs, sac_of, out_off, out);
+  // Stores in groups of four bound a block by its walk (a window of 16,384
+  // samples 0.49 ms from 1 to 1,000 rows), single ones by the rows it writes
+  // (0.42 ms for 33 rows, 0.58 for 64, 1.10 for 128): equal at about 53 rows.
+  // 20,000 such windows 1.04 ms against 2.80.
+  constexpr int kGroupRows = 48;
+  k_simulate<<<(n + threads - 1) / threads, threads, 0, st>>>(opc, n, sacs, sac_of, out_off, out, n >= kGroupRows);
   return cudaGetLastError();
 }
 
