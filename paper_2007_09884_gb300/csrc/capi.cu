@@ -20,6 +20,7 @@
 #include "common.cuh"
 #include "launch.h"
 #include "runtime.h"
+#include "split.h"
 
 using opmm::DevSac;
 
@@ -497,42 +498,10 @@ Status enqueue_fit(opmm_plan* p, cudaStream_t st) {
                      "D2H error word");
 }
 
-// One Nelder-Mead step of a search unit against its 32-candidate chunks, in
-// thousands of SM cycles (2 x 32 packed, 150 samples at 1 kHz; one simplex
-// 22.6, 8 33.7, 16 39.8, 32 53.1, 48 79.2, 64 simplices 101): a chunk's and a
-// decision's latency first, the SM's throughput from about 24 chunks on.
-static double unit_step(int chunks) { return std::max(21.0 + 1.5 * chunks, 5.0 + 2.18 * chunks); }
-
-// Units per saccade: the number of units that n saccades' S simplices are
-// split into evenly, at most G simplices each, or 0 for full units of G and a
-// last one with the rest.  The split with the least turns of the blocks times
-// the step of one unit: a batch with many units per block keeps its units as
-// large as they come (a simplex costs 1.6 k cycles a step in a unit of 64 and
-// 2.5 k in one of 16), a few saccades are spread over every SM (one saccade
-// of 186 simplices: 93 units of two instead of 6 of 32).  A simplex evolves
-// the same in any unit, so the results do not depend on the split.
+// Units per saccade of a variant's split (split.h).
 static int split_units(int n, int S, int variant, int blocks) {
-  const int G = search_variant_g(variant), NG = search_variant_groups(variant);
-  const int nt = search_variant_dim(variant) + 4;
-  auto step = [&](int m) {   // one step of a unit of m simplices in NG even groups
-    int chunks = 0;
-    for (int h = 0; h < NG; ++h) chunks += (nt * ((m * (h + 1)) / NG - (m * h) / NG) + 31) / 32;
-    return unit_step(chunks);
-  };
-  auto turns = [&](int ng) { return std::max(1.0, (double)(((long long)n * ng + blocks - 1) / blocks)); };
-  const int least = (S + G - 1) / G;
-  double best = 1e300;
-  int pick = least;
-  for (int ng = least; ng <= S; ++ng) {
-    const double t = turns(ng) * step((S + ng - 1) / ng);
-    if (t < best * 0.999) {
-      best = t;
-      pick = ng;
-    }
-  }
-  // with many units per saccade an even split only rounds every group up to
-  // whole chunks, and full units lose only in their last one
-  return pick == least && (S % G == 0 || least > 8) ? 0 : pick;
+  return split_units(n, S, SplitShape{search_variant_g(variant), search_variant_groups(variant), search_variant_dim(variant) + 4},
+                     blocks);
 }
 
 // Candidate launch shapes: the search kernel's variants (simplices per block G,
