@@ -530,7 +530,8 @@ static std::vector<std::pair<int, int>> shape_candidates(int lcap, int dim, int 
 
 // Project-written autotuner: time each candidate shape on a sample of this
 // plan's own batch and keep the fastest; the choice is cached per (device,
-// trace capacity, simplices, saccade count bucket).  The sample is every
+// trace capacity, simplices, saccade count bucket, iterations, candidate
+// shapes).  The sample is every
 // k-th saccade in the unit list's order (longest windows first), about
 // kProbeSimplices simplices in all, run for the plan's own iteration count
 // (at most kProbeIters): shapes differ in how they overlap a group's
@@ -540,12 +541,15 @@ static std::vector<std::pair<int, int>> shape_candidates(int lcap, int dim, int 
 // Results of probe runs are overwritten by the real run.
 static Status autotune(opmm_plan* p) {
   opmm_ctx* ctx = p->ctx;
-  // the probes run the plan's own iteration count (at most 32), so it is part
-  // of the key, with the model's coordinate count
-  const auto key = std::make_tuple(p->lcap, p->S, p->n >= 64 ? 64 : p->n,
-                                   std::min(p->opts.iterations, 32) * 64 + (p->dim << 1));
-  auto it = ctx->tune_cache.find(key);
   auto cands = shape_candidates(p->lcap, p->dim, p->n, p->S, ctx->num_sms);
+  unsigned tried = 0;
+  for (const auto& c : cands) tried |= 1u << c.first;
+  // the probes run the plan's own iteration count (at most 32), so it is part
+  // of the key, with the model's coordinate count, and so are the shapes that
+  // are tried, which depend on the exact number of saccades
+  const auto key = std::make_tuple(p->lcap, p->S, p->n >= 64 ? 64 : p->n,
+                                   std::min(p->opts.iterations, 32) * 64 + (p->dim << 1), tried);
+  auto it = ctx->tune_cache.find(key);
   if (cands.empty()) return Status(OPMM_ECUDA, "no launchable search shape (shared memory)");
   if (ctx->forced_variant >= 0) {
     int bps = 0;

@@ -107,8 +107,8 @@ struct opmm_ctx {
   opmm::HostBuf h_scratch[2];         // pinned host scratch of the synchronous entry points
   opmm::FitBuffers once;              // buffers of the one-shot fit calls
   std::mutex once_mu;                 // guards `once` and the surrogate's spare buffers while they change hands
-  std::map<std::tuple<int, int, int, int>, std::pair<int, int>> tune_cache;
-  std::map<std::tuple<int, int, int, int>, std::vector<opmm::TuneProbe>> tune_logs;
+  std::map<std::tuple<int, int, int, int, unsigned>, std::pair<int, int>> tune_cache;
+  std::map<std::tuple<int, int, int, int, unsigned>, std::vector<opmm::TuneProbe>> tune_logs;
   opmm::SurrogateState* surrogate = nullptr;   // owned, released by surrogate_release
   opmm::ServeState* serve = nullptr;           // owned, released by serve_shutdown
   opmm_ctx();

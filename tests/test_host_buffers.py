@@ -34,7 +34,7 @@ def lib(tmp_path_factory):
     lib.fake_move.argtypes = [ctypes.c_void_p, ctypes.c_int]
     for f in ("fake_fail_alloc", "fake_capacity"):
         getattr(lib, f).argtypes = [ctypes.c_longlong]
-    lib.opmm_destroy.restype = None
+    lib.opmm_destroy.restype = lib.opmm_plan_destroy.restype = None
     return lib
 
 
@@ -112,3 +112,26 @@ def test_score_reads_a_trace_in_place_only_where_its_kernel_can(lib, ctx, where,
     assert (lib.fake_scored_at() == at) == in_place
     np.testing.assert_array_equal(np.frombuffer(ctypes.string_at(lib.fake_scored_at(), 4 * L), np.float32), y)
     assert lib.cudaFree(block) == 0
+
+
+def _tuned_shapes(lib, ctx, n, simplices):
+    descs, keep = _batch(n).descriptors()
+    o, keep_o = G.fit_opts(candidates=22 * simplices, iterations=4)
+    plan = ctypes.c_void_p()
+    assert lib.opmm_plan_create(ctx, descs, n, ctypes.byref(o), ctypes.byref(plan)) == G.OPMM_OK
+    variants, count = (ctypes.c_int32 * 16)(), ctypes.c_int32()
+    assert lib.opmm_plan_tuning(plan, variants, None, None, None, None, 16, ctypes.byref(count)) == G.OPMM_OK
+    lib.opmm_plan_destroy(plan)
+    return variants[:count.value]
+
+
+# 64 saccades of 64 simplices leave every unit at 32 simplices, so the larger shapes are not tried; 3,000 do not
+@pytest.mark.parametrize("first,then", [(64, 3000), (3000, 64), (74, 1024)])
+def test_tuning_does_not_depend_on_an_earlier_plan(lib, ctx, first, then):
+    fresh = ctypes.c_void_p()
+    assert lib.opmm_create(0, ctypes.byref(fresh)) == G.OPMM_OK
+    want = _tuned_shapes(lib, fresh, then, 64)
+    lib.opmm_destroy(fresh)
+    assert _tuned_shapes(lib, ctx, first, 64) != want          # the two batches have different candidate shapes
+    assert _tuned_shapes(lib, ctx, then, 64) == want
+    assert _tuned_shapes(lib, ctx, then, 64) == want           # and again, from the cache
