@@ -235,7 +235,7 @@ class SaccadeBatch:
             p, k = _ptr(self.traces)
             keep.append(k)
             if n > _FEW:
-                bases = np.uint64(p.value or 0) + (np.asarray(self.offsets, np.int64) * 4).view(np.uint64)
+                bases = np.uint64(p.value or 0) + (np.asarray(_host(self.offsets), np.int64) * 4).view(np.uint64)
             else:
                 bases = [(p.value or 0) + int(o) * 4 for o in self.offsets]
         return self._fill(bases), keep
@@ -292,7 +292,7 @@ class SaccadeBatch:
             return arr
         d = np.frombuffer(arr, _SACCADE_DTYPE)
         for name in _SACCADE_DTYPE.names:
-            v = bases if name == "trace_deg" else getattr(self, name)
+            v = bases if name == "trace_deg" else _host(getattr(self, name))
             if len(v) < n:
                 raise IndexError(f"{name} has {len(v)} entries for {n} saccades")
             d[name] = v[:n]
@@ -303,6 +303,11 @@ class SaccadeBatch:
 _FEW = 6
 # mean length up to which a list of traces is gathered
 _GATHER_SAMPLES = 1500
+
+
+def _host(v):
+    """Values that numpy reads: a tensor's, wherever it lives, else v itself."""
+    return v.detach().cpu().numpy() if _is_torch(v) else v
 
 
 def _is_flat(a) -> bool:

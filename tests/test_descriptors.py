@@ -103,3 +103,27 @@ def test_fits_read_every_trace(lib, n, L, dtype):
         np.testing.assert_array_equal(d["samples"], batch.traces[i].astype(np.float32))
         if dtype == np.float32 and (long or n <= 6):
             assert d["trace_deg"] == batch.traces[i].ctypes.data
+
+
+# what indexes and converts entry by entry is taken at every size: lists, arrays of other types, tensors (of the
+# device too: any that numpy does not read by itself)
+@pytest.mark.parametrize("n", [3, 7, 50])
+@pytest.mark.parametrize("kind", ["list", "float64", "tensor", "grad"])
+def test_fields_and_offsets_of_every_kind(lib, n, kind):
+    torch = pytest.importorskip("torch")
+    ref = _batch(n, 300)
+    offsets = np.concatenate([[0], np.cumsum(ref.n_samples)[:-1]])
+    convert = {"list": lambda v: [x.item() for x in v], "float64": lambda v: v.astype(np.float64),
+               "tensor": lambda v: torch.tensor(v.tolist()),
+               "grad": lambda v: torch.tensor(v.tolist(), dtype=torch.float64, requires_grad=True)}[kind]
+    packed = np.concatenate(ref.traces)
+    batch = G.SaccadeBatch(packed, convert(offsets), *(convert(getattr(ref, f)) for f in FIELDS))
+    G.opmm_fit_batch(None, batch)
+    for i, d in enumerate(lib.got):
+        _check(d, ref, i)
+        np.testing.assert_array_equal(d["samples"], ref.traces[i])
+    batch = G.SaccadeBatch(ref.traces, None, *(convert(getattr(ref, f)) for f in FIELDS))
+    G.opmm_fit_batch(None, batch)
+    for i, d in enumerate(lib.got):
+        _check(d, ref, i)
+        np.testing.assert_array_equal(d["samples"], ref.traces[i])
