@@ -29,6 +29,11 @@
  *    shows the plant for positive saccades).
  *  - A context is not thread-safe except for the serving calls, which may be
  *    made from any thread.
+ *  - A context keeps buffers between the calls that fit, refine, predict or
+ *    featurize a batch: up to 1 GiB of device and pinned memory for batches
+ *    and up to 1 GiB of device memory for the network's activations (a larger
+ *    call frees its own).  They are freed with the context, before the request
+ *    loop sizes its slots, and when an allocation of this library fails.
  */
 #ifndef OPMM_H
 #define OPMM_H

@@ -63,6 +63,38 @@ static Place place_of(const float* p, int device) {
   return a.device == device && (reinterpret_cast<uintptr_t>(p) & 3u) == 0 ? kInPlace : kOnDevice;
 }
 
+// The contexts that exist.  They are walked when an allocation fails, on any
+// thread: a context's kept buffers change hands under its once_mu only.
+static std::mutex all_mu;
+static std::vector<opmm_ctx*> all_contexts;
+
+bool give_back_kept() {
+  std::lock_guard<std::mutex> all(all_mu);
+  bool any = false;
+  for (opmm_ctx* c : all_contexts) {
+    FitBuffers fit;
+    std::shared_ptr<MlpBuffers> infer;
+    {
+      std::lock_guard<std::mutex> lock(c->once_mu);
+      fit.swap(c->once);
+      infer.swap(c->once_infer);
+    }
+    any = any || fit.bytes() > 0 || infer;
+  }   // freed here
+  return any;
+}
+
+// Runs an allocation, once more if it fails while buffers are kept.
+template <class F>
+static cudaError_t allocate(F f) {
+  cudaError_t e = f();
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    if (give_back_kept()) e = f();
+  }
+  return e;
+}
+
 DevBuf::~DevBuf() { release(); }
 void DevBuf::release() {
   if (ptr) cudaFree(ptr);
@@ -73,7 +105,7 @@ Status DevBuf::ensure(size_t want) {
   if (want <= bytes && ptr) return Status();
   release();
   if (want == 0) want = 16;
-  cudaError_t e = cudaMalloc(&ptr, want);
+  cudaError_t e = allocate([&] { return cudaMalloc(&ptr, want); });
   if (e != cudaSuccess) {
     ptr = nullptr;
     cudaGetLastError();
@@ -93,7 +125,7 @@ Status HostBuf::ensure(size_t want) {
   if (want <= bytes && ptr) return Status();
   release();
   if (want == 0) want = 16;
-  cudaError_t e = cudaHostAlloc(&ptr, want, cudaHostAllocDefault);
+  cudaError_t e = allocate([&] { return cudaHostAlloc(&ptr, want, cudaHostAllocDefault); });
   if (e != cudaSuccess) {
     ptr = nullptr;
     cudaGetLastError();
@@ -223,12 +255,20 @@ extern "C" int opmm_create(int device_ordinal, opmm_ctx** out) {
     return code;
   }
   ctx->stream = ctx->own_stream;
+  {
+    std::lock_guard<std::mutex> lock(all_mu);
+    all_contexts.push_back(ctx);
+  }
   *out = ctx;
   return OPMM_OK;
 }
 
 extern "C" void opmm_destroy(opmm_ctx* ctx) {
   if (!ctx) return;
+  {
+    std::lock_guard<std::mutex> lock(all_mu);
+    all_contexts.erase(std::remove(all_contexts.begin(), all_contexts.end(), ctx), all_contexts.end());
+  }
   cudaSetDevice(ctx->device);
   serve_shutdown(ctx);
   surrogate_release(ctx);

@@ -75,7 +75,8 @@ struct HostBuf {
 // results.  A plan owns its own; one-shot calls borrow the context's, which
 // keep their size from call to call up to kKeepBytes in all (allocating and
 // freeing them took 0.1 ms of a 1.1 ms single fit, and each free waits for
-// the device).
+// the device).  What is kept is given back before the request loop sizes its
+// slots, and when an allocation of the library fails (give_back_kept).
 struct FitBuffers {
   DevBuf d_sacs, d_traces, d_pc, d_sac_index, d_units, d_ustart, d_unit_best, d_counter, d_results, d_src;
   DevBuf d_pc_given;            // caller's centres when the surrogate rescales them
@@ -85,6 +86,7 @@ struct FitBuffers {
   size_t bytes() const;
 };
 
+struct MlpBuffers;       // activations of the surrogate (surrogate.cu)
 struct SurrogateState;
 struct ServeState;
 
@@ -106,7 +108,8 @@ struct opmm_ctx {
   opmm::DevBuf scratch[16];           // per-call scratch of the synchronous entry points
   opmm::HostBuf h_scratch[2];         // pinned host scratch of the synchronous entry points
   opmm::FitBuffers once;              // buffers of the one-shot fit calls
-  std::mutex once_mu;                 // guards `once` and the surrogate's spare buffers while they change hands
+  std::shared_ptr<opmm::MlpBuffers> once_infer;   // inference buffers of the one-shot calls, up to kKeepBytes
+  std::mutex once_mu;                 // guards `once` and `once_infer` while they change hands
   std::map<std::tuple<int, int, int, int, unsigned>, std::pair<int, int>> tune_cache;
   std::map<std::tuple<int, int, int, int, unsigned>, std::vector<opmm::TuneProbe>> tune_logs;
   opmm::SurrogateState* surrogate = nullptr;   // owned, released by surrogate_release
@@ -161,6 +164,10 @@ void pack_host_traces(opmm_plan* p);
 void surrogate_release(opmm_ctx* ctx);
 // once: the plan is used by this call only and may borrow the context's buffers
 Status surrogate_prepare_plan(opmm_ctx* ctx, opmm_plan* p, int32_t n, bool once);
+
+// Frees what the contexts keep between calls (buffers that a call has borrowed
+// are not among it); whether there was any.
+bool give_back_kept();
 
 // Lends the context's one-shot buffers to a plan for the length of a call.
 struct BorrowBuffers {

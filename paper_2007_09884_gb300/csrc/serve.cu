@@ -288,6 +288,7 @@ extern "C" int opmm_serve_start(opmm_ctx* ctx, const opmm_serve_opts* cfg, const
   const size_t slot_bytes = (size_t)sv->S * kSearchStateFloats * 4 + (size_t)sv->ngroups * kUnitRecFloats * 4 +
                             (size_t)sv->lcap * 4 + OPMM_NPARAM * 4 + sizeof(DevSac) + sizeof(opmm_fit_result) + 16;
   size_t free_b = 0, total_b = 0;
+  give_back_kept();   // memory that earlier calls left for the next ones counts as free
   if (s.ok()) s = cuda_status(cudaMemGetInfo(&free_b, &total_b), "memory info");
   size_t budget = cfg->max_device_bytes ? (size_t)cfg->max_device_bytes : free_b / 2;
   if (budget > free_b) budget = free_b;

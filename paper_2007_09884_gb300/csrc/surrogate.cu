@@ -79,7 +79,6 @@ struct SurrogateState {
   DevBuf cal_amp, cal_pulse;             // agonist pulse by amplitude (calibrated nominal)
   MlpBuffers buf;
   MlpBuffers infer;                      // admission-time inference of the request loop
-  std::unique_ptr<MlpBuffers> spare;     // inference buffers of the last one-shot call (once_mu)
   // training data: two slots, so that one batch is generated (on a side
   // stream) while the network trains on the other
   struct DataSlot {
@@ -319,17 +318,16 @@ Status surrogate_prepare_plan(opmm_ctx* ctx, opmm_plan* p, int32_t n, bool once)
   // and leaves them for the next
   std::shared_ptr<MlpBuffers> keep;
   if (once) {
-    MlpBuffers* b = nullptr;
+    std::shared_ptr<MlpBuffers> own;
     {
       std::lock_guard<std::mutex> lock(ctx->once_mu);
-      b = ctx->surrogate->spare.release();
+      own.swap(ctx->once_infer);
     }
-    keep = std::shared_ptr<MlpBuffers>(b ? b : new MlpBuffers(), [ctx](MlpBuffers* q) {
-      std::unique_ptr<MlpBuffers> own(q), old;   // `old` is freed outside the lock
+    if (!own) own = std::make_shared<MlpBuffers>();
+    keep = std::shared_ptr<MlpBuffers>(own.get(), [ctx, own](MlpBuffers* q) mutable {
       if ((size_t)q->rows * kHidden * 6 > FitBuffers::kKeepBytes) return;
       std::lock_guard<std::mutex> lock(ctx->once_mu);
-      old.swap(ctx->surrogate->spare);
-      ctx->surrogate->spare.swap(own);
+      own.swap(ctx->once_infer);   // what is there already is freed with `own`, outside the lock
     });
   } else {
     keep = std::make_shared<MlpBuffers>();

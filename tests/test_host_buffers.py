@@ -135,3 +135,47 @@ def test_tuning_does_not_depend_on_an_earlier_plan(lib, ctx, first, then):
     assert _tuned_shapes(lib, ctx, first, 64) != want          # the two batches have different candidate shapes
     assert _tuned_shapes(lib, ctx, then, 64) == want
     assert _tuned_shapes(lib, ctx, then, 64) == want           # and again, from the cache
+
+
+def _slots(lib, ctx):
+    cfg = G.opmm_serve_opts(max_slots=1 << 30, max_queue=4, max_samples=400, round_iters=5, max_admit_per_round=4)
+    o, keep = G.fit_opts(candidates=4096, iterations=4)
+    stats = G.opmm_serve_stats()
+    assert lib.opmm_serve_start(ctx, ctypes.byref(cfg), ctypes.byref(o)) == G.OPMM_OK
+    assert lib.opmm_serve_stats_get(ctx, ctypes.byref(stats)) == G.OPMM_OK
+    assert lib.opmm_serve_stop(ctx) == G.OPMM_OK
+    return stats.slots
+
+
+def test_kept_buffers_do_not_shrink_the_request_loop(lib, ctx):
+    lib.fake_capacity(lib.fake_in_use() + (1 << 30))
+    try:
+        slots = _slots(lib, ctx)
+        assert _predict(lib, ctx, 50000) == G.OPMM_OK     # leaves 150 MB of activations and 30 MB beside
+        assert lib.fake_in_use() > (100 << 20)
+        assert _slots(lib, ctx) == slots
+    finally:
+        lib.fake_capacity(1 << 40)
+
+
+@pytest.mark.parametrize("call", [_train, _grad], ids=["train", "grad"])
+def test_kept_buffers_are_given_back_when_memory_runs_out(lib, ctx, call):
+    m = 128 * 200
+    own = lib.fake_in_use()
+    other = ctypes.c_void_p()
+    assert lib.opmm_create(0, ctypes.byref(other)) == G.OPMM_OK
+    assert lib.opmm_surrogate_init(other, ctypes.c_uint64(1)) == G.OPMM_OK
+    base = lib.fake_in_use()
+    assert call(lib, other, m) == G.OPMM_OK
+    need = lib.fake_in_use() - base
+    lib.opmm_destroy(other)
+    assert _predict(lib, ctx, 50000) == G.OPMM_OK
+    kept = lib.fake_in_use() - own
+    assert kept > (100 << 20)
+    lib.fake_capacity(own + need + (64 << 20))            # room for the call, but not beside what is kept
+    try:
+        assert call(lib, ctx, m) == G.OPMM_OK
+    finally:
+        lib.fake_capacity(1 << 40)
+    assert _predict(lib, ctx, 300) == G.OPMM_OK           # and the next one-shot call allocates anew
+    assert lib.fake_bad() == 0
