@@ -991,7 +991,7 @@ __global__ void __launch_bounds__(search_threads<G, N>(), MINB) k_search(SearchP
       g.done = 0;
     }
     if (it0 > 0) {
-      // restore the simplices: vertices, values, centroid, order, flags
+      // restore the simplices: vertices, values, order, flags
       const float* gstate = P.state + ((size_t)b * P.S + (size_t)s0) * state_floats<N>();
       for (int idx = tid; idx < nunit * state_floats<N>(); idx += NT) {
         const int sg = idx / state_floats<N>(), r = idx - sg * state_floats<N>();

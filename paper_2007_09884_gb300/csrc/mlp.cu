@@ -845,19 +845,24 @@ __device__ __forceinline__ float u01(uint32_t x) { return (float)(x >> 8) * (1.0
 // normalised by the amplitude (start fixation = 0, end fixation = 1) and
 // velocity as 10 x the per-millisecond difference.  Output BF16 [n][512].
 // One warp per saccade, lane l the point pairs 2 l + 64 j, stored as they are
-// formed: nothing is staged, so a block needs no shared memory and runs
-// beside a network block that takes nearly all of an SM's (training data are
-// made while the network trains), and 4,096 saccades are 1,024 blocks at once
-// instead of 128 that take eight saccades per warp in turn.  Bound by the
-// chain descriptor -> samples -> store: 4,096 training
-// saccades with their noise 6.2 us, where noise (8 us) and features (12 us)
+// formed: the features are not staged, so a block runs beside a network block
+// that takes nearly all of an SM's shared memory (training data are made while
+// the network trains), and 4,096 saccades are 1,024 blocks at once instead of
+// 128 that take eight saccades per warp in turn.  Bound by the chain
+// descriptor -> samples -> store: 4,096 training saccades with their noise 6.2
+// us, where noise (8 us) and features (12 us, 33 KB of shared memory a block)
 // took two kernels; 96 training steps 11.6 -> 10.7 ms, since the network's
 // blocks no longer wait for an SM whose shared memory features hold.
 constexpr int kFeatWarps = 4;
 static_assert(kFeatPoints % 64 == 0 && kIn == 2 * kFeatPoints, "whole pairs per lane");
+// the noisy trajectories (below) leave room beside a network block: 228 KB an
+// SM, of which every block takes 1 KB besides its own
+static_assert(sizeof(float) * kFeatWarps * kTrainLcap + gemm_smem(6, 128) + 2 * 1024 <= 228 * 1024 &&
+                  sizeof(float) * kFeatWarps * kTrainLcap + gemm_smem(4, 256) + 2 * 1024 <= 228 * 1024,
+              "a features block fits beside a network block");
 
 // NOISE: training data.  The warp first takes its trajectory to shared memory
-// with N(0, sigma^2) deg of noise added (Philox stream 3 of sample *base + b,
+// (6.4 KB a block) with N(0, sigma^2) deg of noise added (Philox stream 3 of sample *base + b,
 // a Box-Muller pair per two samples), as far as the features reach; a noise
 // kernel of its own wrote and read every trajectory once more.
 template <bool NOISE>
@@ -916,13 +921,9 @@ __global__ void __launch_bounds__(32 * kFeatWarps) k_featurize(const DevSac* sac
   }
 }
 
-// Device-side counters of a replayable training step: *p64 += by64 (the
-// sample base of a data slot), *p32 += 1 (the step index).
-__global__ void k_bump(long long* p64, long long by64, int* p32) {
-  if (threadIdx.x == 0) {
-    if (p64) *p64 += by64;
-    if (p32) *p32 += 1;
-  }
+// Sample base of a data slot's next batch in a replayable training step.
+__global__ void k_bump(long long* p, long long by) {
+  if (threadIdx.x == 0) *p += by;
 }
 
 // Training data: per sample g = base + i, Philox4x32-10 (key = seed,
@@ -1175,8 +1176,8 @@ cudaError_t featurize_noisy(uint64_t seed, const long long* base, const DevSac* 
   return cudaGetLastError();
 }
 
-cudaError_t bump(long long* p64, long long by64, int* p32, cudaStream_t st) {
-  k_bump<<<1, 32, 0, st>>>(p64, by64, p32);
+cudaError_t bump(long long* p, long long by, cudaStream_t st) {
+  k_bump<<<1, 32, 0, st>>>(p, by);
   return cudaGetLastError();
 }
 

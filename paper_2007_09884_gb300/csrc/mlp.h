@@ -155,7 +155,7 @@ cudaError_t adamw(float* w, const float* g, float* m1, float* m2, int n, float l
                   float wd, int step, const AdamLayout& L, __nv_bfloat16* wb, cudaStream_t st);
 cudaError_t pack_params(const float* w, int n, const AdamLayout& L, __nv_bfloat16* wb, cudaStream_t st);
 cudaError_t featurize(const DevSac* sacs, const float* traces, int n, __nv_bfloat16* X, cudaStream_t st);
-cudaError_t bump(long long* p64, long long by64, int* p32, cudaStream_t st);
+cudaError_t bump(long long* p, long long by, cudaStream_t st);   // *p += by
 cudaError_t gen_desc(uint64_t seed, const long long* base, int n, const float* cal_amp, const float* cal_pulse, int ncal,
                      DevSac* sacs, float* hidden, float* target, int lcap, cudaStream_t st);
 cudaError_t featurize_noisy(uint64_t seed, const long long* base, const DevSac* sacs, const float* traces, int n,

@@ -547,7 +547,7 @@ extern "C" int opmm_surrogate_train(opmm_ctx* ctx, int32_t steps, int32_t batch,
     if (r.ok())
       r = cuda_status(featurize_noisy(data_seed, gbase + b, D.sacs.as<DevSac>(), f32(D.traces), batch, 0.05f, bf(D.X), s2),
                       "featurize");
-    if (r.ok()) r = cuda_status(bump(gbase + b, 2LL * batch, nullptr, s2), "advance sample base");
+    if (r.ok()) r = cuda_status(bump(gbase + b, 2LL * batch, s2), "advance sample base");
     return r;
   };
   auto net = [&](int b, cudaStream_t s1) -> Status {

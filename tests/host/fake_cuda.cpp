@@ -258,7 +258,7 @@ cudaError_t featurize_noisy(uint64_t, const long long*, const DevSac* sacs, cons
   touch(X, 2 * (size_t)n * kIn);
   return cudaSuccess;
 }
-cudaError_t bump(long long* p, long long, int*, cudaStream_t) { return touch(p, 8), cudaSuccess; }
+cudaError_t bump(long long* p, long long, cudaStream_t) { return touch(p, 8), cudaSuccess; }
 cudaError_t gen_desc(uint64_t, const long long*, int n, const float*, const float*, int, DevSac* sacs, float* hidden,
                      float* target, int, cudaStream_t) {
   touch(sacs, sizeof(DevSac) * (size_t)n);
