@@ -25,6 +25,8 @@
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+
+#include <algorithm>
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
@@ -845,34 +847,37 @@ __device__ __forceinline__ float u01(uint32_t x) { return (float)(x >> 8) * (1.0
 // normalised by the amplitude (start fixation = 0, end fixation = 1) and
 // velocity as 10 x the per-millisecond difference.  Output BF16 [n][512].
 // One warp per saccade, lane l the point pairs 2 l + 64 j, stored as they are
-// formed: the features are not staged, so a block runs beside a network block
-// that takes nearly all of an SM's shared memory (training data are made while
-// the network trains), and 4,096 saccades are 1,024 blocks at once instead of
-// 128 that take eight saccades per warp in turn.  Bound by the chain
-// descriptor -> samples -> store: 4,096 training saccades with their noise 6.2
-// us, where noise (8 us) and features (12 us, 33 KB of shared memory a block)
-// took two kernels; 96 training steps 11.6 -> 10.7 ms, since the network's
-// blocks no longer wait for an SM whose shared memory features hold.
+// formed: the features are not staged, so a block needs no shared memory, and
+// 4,096 saccades are 1,024 blocks at once instead of 128 that take eight
+// saccades per warp in turn.  Bound by the chain descriptor -> samples ->
+// store.
 constexpr int kFeatWarps = 4;
 static_assert(kFeatPoints % 64 == 0 && kIn == 2 * kFeatPoints, "whole pairs per lane");
-// the noisy trajectories (below) leave room beside a network block: 228 KB an
-// SM, of which every block takes 1 KB besides its own
-static_assert(sizeof(float) * kFeatWarps * kTrainLcap + gemm_smem(6, 128) + 2 * 1024 <= 228 * 1024 &&
-                  sizeof(float) * kFeatWarps * kTrainLcap + gemm_smem(4, 256) + 2 * 1024 <= 228 * 1024,
-              "a features block fits beside a network block");
 
 // NOISE: training data.  The warp first takes its trajectory to shared memory
-// (6.4 KB a block) with N(0, sigma^2) deg of noise added (Philox stream 3 of sample *base + b,
-// a Box-Muller pair per two samples), as far as the features reach; a noise
-// kernel of its own wrote and read every trajectory once more.
+// (6.4 KB a block) with N(0, sigma^2) deg of noise added (Philox stream 3 of
+// sample *base + b, a Box-Muller pair per two samples), as far as the features
+// reach; a noise kernel of its own wrote and read every trajectory once more.
+//
+// Training data are made while the network trains, whose blocks take nearly
+// all of an SM, so they are made by at most kFeatBlocksPerSm blocks per SM,
+// each warp taking saccades in turn: a network block finds room beside those
+// (10 k registers and 34 KB are left beside an error GEMM's).  With a block per
+// four saccades, up to sixteen of them filled each SM that a network block
+// left, and the next one waited for them: 96 steps of 4,096 10.91 ms against
+// 10.58 (10.57 with one per SM, but 8,192 saccades a step then take 8.76
+// instead of 8.64 ms).  Noise and features as two kernels in 33 KB blocks took
+// 12 + 8 us of their own and 11.6 ms in 96 steps.
+constexpr int kFeatBlocksPerSm = 2;
+static_assert(sizeof(float) * kFeatWarps * kTrainLcap * kFeatBlocksPerSm + gemm_smem(6, 128) + (kFeatBlocksPerSm + 1) * 1024 <=
+                      228 * 1024 &&
+                  gemm_smem(4, 256) <= gemm_smem(6, 128),
+              "features beside a network block: 228 KB an SM, every block 1 KB besides its own");
 template <bool NOISE>
-__global__ void __launch_bounds__(32 * kFeatWarps) k_featurize(const DevSac* sacs, const float* traces, int n,
-                                                               __nv_bfloat16* X, uint64_t seed,
-                                                               const long long* base_ptr, float sigma) {
-  __shared__ float noisy[NOISE ? kFeatWarps : 1][NOISE ? kTrainLcap : 1];
+__device__ __forceinline__ void features_of(int b, const DevSac* sacs, const float* traces, __nv_bfloat16* X, uint64_t seed,
+                                            const long long* base_ptr, float sigma,
+                                            float (&noisy)[NOISE ? kFeatWarps : 1][NOISE ? kTrainLcap : 1]) {
   const int lane = threadIdx.x & 31;
-  const int b = blockIdx.x * kFeatWarps + (threadIdx.x >> 5);
-  if (b >= n) return;
   const DevSac d = sacs[b];
   const float* y = traces + d.off;
   if constexpr (NOISE) {   // d.L <= kTrainLcap (k_gen_desc)
@@ -918,6 +923,22 @@ __global__ void __launch_bounds__(32 * kFeatWarps) k_featurize(const DevSac* sac
     const bool last = j + 1 == kPairs && lane == 31;                    // the last point's velocity is 0
     x[32 * j] = __floats2bfloat162_rn(p0[j], p1[j]);
     x[kFeatPoints / 2 + 32 * j] = __floats2bfloat162_rn(10.0f * (p1[j] - p0[j]), last ? 0.0f : 10.0f * (nxt - p1[j]));
+  }
+}
+
+template <bool NOISE>
+__global__ void __launch_bounds__(32 * kFeatWarps) k_featurize(const DevSac* sacs, const float* traces, int n,
+                                                               __nv_bfloat16* X, uint64_t seed,
+                                                               const long long* base_ptr, float sigma) {
+  __shared__ float noisy[NOISE ? kFeatWarps : 1][NOISE ? kTrainLcap : 1];
+  int b = blockIdx.x * kFeatWarps + (threadIdx.x >> 5);
+  if constexpr (NOISE) {
+    for (; b < n; b += gridDim.x * kFeatWarps) {
+      features_of<true>(b, sacs, traces, X, seed, base_ptr, sigma, noisy);
+      __syncwarp();   // the next trajectory takes this one's place
+    }
+  } else {
+    if (b < n) features_of<false>(b, sacs, traces, X, seed, base_ptr, sigma, noisy);
   }
 }
 
@@ -1171,8 +1192,9 @@ cudaError_t featurize(const DevSac* sacs, const float* traces, int n, __nv_bfloa
 }
 
 cudaError_t featurize_noisy(uint64_t seed, const long long* base, const DevSac* sacs, const float* traces, int n,
-                            float sigma, __nv_bfloat16* X, cudaStream_t st) {
-  k_featurize<true><<<(n + kFeatWarps - 1) / kFeatWarps, 32 * kFeatWarps, 0, st>>>(sacs, traces, n, X, seed, base, sigma);
+                            float sigma, __nv_bfloat16* X, int num_sms, cudaStream_t st) {
+  const int blocks = std::min((n + kFeatWarps - 1) / kFeatWarps, kFeatBlocksPerSm * num_sms);
+  k_featurize<true><<<blocks, 32 * kFeatWarps, 0, st>>>(sacs, traces, n, X, seed, base, sigma);
   return cudaGetLastError();
 }
 

@@ -159,7 +159,7 @@ cudaError_t bump(long long* p, long long by, cudaStream_t st);   // *p += by
 cudaError_t gen_desc(uint64_t seed, const long long* base, int n, const float* cal_amp, const float* cal_pulse, int ncal,
                      DevSac* sacs, float* hidden, float* target, int lcap, cudaStream_t st);
 cudaError_t featurize_noisy(uint64_t seed, const long long* base, const DevSac* sacs, const float* traces, int n,
-                            float sigma, __nv_bfloat16* X, cudaStream_t st);
+                            float sigma, __nv_bfloat16* X, int num_sms, cudaStream_t st);
 
 }  // namespace mlp
 }  // namespace opmm

@@ -545,7 +545,8 @@ extern "C" int opmm_surrogate_train(opmm_ctx* ctx, int32_t steps, int32_t batch,
       r = cuda_status(launch_simulate(f32(D.hidden), batch, D.sacs.as<DevSac>(), nullptr, S.outoff.as<long long>(),
                                       f32(D.traces), s2, kSimThreads), "simulate");
     if (r.ok())
-      r = cuda_status(featurize_noisy(data_seed, gbase + b, D.sacs.as<DevSac>(), f32(D.traces), batch, 0.05f, bf(D.X), s2),
+      r = cuda_status(featurize_noisy(data_seed, gbase + b, D.sacs.as<DevSac>(), f32(D.traces), batch, 0.05f, bf(D.X),
+                                      ctx->num_sms, s2),
                       "featurize");
     if (r.ok()) r = cuda_status(bump(gbase + b, 2LL * batch, s2), "advance sample base");
     return r;

@@ -252,7 +252,7 @@ cudaError_t featurize(const DevSac* sacs, const float* traces, int n, __nv_bfloa
   return cudaSuccess;
 }
 cudaError_t featurize_noisy(uint64_t, const long long*, const DevSac* sacs, const float* traces, int n, float,
-                            __nv_bfloat16* X, cudaStream_t) {
+                            __nv_bfloat16* X, int, cudaStream_t) {
   touch(sacs, sizeof(DevSac) * (size_t)n);
   touch(traces, 4 * (size_t)n * kTrainLcap);
   touch(X, 2 * (size_t)n * kIn);
