@@ -28,7 +28,9 @@ constexpr float kCalLo = 0.5f, kCalHi = 45.0f;
 // of 4,096 takes 16 SMs.  The kernel's registers leave no room for a GEMM
 // block beside it, and the network's GEMMs need 128 of the 152 SMs at once: in
 // blocks of 128 threads on 32 SMs it sent eight of their blocks into a second
-// wave for as long as it ran.
+// wave for as long as it ran.  40 steps with 256 against 128 threads: 512 to
+// 4,096 saccades a step the same within 1%, 1,024 4.00 against 4.05 ms, 8,192
+// 8.75 against 8.78, 16,384 16.3 against 16.4.
 constexpr int kSimThreads = 256;
 }  // namespace
 
