@@ -327,7 +327,8 @@ Status surrogate_prepare_plan(opmm_ctx* ctx, opmm_plan* p, int32_t n, bool once)
     }
     if (!own) own = std::make_shared<MlpBuffers>();
     keep = std::shared_ptr<MlpBuffers>(own.get(), [ctx, own](MlpBuffers* q) mutable {
-      if ((size_t)q->rows * kHidden * 6 > FitBuffers::kKeepBytes) return;
+      // kept up to the limit; buffers that could not grow (rows 0) hold what nothing accounts for
+      if (q->rows == 0 || (size_t)q->rows * kHidden * 6 > FitBuffers::kKeepBytes) return;
       std::lock_guard<std::mutex> lock(ctx->once_mu);
       own.swap(ctx->once_infer);   // what is there already is freed with `own`, outside the lock
     });

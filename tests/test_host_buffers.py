@@ -179,3 +179,14 @@ def test_kept_buffers_are_given_back_when_memory_runs_out(lib, ctx, call):
         lib.fake_capacity(1 << 40)
     assert _predict(lib, ctx, 300) == G.OPMM_OK           # and the next one-shot call allocates anew
     assert lib.fake_bad() == 0
+
+
+def test_what_a_failed_call_leaves_is_bounded(lib, ctx):
+    assert _predict(lib, ctx, 256) == G.OPMM_OK
+    own = lib.fake_in_use()
+    for nth in range(1, 3):                                # activations: X grows, then a layer's buffer fails
+        lib.fake_fail_alloc(nth)
+        assert _predict(lib, ctx, 1200000) == G.OPMM_ENOMEM
+        lib.fake_fail_alloc(-1)
+        assert lib.fake_in_use() <= own
+    assert _predict(lib, ctx, 256) == G.OPMM_OK
